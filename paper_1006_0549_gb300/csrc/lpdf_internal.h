@@ -244,26 +244,28 @@ constexpr int kIn = 8, kInP = 16, kH = 128, kOut = 7, kOutP = 16;
 // W3[128][128], b3[128], W4[16][128] (rows 7..15 zero), b4[16]
 constexpr int oW1 = 0, ob1 = oW1 + kH * kInP, oW2 = ob1 + kH, ob2 = oW2 + kH * kH, oW3 = ob2 + kH, ob3 = oW3 + kH * kH,
               oW4 = ob3 + kH, ob4 = oW4 + kOutP * kH, kParams = ob4 + kOutP;
-// BF16 packs: row-major [out][in] for the forward, [in][out] for the backward
-constexpr int pW1 = 0, pW2 = pW1 + kH * kInP, pW3 = pW2 + kH * kH, pW4 = pW3 + kH * kH, pT2 = pW4 + kOutP * kH,
-              pT3 = pT2 + kH * kH, pT4 = pT3 + kH * kH, kPack = pT4 + kH * kOutP;
-// per-CTA gradient partials: W^T layouts [in][out] and the biases
+// BF16 pack of W1..W4 as the kernels stage it: each [out][in] in the core-matrix layout of lpdf_tc.cuh
+constexpr int pW1 = 0, pW2 = pW1 + kH * kInP, pW3 = pW2 + kH * kH, pW4 = pW3 + kH * kH, kPack = pW4 + kOutP * kH;
+// per-tile gradient partials: W1 and the biases as they are, W2..W4 transposed ([in][out])
 constexpr int gW1 = 0, gW2 = gW1 + kInP * kH, gW3 = gW2 + kH * kH, gW4 = gW3 + kH * kH, gb1 = gW4 + kH * kOutP,
               gb2 = gb1 + kH, gb3 = gb2 + kH, gb4 = gb3 + kH, kPart = gb4 + kOutP;
+constexpr int kLossParts = 4;   // partial losses per tile
 // standardisation block: feature means and deviations, loss weights, target means and deviations
 constexpr int nFM = 0, nFS = nFM + kIn, nW = nFS + kIn, nTM = nW + kOut, nTS = nTM + kOut, kNorm = nTS + kOut;
 }  // namespace mlp
 cudaError_t mlp_configure();
 cudaError_t launch_mlp_forward(const float* feat, int64_t B, const float* P, const void* pack, const float* norm,
-                               float* out, float* out_user, void* act, unsigned* error, cudaStream_t st);
-// per-CTA partials into part ((B + 127) / 128 x kPart), then their sum in CTA order into grad
-cudaError_t launch_mlp_backward(const float* feat, const float* tgt, int64_t B, const void* pack, const float* norm,
-                                const float* out, const void* act, float* part, float* grad, unsigned* error,
-                                cudaStream_t st);
-cudaError_t launch_mlp_adam(float* P, const float* grad, float* m, float* v, float lr, int step, void* pack,
-                            cudaStream_t st);
-cudaError_t launch_mlp_loss(const float* out, const float* tgt, int64_t B, const float* norm, double* loss,
-                            cudaStream_t st);
+                               float* out, float* out_user, unsigned* error, cudaStream_t st);
+// forward and backward of a batch: gradient partials into part ((B + 127) / 128 x kPart) and losses
+// into lpart ((B + 127) / 128 x kLossParts)
+cudaError_t launch_mlp_gradient(const float* feat, const float* tgt, int64_t B, const float* P, const void* pack,
+                                const float* norm, float* part, double* lpart, unsigned* error, cudaStream_t st);
+// the partials of a batch of B rows summed in tile order: the loss into loss[0]; with grad != NULL the
+// gradient into it, else an Adam step (number `step`) and the new pack
+cudaError_t launch_mlp_reduce(const float* part, const double* lpart, int64_t B, float* grad, float* P, float* m,
+                              float* v, float lr, int step, void* pack, double* loss, cudaStream_t st);
+// the padding zeroed and the pack written
+cudaError_t launch_mlp_pack(float* P, void* pack, cudaStream_t st);
 // feature and target means and deviations of a data set into norm (weights untouched)
 cudaError_t launch_mlp_fit_norm(const float* feat, const float* tgt, int64_t B, float* norm, cudaStream_t st);
 

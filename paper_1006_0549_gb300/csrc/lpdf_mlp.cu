@@ -6,6 +6,8 @@
 // releases the warpgroup, and each thread reads its row of D from its TMEM lane.
 #include <cuda_runtime.h>
 
+#include <algorithm>
+
 #include "lpdf_device.cuh"
 #include "lpdf_internal.h"
 #include "lpdf_tc.cuh"
@@ -114,289 +116,283 @@ namespace {
 
 using namespace mlp;
 
-// element (r, k) of a row-major BF16 matrix (R x K) staged in the core layout, all threads
-__device__ __forceinline__ void stage(unsigned char* dst, const __nv_bfloat16* __restrict__ src, int R, int K)
+// 8 consecutive values of row r from column k (a multiple of 8): one 16-byte piece of the core layout
+__device__ __forceinline__ void put8(unsigned char* dst, int r, int k, int K, const float* v)
 {
-    for (int i = threadIdx.x; i < R * K; i += blockDim.x) {
-        const int r = i / K, k = i - (i / K) * K;
-        *reinterpret_cast<__nv_bfloat16*>(dst + tc::core_offset(r, k, K)) = src[i];
+    uint4 q;
+    uint32_t* w = reinterpret_cast<uint32_t*>(&q);
+#pragma unroll
+    for (int j = 0; j < 4; ++j) {
+        const __nv_bfloat162 b = __floats2bfloat162_rn(v[2 * j], v[2 * j + 1]);
+        w[j] = *reinterpret_cast<const uint32_t*>(&b);
+    }
+    *reinterpret_cast<uint4*>(dst + tc::core_offset(r, k, K)) = q;
+}
+__device__ __forceinline__ void get8(const unsigned char* src, int r, int k, int K, float* v)
+{
+    const uint4 q = *reinterpret_cast<const uint4*>(src + tc::core_offset(r, k, K));
+    const uint32_t w[4] = {q.x, q.y, q.z, q.w};
+#pragma unroll
+    for (int j = 0; j < 4; ++j) {
+        v[2 * j] = __uint_as_float(w[j] << 16);
+        v[2 * j + 1] = __uint_as_float(w[j] & 0xffff0000u);
     }
 }
 
-__device__ __forceinline__ void put(unsigned char* dst, int r, int k, int K, float v)
+constexpr int kNetThreads = 512;
+constexpr uint32_t kPackBytes = 2 * kPack, kXBytes = 2 * kH * kInP, kHBytes = 2 * kH * kH;
+
+// dynamic shared memory: the weight pack, then per group the inputs and the activations (one buffer
+// that every layer overwrites, or with kTrain the three layers'), then dZ4 with kTrain
+template <int kGroups, bool kTrain>
+constexpr uint32_t net_smem()
 {
-    *reinterpret_cast<__nv_bfloat16*>(dst + tc::core_offset(r, k, K)) = __float2bfloat16(v);
+    return kPackBytes + kGroups * (kXBytes + (kTrain ? 3 : 1) * kHBytes) + (kTrain ? kXBytes : 0);
 }
 
-// issue a GEMM from thread 0, wait (bounded) for it, order the TMEM reads after it
-__device__ __forceinline__ bool gemm_sync(uint32_t tmem, const void* A, const void* B, int N, int K,
-                                          unsigned long long* bar, uint32_t& phase, unsigned* error)
+// thread order of the columns after the halving reduction below: lane l holds column l
+// (the sums of 32 columns of a warp's rows; the same additions as 32 butterflies)
+__device__ __forceinline__ float column_sums32(float* v, int lane)
 {
-    tc::fence_async_smem();
-    tc::fence_before_sync();
-    __syncthreads();
-    tc::fence_after_sync();
-    if (threadIdx.x == 0) tc::gemm_issue(tmem, A, B, N, K, bar);
-    bool ok = tc::mbar_wait(bar, phase);
-    if (!ok) {
-        atomicOr(error, 1u);
-        ok = tc::mbar_wait(bar, phase);
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) {
+        const bool up = lane & o;
+#pragma unroll
+        for (int j = 0; j < o; ++j) {
+            const float keep = up ? v[j + o] : v[j], give = up ? v[j] : v[j + o];
+            v[j] = keep + __shfl_xor_sync(0xffffffffu, give, o);
+        }
     }
-    phase ^= 1u;
-    tc::fence_after_sync();
-    return ok;
+    return v[0];
 }
 
-__device__ __forceinline__ uint32_t lane_addr(uint32_t tmem, int col)
+// The network on 128-row tiles, one tile per group of 512 / kGroups threads at a time, the grid's groups
+// striding over the tiles. feat (B x 8, FP32) is standardised with norm's feature means and deviations;
+// out (may be NULL: B x 16, the 7 standardised outputs, then zeros), out_user (may be NULL: B x 7, in
+// target units). With kTrain (a tile per CTA) the backward pass follows in the same launch: the gradient
+// of the mean squared error over the 7 standardised outputs (weights norm[nW]) with respect to every
+// parameter as this tile's partial sums, and the tile's loss.
+//
+// What bounds it: the chain of GEMM, TMEM read, tanh, shared-memory store, barrier through the layers of
+// a tile, at a few tiles; the tanh instructions of the whole grid (2 x 10^7 per 50,000 rows) at many. So
+// the epilogue of a tile is spread over 512 threads (a warp takes 32 rows x 32 columns), or over 256 with
+// two tiles in flight per SM, one computing while the other waits (kGroups = 2, when there are more
+// tiles than SMs). The weights arrive as one bulk copy of the pack, already in the operand layout, once
+// per CTA. The backward needs no transposed copies: the transposed operands are the same buffers read
+// MN-major, dZ overwrites the activations it came from, and the weight gradient and the next error
+// signal are issued together into the two halves of TMEM.
+template <int kGroups, bool kTrain>
+__global__ void __launch_bounds__(kNetThreads, 1) mlp_kernel(const float* __restrict__ feat, const float* __restrict__ tgt,
+                                                             int64_t B, const float* __restrict__ P,
+                                                             const __nv_bfloat16* __restrict__ pack,
+                                                             const float* __restrict__ norm, float* __restrict__ out,
+                                                             float* __restrict__ out_user, float* __restrict__ part,
+                                                             double* __restrict__ lpart, unsigned* __restrict__ error)
 {
-    return tmem + ((uint32_t)(32 * ((threadIdx.x >> 5) & 3)) << 16) + (uint32_t)col;
-}
-
-struct FwdSmem {
-    alignas(1024) unsigned char x[kH * kInP * 2];
-    alignas(1024) unsigned char h[kH * kH * 2];
-    alignas(1024) unsigned char w1[kH * kInP * 2];
-    alignas(1024) unsigned char w2[kH * kH * 2];
-    alignas(1024) unsigned char w3[kH * kH * 2];
-    alignas(1024) unsigned char w4[kOutP * kH * 2];
-    float b[3 * kH + kOutP];
-    unsigned long long bar;
-    uint32_t tmem;
-};
-
-// Forward on rows [128 blockIdx, +128): feat (B x 8, FP32) standardised with the feature means and
-// deviations of norm; out (may be NULL: B x 16, FP32, the 7 standardised outputs, then zeros);
-// out_user (may be NULL: B x 7, the outputs in target units); with act != NULL also the three
-// hidden activations (B x 128 BF16 each, for the backward pass).
-__global__ void __launch_bounds__(kH, 1) mlp_fwd_kernel(const float* __restrict__ feat, int64_t B,
-                                                        const float* __restrict__ P, const __nv_bfloat16* __restrict__ pack,
-                                                        const float* __restrict__ norm, float* __restrict__ out,
-                                                        float* __restrict__ out_user, __nv_bfloat16* __restrict__ act,
-                                                        unsigned* __restrict__ error)
-{
-    extern __shared__ __align__(1024) unsigned char smem_raw[];
-    FwdSmem& sm = *reinterpret_cast<FwdSmem*>(smem_raw);
-    const int t = threadIdx.x, wid = t >> 5;
-    const int64_t row = (int64_t)blockIdx.x * kH + t;
-    stage(sm.w1, pack + pW1, kH, kInP);
-    stage(sm.w2, pack + pW2, kH, kH);
-    stage(sm.w3, pack + pW3, kH, kH);
-    stage(sm.w4, pack + pW4, kOutP, kH);
-    for (int i = t; i < 3 * kH; i += kH) sm.b[i] = P[(i < kH ? ob1 : (i < 2 * kH ? ob2 - kH : ob3 - 2 * kH)) + i];
-    if (t < kOutP) sm.b[3 * kH + t] = P[ob4 + t];
-    for (int k = 0; k < kInP; ++k) {
-        float v = 0.0f;
-        if (k < kIn && row < B) v = (feat[row * kIn + k] - norm[nFM + k]) / norm[nFS + k];
-        put(sm.x, t, k, kInP, v);
+    static_assert(!kTrain || kGroups == 1, "a tile per CTA");
+    constexpr int GT = kNetThreads / kGroups, kCols = kH / (GT / 128);   // columns per thread of an epilogue
+    constexpr uint32_t kTmem = kTrain ? 256 : (kGroups == 1 ? 128 : 256);
+    extern __shared__ __align__(1024) unsigned char dyn[];
+    __shared__ float sb[3 * kH + kOutP], snorm[kNorm], wpart[4][kH];
+    __shared__ unsigned long long wbar, gbar[kGroups];
+    __shared__ uint32_t tmem_slot;
+    const int g = threadIdx.x / GT, t = threadIdx.x - g * GT, warp = t >> 5, lane = t & 31;
+    const int quad = warp & 3, cb = warp >> 2, r = 32 * quad + lane;     // the thread's row and column block
+    unsigned char* const w1 = dyn;
+    unsigned char* const w2 = w1 + 2 * (pW2 - pW1);
+    unsigned char* const w3 = w2 + kHBytes;
+    unsigned char* const w4 = w3 + kHBytes;
+    unsigned char* const x = dyn + kPackBytes + g * (kXBytes + (kTrain ? 3 : 1) * kHBytes);
+    unsigned char* const h[3] = {x + kXBytes, x + kXBytes + (kTrain ? kHBytes : 0), x + kXBytes + (kTrain ? 2 * kHBytes : 0)};
+    auto sync = [&]() {
+        if (kGroups == 1) __syncthreads();
+        else asm volatile("bar.sync %0, %1;" ::"r"(g + 1), "n"(GT) : "memory");
+    };
+    if (threadIdx.x == 0) {
+        tc::mbar_init1(&wbar);
+        for (int q = 0; q < kGroups; ++q) tc::mbar_init1(&gbar[q]);
+        mbar_expect_tx(&wbar, kPackBytes);
+        bulk_load(dyn, pack, kPackBytes, &wbar);
     }
-    if (wid == 0) {
-        tc::tmem_alloc(&sm.tmem, kH);
+    if (threadIdx.x < 32) {
+        tc::tmem_alloc(&tmem_slot, kTmem);
         tc::tmem_relinquish();
     }
-    if (t == 0) tc::mbar_init1(&sm.bar);
+    for (int i = threadIdx.x; i < 3 * kH + kOutP; i += kNetThreads)
+        sb[i] = P[i < kH ? ob1 + i : (i < 2 * kH ? ob2 - kH + i : (i < 3 * kH ? ob3 - 2 * kH + i : ob4 - 3 * kH + i))];
+    for (int i = threadIdx.x; i < kNorm; i += kNetThreads) snorm[i] = norm[i];
     tc::fence_before_sync();
     __syncthreads();
     tc::fence_after_sync();
-    const uint32_t tmem = sm.tmem;
+    const uint32_t tmem = tmem_slot + (kGroups == 1 ? 0u : 128u * g);
+    const uint32_t lanes = (uint32_t)(32 * quad) << 16;
+    unsigned long long* const bar = &gbar[g];
     uint32_t phase = 0;
-    bool ok = true;
-    const unsigned char* a_op = sm.x;
-    int K = kInP;
-    const unsigned char* w_op[3] = {sm.w1, sm.w2, sm.w3};
-    for (int l = 0; l < 3 && ok; ++l) {
-        ok = gemm_sync(tmem, a_op, w_op[l], kH, K, &sm.bar, phase, error);
-        if (!ok) break;
-        for (int c0 = 0; c0 < kH; c0 += 16) {
-            float v[16];
-            tc::tmem_ld16(lane_addr(tmem, c0), v);
-            tc::wait_ld();
-#pragma unroll
-            for (int j = 0; j < 16; ++j) {
-                const float a = tanhf(v[j] + sm.b[l * kH + c0 + j]);
-                const __nv_bfloat16 ab = __float2bfloat16(a);
-                *reinterpret_cast<__nv_bfloat16*>(sm.h + tc::core_offset(t, c0 + j, kH)) = ab;
-                if (act && row < B) act[((size_t)l * B + row) * kH + c0 + j] = ab;
-            }
-        }
-        a_op = sm.h;
-        K = kH;
-    }
-    if (ok) ok = gemm_sync(tmem, sm.h, sm.w4, kOutP, kH, &sm.bar, phase, error);
-    if (ok) {
-        float v[16];
-        tc::tmem_ld16(lane_addr(tmem, 0), v);
-        tc::wait_ld();
-        if (row < B && out)
-#pragma unroll
-            for (int j = 0; j < kOutP; ++j) out[row * kOutP + j] = j < kOut ? v[j] + sm.b[3 * kH + j] : 0.0f;
-        if (row < B && out_user)
-#pragma unroll
-            for (int j = 0; j < kOut; ++j) out_user[row * kOut + j] = (v[j] + sm.b[3 * kH + j]) * norm[nTS + j] + norm[nTM + j];
-    }
-    tc::fence_before_sync();
-    __syncthreads();
-    if (wid == 0) tc::tmem_dealloc(tmem, kH);
-}
-
-struct BwdSmem {
-    alignas(1024) unsigned char sat[kH * kH * 2];   // A operand, transposed activations [in][batch]
-    alignas(1024) unsigned char sbt[kH * kH * 2];   // B operand, transposed dZ [out][batch]
-    alignas(1024) unsigned char sar[kH * kH * 2];   // A operand, dZ rows [batch][out]
-    alignas(1024) unsigned char t2[kH * kH * 2];    // W2^T [in][out]
-    alignas(1024) unsigned char t3[kH * kH * 2];
-    alignas(1024) unsigned char t4[kH * kOutP * 2];
-    float wpart[4][kH];                             // per-warp column sums (bias gradients)
-    unsigned long long bar;
-    uint32_t tmem;
-};
-
-// column sums of v[0..15] (this thread's row, columns c0..c0+15) over the CTA, added to acc[c0..]
-__device__ __forceinline__ void colsum16(float (*wpart)[kH], const float* v, int c0)
-{
-    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-#pragma unroll
-    for (int j = 0; j < 16; ++j) {
-        float s = v[j];
-#pragma unroll
-        for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
-        if (lane == 0) wpart[wid][c0 + j] = s;
-    }
-}
-
-// Backward on rows [128 blockIdx, +128) of a batch of B rows: the gradient of the mean squared
-// error over the 7 standardised outputs (weights w[7]) with respect to every parameter, as this
-// CTA's partial sums (W^T layouts).
-__global__ void __launch_bounds__(kH, 1) mlp_bwd_kernel(const float* __restrict__ feat, const float* __restrict__ tgt,
-                                                        int64_t B, const __nv_bfloat16* __restrict__ pack,
-                                                        const float* __restrict__ norm, const float* __restrict__ out,
-                                                        const __nv_bfloat16* __restrict__ act,
-                                                        float* __restrict__ part, unsigned* __restrict__ error)
-{
-    extern __shared__ __align__(1024) unsigned char smem_raw[];
-    BwdSmem& sm = *reinterpret_cast<BwdSmem*>(smem_raw);
-    const int t = threadIdx.x, wid = t >> 5;
-    const int64_t row = (int64_t)blockIdx.x * kH + t;
-    const bool live = row < B;
-    float* const pp = part + (size_t)blockIdx.x * kPart;
-    stage(sm.t2, pack + pT2, kH, kH);
-    stage(sm.t3, pack + pT3, kH, kH);
-    stage(sm.t4, pack + pT4, kH, kOutP);
-    // dZ4 = d loss / d out: 2 (out - target) w_j / (7 B)
-    float dz4[kOutP];
-#pragma unroll
-    for (int j = 0; j < kOutP; ++j) {
-        float d = 0.0f;
-        if (live && j < kOut) {
-            const float y = (tgt[row * kOut + j] - norm[nTM + j]) / norm[nTS + j];
-            d = 2.0f * (out[row * kOutP + j] - y) * norm[nW + j] / (float)(kOut * B);
-        }
-        dz4[j] = d;
-    }
-    colsum16(sm.wpart, dz4, 0);
-    // dW4^T = A3^T dZ4: A = A3^T [in][batch], B = dZ4^T [out][batch]
-    const __nv_bfloat16* a3 = act + (2 * (size_t)B + (live ? row : 0)) * kH;
-    for (int i = 0; i < kH; ++i)
-        *reinterpret_cast<__nv_bfloat16*>(sm.sat + tc::core_offset(i, t, kH)) = live ? a3[i] : __float2bfloat16(0.0f);
-#pragma unroll
-    for (int j = 0; j < kOutP; ++j) {
-        put(sm.sbt, j, t, kH, dz4[j]);
-        put(sm.sar, t, j, kOutP, dz4[j]);
-    }
-    if (wid == 0) {
-        tc::tmem_alloc(&sm.tmem, kH);
-        tc::tmem_relinquish();
-    }
-    if (t == 0) tc::mbar_init1(&sm.bar);
-    tc::fence_before_sync();
-    __syncthreads();
-    tc::fence_after_sync();
-    if (t < kOutP) pp[gb4 + t] = sm.wpart[0][t] + sm.wpart[1][t] + sm.wpart[2][t] + sm.wpart[3][t];
-    const uint32_t tmem = sm.tmem;
-    uint32_t phase = 0;
-    bool ok = gemm_sync(tmem, sm.sat, sm.sbt, kOutP, kH, &sm.bar, phase, error);
-    if (ok) {
-        float v[16];
-        tc::tmem_ld16(lane_addr(tmem, 0), v);
-        tc::wait_ld();
-#pragma unroll
-        for (int j = 0; j < kOutP; ++j) pp[gW4 + t * kOutP + j] = v[j];
-    }
-    // hidden layers 3, 2, 1: dH = dZ W (A = dZ rows, B = W^T), dZ = dH (1 - a^2),
-    // dW^T = A_prev^T dZ, bias gradient = column sums of dZ
-    const unsigned char* tw[3] = {sm.t4, sm.t3, sm.t2};
-    const int kw[3] = {kOutP, kH, kH};
-    const int gw[3] = {gW3, gW2, gW1};
-    const int gb[3] = {gb3, gb2, gb1};
-    for (int s = 0; s < 3 && ok; ++s) {
-        const int l = 2 - s;                       // hidden layer index (0-based) whose dZ is formed
+    bool first = true;
+    // after everyone's shared-memory stores: thread 0 of the group issues the GEMMs; all wait for them
+    auto gemms = [&](auto issue) {
+        tc::fence_async_smem();
         tc::fence_before_sync();
-        ok = gemm_sync(tmem, sm.sar, tw[s], kH, kw[s], &sm.bar, phase, error);
-        if (!ok) break;
-        const __nv_bfloat16* al = act + ((size_t)l * B + (live ? row : 0)) * kH;
-        for (int c0 = 0; c0 < kH; c0 += 16) {
+        sync();
+        tc::fence_after_sync();
+        if (t == 0) {
+            if (first && !tc::mbar_wait(&wbar, 0)) atomicOr(error, 1u);
+            issue();
+            tc::mma_commit(bar);
+        }
+        first = false;
+        if (!tc::mbar_wait(bar, phase)) {
+            atomicOr(error, 1u);
+            tc::mbar_wait(bar, phase);
+        }
+        phase ^= 1u;
+        tc::fence_after_sync();
+    };
+    const int64_t ntiles = (B + kH - 1) / kH;
+    for (int64_t tile = (int64_t)blockIdx.x * kGroups + g; tile < ntiles; tile += (int64_t)gridDim.x * kGroups) {
+        const int64_t row0 = tile * kH, row = row0 + r;
+        const bool live = row < B;
+        // the inputs: a thread standardises 2 (4) columns of a row; columns 8..15 are zero
+        {
+            constexpr int kPer = kIn * kH / GT;
+            const int rr = t / (kIn / kPer), k0 = kPer * (t % (kIn / kPer));
+            float v[kPer];
+#pragma unroll
+            for (int k = 0; k < kPer; ++k)
+                v[k] = row0 + rr < B ? (feat[(row0 + rr) * kIn + k0 + k] - snorm[nFM + k0 + k]) / snorm[nFS + k0 + k] : 0.0f;
+#pragma unroll
+            for (int k = 0; k < kPer; k += 2)
+                *reinterpret_cast<__nv_bfloat162*>(x + tc::core_offset(rr, k0 + k, kInP)) = __floats2bfloat162_rn(v[k], v[k + 1]);
+            if (t < kH) *reinterpret_cast<uint4*>(x + tc::core_offset(t, kIn, kInP)) = make_uint4(0u, 0u, 0u, 0u);
+        }
+#pragma unroll
+        for (int l = 0; l < 3; ++l) {
+            gemms([&]() {
+                if (l == 0) tc::gemm_issue_op(tmem, tc::k_major(x, kInP), tc::k_major(w1, kInP), kH, 1, false, false);
+                else tc::gemm_issue_op(tmem, tc::k_major(h[l - 1], kH), tc::k_major(l == 1 ? w2 : w3, kH), kH, 8, false, false);
+            });
+#pragma unroll 1
+            for (int c0 = cb * kCols; c0 < (cb + 1) * kCols; c0 += 32) {
+                float v[32];
+                tc::tmem_ld32(tmem + lanes + c0, v);
+                tc::wait_ld();
+#pragma unroll
+                for (int j = 0; j < 32; ++j) v[j] = tanhf(v[j] + sb[l * kH + c0 + j]);
+#pragma unroll
+                for (int j = 0; j < 32; j += 8) put8(h[l], r, c0 + j, kH, v + j);
+            }
+        }
+        gemms([&]() { tc::gemm_issue_op(tmem, tc::k_major(h[2], kH), tc::k_major(w4, kH), kOutP, 8, false, false); });
+        unsigned char* const z4 = x + kXBytes + 3 * kHBytes;   // kTrain
+        if (cb == 0 || (kTrain && cb == 1)) {
             float v[16];
-            tc::tmem_ld16(lane_addr(tmem, c0), v);
+            tc::tmem_ld16(tmem + lanes, v);
             tc::wait_ld();
 #pragma unroll
-            for (int j = 0; j < 16; ++j) {
-                const float a = live ? __bfloat162float(al[c0 + j]) : 0.0f;
-                v[j] = live ? v[j] * (1.0f - a * a) : 0.0f;
-                put(sm.sbt, c0 + j, t, kH, v[j]);
-                put(sm.sar, t, c0 + j, kH, v[j]);
-            }
-            colsum16(sm.wpart, v, c0);
-        }
-        // A operand: the previous activations transposed (the standardised inputs for layer 1)
-        if (l > 0) {
-            const __nv_bfloat16* ap = act + ((size_t)(l - 1) * B + (live ? row : 0)) * kH;
-            for (int i = 0; i < kH; ++i)
-                *reinterpret_cast<__nv_bfloat16*>(sm.sat + tc::core_offset(i, t, kH)) =
-                    live ? ap[i] : __float2bfloat16(0.0f);
-        } else {
-            for (int i = 0; i < kH; ++i) {
-                float x = 0.0f;
-                if (i < kIn && live) x = (feat[row * kIn + i] - norm[nFM + i]) / norm[nFS + i];
-                put(sm.sat, i, t, kH, x);
-            }
-        }
-        tc::fence_before_sync();
-        __syncthreads();
-        pp[gb[s] + t] = sm.wpart[0][t] + sm.wpart[1][t] + sm.wpart[2][t] + sm.wpart[3][t];
-        ok = gemm_sync(tmem, sm.sat, sm.sbt, kH, kH, &sm.bar, phase, error);
-        if (!ok) break;
-        // the loads are warp-collective: every thread loads, the rows that exist are stored
-        const bool keep = t < (l > 0 ? kH : kInP);
-        for (int c0 = 0; c0 < kH; c0 += 16) {
-            float v[16];
-            tc::tmem_ld16(lane_addr(tmem, c0), v);
-            tc::wait_ld();
-            if (keep)
+            for (int j = 0; j < kOutP; ++j) v[j] = j < kOut ? v[j] + sb[3 * kH + j] : 0.0f;
+            if (!kTrain) {
+                if (live && out)
 #pragma unroll
-                for (int j = 0; j < 16; ++j) pp[gw[s] + t * kH + c0 + j] = v[j];
+                    for (int j = 0; j < kOutP; j += 4)
+                        *reinterpret_cast<float4*>(out + row * kOutP + j) = make_float4(v[j], v[j + 1], v[j + 2], v[j + 3]);
+                if (live && out_user)
+#pragma unroll
+                    for (int j = 0; j < kOut; ++j) out_user[row * kOut + j] = v[j] * snorm[nTS + j] + snorm[nTM + j];
+            } else if (cb == 0) {
+                // dZ4 = d loss / d out: 2 (out - target) w_j / (7 B)
+                float s[32];
+#pragma unroll
+                for (int j = 0; j < 32; ++j) s[j] = 0.0f;
+#pragma unroll
+                for (int j = 0; j < kOut; ++j)
+                    if (live) {
+                        const float y = (tgt[row * kOut + j] - snorm[nTM + j]) / snorm[nTS + j];
+                        s[j] = 2.0f * (v[j] - y) * snorm[nW + j] / (float)(kOut * B);
+                    }
+                put8(z4, r, 0, kOutP, s);
+                put8(z4, r, 8, kOutP, s + 8);
+                const float cs = column_sums32(s, lane);
+                if (lane < kOutP) wpart[quad][lane] = cs;
+            } else {
+                // the loss of the warp's rows in FP64
+                double s = 0.0;
+#pragma unroll
+                for (int j = 0; j < kOut; ++j)
+                    if (live) {
+                        const double y = ((double)tgt[row * kOut + j] - snorm[nTM + j]) / snorm[nTS + j];
+                        const double d = (double)v[j] - y;
+                        s += snorm[nW + j] * d * d;
+                    }
+#pragma unroll
+                for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+                if (lane == 0) lpart[tile * kLossParts + quad] = s;
+            }
+        }
+        if constexpr (kTrain) {
+            float* const pp = part + (size_t)tile * kPart;
+            // a layer: dW^T of the layer above (its input as the rows, its dZ as the columns) into the
+            // upper half of TMEM and dH = dZ W into the lower; then dZ = dH (1 - h^2) over h, the bias
+            // gradient (column sums of dZ) and dW^T to the partials
+#pragma unroll
+            for (int l = 2; l >= 0; --l) {
+                gemms([&]() {
+                    if (l == 2) {
+                        tc::gemm_issue_op(tmem, tc::k_major(z4, kOutP), tc::mn_major(w4, kH), kH, 1, false, true);
+                        tc::gemm_issue_op(tmem + 128, tc::mn_major(h[2], kH), tc::mn_major(z4, kOutP), kOutP, 8, true, true);
+                    } else {
+                        tc::gemm_issue_op(tmem, tc::k_major(h[l + 1], kH), tc::mn_major(l == 1 ? w3 : w2, kH), kH, 8, false, true);
+                        tc::gemm_issue_op(tmem + 128, tc::mn_major(h[l], kH), tc::mn_major(h[l + 1], kH), kH, 8, true, true);
+                    }
+                });
+                if (t < (l == 2 ? kOutP : kH))
+                    pp[(l == 2 ? gb4 : (l == 1 ? gb3 : gb2)) + t] = wpart[0][t] + wpart[1][t] + wpart[2][t] + wpart[3][t];
+                const int c0 = 32 * cb;
+                float v[32];
+                tc::tmem_ld32(tmem + lanes + c0, v);
+                tc::wait_ld();
+                sync();   // wpart is read
+#pragma unroll
+                for (int j = 0; j < 32; j += 8) {
+                    float a[8];
+                    get8(h[l], r, c0 + j, kH, a);
+#pragma unroll
+                    for (int q = 0; q < 8; ++q) v[j + q] = live ? v[j + q] * (1.0f - a[q] * a[q]) : 0.0f;
+                    put8(h[l], r, c0 + j, kH, v + j);
+                }
+                wpart[quad][c0 + lane] = column_sums32(v, lane);
+                if (l == 2) {
+                    if (cb == 0) {
+                        tc::tmem_ld16(tmem + 128 + lanes, v);
+                        tc::wait_ld();
+#pragma unroll
+                        for (int j = 0; j < kOutP; j += 4)
+                            *reinterpret_cast<float4*>(pp + gW4 + r * kOutP + j) = make_float4(v[j], v[j + 1], v[j + 2], v[j + 3]);
+                    }
+                } else {
+                    tc::tmem_ld32(tmem + 128 + lanes + c0, v);
+                    tc::wait_ld();
+#pragma unroll
+                    for (int j = 0; j < 32; j += 4)
+                        *reinterpret_cast<float4*>(pp + (l == 1 ? gW3 : gW2) + r * kH + c0 + j) =
+                            make_float4(v[j], v[j + 1], v[j + 2], v[j + 3]);
+                }
+            }
+            // dW1 = dZ1^T X: a row per output
+            gemms([&]() { tc::gemm_issue_op(tmem, tc::mn_major(h[0], kH), tc::mn_major(x, kInP), kInP, 8, true, true); });
+            if (t < kH) pp[gb1 + t] = wpart[0][t] + wpart[1][t] + wpart[2][t] + wpart[3][t];
+            if (cb == 1) {
+                float v[16];
+                tc::tmem_ld16(tmem + lanes, v);
+                tc::wait_ld();
+#pragma unroll
+                for (int j = 0; j < kInP; j += 4)
+                    *reinterpret_cast<float4*>(pp + gW1 + r * kInP + j) = make_float4(v[j], v[j + 1], v[j + 2], v[j + 3]);
+            }
         }
     }
     tc::fence_before_sync();
     __syncthreads();
-    if (wid == 0) tc::tmem_dealloc(tmem, kH);
-}
-
-// grad (padded parameter layout) = the sum of the CTA partials in CTA order
-__global__ void mlp_reduce_kernel(const float* __restrict__ part, int nparts, float* __restrict__ grad)
-{
-    const int i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= kParams) return;
-    int src;   // the partial that holds parameter i
-    if (i < ob1) { const int o = i / kInP, k = i % kInP; src = gW1 + k * kH + o; }
-    else if (i < oW2) src = gb1 + (i - ob1);
-    else if (i < ob2) { const int j = i - oW2, o = j / kH, k = j % kH; src = gW2 + k * kH + o; }
-    else if (i < oW3) src = gb2 + (i - ob2);
-    else if (i < ob3) { const int j = i - oW3, o = j / kH, k = j % kH; src = gW3 + k * kH + o; }
-    else if (i < oW4) src = gb3 + (i - ob3);
-    else if (i < ob4) { const int j = i - oW4, o = j / kH, k = j % kH; src = gW4 + k * kOutP + o; }
-    else src = gb4 + (i - ob4);
-    double s = 0.0;
-    for (int c = 0; c < nparts; ++c) s += part[(size_t)c * kPart + src];
-    grad[i] = (float)s;
+    if (threadIdx.x < 32) tc::tmem_dealloc(tmem_slot, kTmem);
 }
 
 // parameters that exist (the padding stays zero)
@@ -408,65 +404,72 @@ __device__ __forceinline__ bool is_param(int i)
     return true;
 }
 
-// Adam step (t = step number from 1), then the BF16 packs
-__global__ void mlp_adam_kernel(float* __restrict__ P, const float* __restrict__ g, float* __restrict__ m,
-                                float* __restrict__ v, float lr, float b1, float b2, float eps, int step,
-                                __nv_bfloat16* __restrict__ pack)
+// parameter i in the BF16 pack (biases are not packed)
+__device__ __forceinline__ void pack_param(__nv_bfloat16* __restrict__ pack, int i, float p)
+{
+    int at = -1;
+    if (i < ob1) at = pW1 + (int)tc::core_offset(i / kInP, i % kInP, kInP) / 2;
+    else if (i >= oW2 && i < ob2) at = pW2 + (int)tc::core_offset((i - oW2) / kH, (i - oW2) % kH, kH) / 2;
+    else if (i >= oW3 && i < ob3) at = pW3 + (int)tc::core_offset((i - oW3) / kH, (i - oW3) % kH, kH) / 2;
+    else if (i >= oW4 && i < ob4) at = pW4 + (int)tc::core_offset((i - oW4) / kH, (i - oW4) % kH, kH) / 2;
+    if (at >= 0) pack[at] = __float2bfloat16(p);
+}
+
+__global__ void mlp_pack_kernel(float* __restrict__ P, __nv_bfloat16* __restrict__ pack)
 {
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= kParams) return;
-    float p = P[i];
-    if (step > 0 && is_param(i)) {
-        const float gi = g[i];
-        const float mi = b1 * m[i] + (1.0f - b1) * gi;
-        const float vi = b2 * v[i] + (1.0f - b2) * gi * gi;
-        m[i] = mi;
-        v[i] = vi;
-        const float mh = mi / (1.0f - powf(b1, (float)step)), vh = vi / (1.0f - powf(b2, (float)step));
-        p -= lr * mh / (sqrtf(vh) + eps);
-        P[i] = p;
-    }
-    if (!is_param(i)) {
-        P[i] = 0.0f;
-        p = 0.0f;
-    }
-    const __nv_bfloat16 pb = __float2bfloat16(p);
-    if (i < ob1) {
-        pack[pW1 + i] = pb;
-    } else if (i >= oW2 && i < ob2) {
-        const int j = i - oW2, o = j / kH, k = j % kH;
-        pack[pW2 + j] = pb;
-        pack[pT2 + k * kH + o] = pb;
-    } else if (i >= oW3 && i < ob3) {
-        const int j = i - oW3, o = j / kH, k = j % kH;
-        pack[pW3 + j] = pb;
-        pack[pT3 + k * kH + o] = pb;
-    } else if (i >= oW4 && i < ob4) {
-        const int j = i - oW4, o = j / kH, k = j % kH;
-        pack[pW4 + j] = pb;
-        pack[pT4 + k * kOutP + o] = pb;
-    }
+    if (!is_param(i)) P[i] = 0.0f;
+    pack_param(pack, i, P[i]);
 }
 
-// loss[0] = the weighted mean squared error over the 7 standardised outputs (one block)
-__global__ void mlp_loss_kernel(const float* __restrict__ out, const float* __restrict__ tgt, int64_t B,
-                                const float* __restrict__ norm, double* __restrict__ loss)
+// The tiles' partials summed in tile order in FP64, per parameter; with grad they go there, else Adam
+// step `step` (from 1) follows with the new pack. The last block sums the losses.
+__global__ void mlp_reduce_kernel(const float* __restrict__ part, const double* __restrict__ lpart, int nparts, int64_t B,
+                                  float* __restrict__ grad, float* __restrict__ P, float* __restrict__ m,
+                                  float* __restrict__ v, float lr, float b1, float b2, float eps, int step,
+                                  __nv_bfloat16* __restrict__ pack, double* __restrict__ loss)
 {
-    __shared__ double sh[256];
-    double s = 0.0;
-    for (int64_t r = threadIdx.x; r < B; r += blockDim.x)
-        for (int j = 0; j < kOut; ++j) {
-            const double y = ((double)tgt[r * kOut + j] - norm[nTM + j]) / norm[nTS + j];
-            const double d = (double)out[r * kOutP + j] - y;
-            s += norm[nW + j] * d * d;
-        }
-    sh[threadIdx.x] = s;
-    __syncthreads();
-    for (int o = 128; o > 0; o >>= 1) {
-        if (threadIdx.x < o) sh[threadIdx.x] += sh[threadIdx.x + o];
-        __syncthreads();
+    __shared__ float corr[2];
+    if (blockIdx.x == gridDim.x - 1) {
+        if (threadIdx.x >= 32) return;
+        double s = 0.0;
+        for (int q = threadIdx.x; q < nparts * kLossParts; q += 32) s += lpart[q];
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+        if (threadIdx.x == 0) loss[0] = s / (double)(kOut * B);
+        return;
     }
-    if (threadIdx.x == 0) loss[0] = sh[0] / (double)(kOut * B);
+    if (threadIdx.x < 2) corr[threadIdx.x] = 1.0f - powf(threadIdx.x ? b2 : b1, (float)step);
+    __syncthreads();
+    const int i = blockIdx.x * blockDim.x + threadIdx.x;
+    if (i >= kParams) return;
+    int src;   // the partial that holds parameter i
+    if (i < ob1) src = gW1 + i;
+    else if (i < oW2) src = gb1 + (i - ob1);
+    else if (i < ob2) { const int j = i - oW2, o = j / kH, k = j % kH; src = gW2 + k * kH + o; }
+    else if (i < oW3) src = gb2 + (i - ob2);
+    else if (i < ob3) { const int j = i - oW3, o = j / kH, k = j % kH; src = gW3 + k * kH + o; }
+    else if (i < oW4) src = gb3 + (i - ob3);
+    else if (i < ob4) { const int j = i - oW4, o = j / kH, k = j % kH; src = gW4 + k * kOutP + o; }
+    else src = gb4 + (i - ob4);
+    double s = 0.0;
+#pragma unroll 8
+    for (int c = 0; c < nparts; ++c) s += part[(size_t)c * kPart + src];
+    const float gi = (float)s;
+    if (grad) {
+        grad[i] = gi;
+        return;
+    }
+    if (!is_param(i)) return;
+    const float mi = b1 * m[i] + (1.0f - b1) * gi;
+    const float vi = b2 * v[i] + (1.0f - b2) * gi * gi;
+    m[i] = mi;
+    v[i] = vi;
+    const float mh = mi / corr[0], vh = vi / corr[1];
+    const float p = P[i] - lr * mh / (sqrtf(vh) + eps);
+    P[i] = p;
+    pack_param(pack, i, p);
 }
 
 // column c of the data set (features 0..7, then targets 8..14): mean and deviation (one block each;
@@ -513,46 +516,53 @@ __global__ void mlp_fit_norm_kernel(const float* __restrict__ feat, const float*
 
 cudaError_t mlp_configure()
 {
-    cudaError_t e = cudaFuncSetAttribute(mlp_fwd_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(FwdSmem));
+    cudaError_t e = cudaFuncSetAttribute(mlp_kernel<1, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)net_smem<1, false>());
     if (e == cudaSuccess)
-        e = cudaFuncSetAttribute(mlp_bwd_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(BwdSmem));
+        e = cudaFuncSetAttribute(mlp_kernel<2, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)net_smem<2, false>());
+    if (e == cudaSuccess)
+        e = cudaFuncSetAttribute(mlp_kernel<1, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)net_smem<1, true>());
     return e;
 }
 
 cudaError_t launch_mlp_forward(const float* feat, int64_t B, const float* P, const void* pack, const float* norm,
-                               float* out, float* out_user, void* act, unsigned* error, cudaStream_t st)
+                               float* out, float* out_user, unsigned* error, cudaStream_t st)
 {
     if (B <= 0) return cudaSuccess;
-    mlp_fwd_kernel<<<(unsigned)((B + kH - 1) / kH), kH, sizeof(FwdSmem), st>>>(
-        feat, B, P, static_cast<const __nv_bfloat16*>(pack), norm, out, out_user, static_cast<__nv_bfloat16*>(act),
-        error);
+    const int64_t tiles = (B + kH - 1) / kH;
+    const __nv_bfloat16* pk = static_cast<const __nv_bfloat16*>(pack);
+    const int sms = sm_count();
+    // a tile per SM is soonest done by all its threads; more tiles than SMs go two at a time
+    if (tiles <= sms)
+        mlp_kernel<1, false><<<(unsigned)tiles, kNetThreads, net_smem<1, false>(), st>>>(feat, nullptr, B, P, pk, norm, out,
+                                                                                         out_user, nullptr, nullptr, error);
+    else
+        mlp_kernel<2, false><<<(unsigned)std::min<int64_t>((tiles + 1) / 2, sms), kNetThreads, net_smem<2, false>(), st>>>(
+            feat, nullptr, B, P, pk, norm, out, out_user, nullptr, nullptr, error);
     return cudaGetLastError();
 }
 
-cudaError_t launch_mlp_backward(const float* feat, const float* tgt, int64_t B, const void* pack, const float* norm,
-                                const float* out, const void* act, float* part, float* grad, unsigned* error,
-                                cudaStream_t st)
+cudaError_t launch_mlp_gradient(const float* feat, const float* tgt, int64_t B, const float* P, const void* pack,
+                                const float* norm, float* part, double* lpart, unsigned* error, cudaStream_t st)
 {
     if (B <= 0) return cudaSuccess;
-    const unsigned nb = (unsigned)((B + kH - 1) / kH);
-    mlp_bwd_kernel<<<nb, kH, sizeof(BwdSmem), st>>>(feat, tgt, B, static_cast<const __nv_bfloat16*>(pack), norm, out,
-                                                    static_cast<const __nv_bfloat16*>(act), part, error);
-    mlp_reduce_kernel<<<(kParams + 255) / 256, 256, 0, st>>>(part, (int)nb, grad);
+    const int64_t tiles = (B + kH - 1) / kH;
+    mlp_kernel<1, true><<<(unsigned)std::min<int64_t>(tiles, sm_count()), kNetThreads, net_smem<1, true>(), st>>>(
+        feat, tgt, B, P, static_cast<const __nv_bfloat16*>(pack), norm, nullptr, nullptr, part, lpart, error);
     return cudaGetLastError();
 }
 
-cudaError_t launch_mlp_adam(float* P, const float* grad, float* m, float* v, float lr, int step, void* pack,
-                            cudaStream_t st)
+cudaError_t launch_mlp_reduce(const float* part, const double* lpart, int64_t B, float* grad, float* P, float* m,
+                              float* v, float lr, int step, void* pack, double* loss, cudaStream_t st)
 {
-    mlp_adam_kernel<<<(kParams + 255) / 256, 256, 0, st>>>(P, grad, m, v, lr, 0.9f, 0.999f, 1e-8f, step,
-                                                           static_cast<__nv_bfloat16*>(pack));
+    mlp_reduce_kernel<<<(kParams + 127) / 128 + 1, 128, 0, st>>>(part, lpart, (int)((B + kH - 1) / kH), B, grad, P, m, v,
+                                                                 lr, 0.9f, 0.999f, 1e-8f, step,
+                                                                 static_cast<__nv_bfloat16*>(pack), loss);
     return cudaGetLastError();
 }
 
-cudaError_t launch_mlp_loss(const float* out, const float* tgt, int64_t B, const float* norm, double* loss,
-                            cudaStream_t st)
+cudaError_t launch_mlp_pack(float* P, void* pack, cudaStream_t st)
 {
-    mlp_loss_kernel<<<1, 256, 0, st>>>(out, tgt, B, norm, loss);
+    mlp_pack_kernel<<<(kParams + 255) / 256, 256, 0, st>>>(P, static_cast<__nv_bfloat16*>(pack));
     return cudaGetLastError();
 }
 

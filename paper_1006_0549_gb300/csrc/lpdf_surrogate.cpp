@@ -19,8 +19,7 @@ struct lpdf_mlp {
     float* v = nullptr;
     float* grad = nullptr;      // mlp::kParams
     float* part = nullptr;      // per-tile partial gradients
-    void* act = nullptr;        // 3 x max_batch x 128 BF16
-    float* out = nullptr;       // max_batch x 16
+    double* lpart = nullptr;    // per-tile partial losses
     double* losses = nullptr;   // per training step
     int losses_cap = 0;
     unsigned* error = nullptr;
@@ -125,8 +124,7 @@ int lpdf_mlp_create(int64_t max_batch, lpdf_mlp** out)
         (e = cudaMalloc((void**)&m->v, sizeof(float) * kParams)) ||
         (e = cudaMalloc((void**)&m->grad, sizeof(float) * kParams)) ||
         (e = cudaMalloc((void**)&m->part, sizeof(float) * kPart * (size_t)tiles)) ||
-        (e = cudaMalloc(&m->act, 2 * 3 * (size_t)kH * (size_t)(tiles * kH))) ||
-        (e = cudaMalloc((void**)&m->out, sizeof(float) * kOutP * (size_t)(tiles * kH))) ||
+        (e = cudaMalloc((void**)&m->lpart, sizeof(double) * kLossParts * (size_t)tiles)) ||
         (e = cudaMalloc((void**)&m->s_cmp, sizeof(double) * 2)) ||
         (e = cudaMalloc((void**)&m->error, sizeof(unsigned))) || (e = cudaMemset(m->error, 0, sizeof(unsigned)))) {
         lpdf_mlp_free(m);
@@ -146,7 +144,7 @@ int lpdf_mlp_create(int64_t max_batch, lpdf_mlp** out)
 void lpdf_mlp_free(lpdf_mlp* m)
 {
     if (!m) return;
-    void* ps[] = {m->P, m->pack, m->norm, m->m, m->v, m->grad, m->part, m->act, m->out, m->losses, m->error,
+    void* ps[] = {m->P, m->pack, m->norm, m->m, m->v, m->grad, m->part, m->lpart, m->losses, m->error,
                   m->s_feat, m->s_out, m->s_fields, m->s_cmp};
     for (void* p : ps) cudaFree(p);
     delete m;
@@ -162,7 +160,7 @@ int lpdf_mlp_set_params(lpdf_mlp* m, const float* params, const float* norm)
     TRY(cudaMemset(m->m, 0, sizeof(float) * kParams));
     TRY(cudaMemset(m->v, 0, sizeof(float) * kParams));
     m->step = 0;
-    TRY(launch_mlp_adam(m->P, m->grad, m->m, m->v, 0.0f, 0, m->pack, nullptr));   // step 0: packs only
+    TRY(launch_mlp_pack(m->P, m->pack, nullptr));
     TRY(cudaDeviceSynchronize());
     return LPDF_OK;
 }
@@ -190,7 +188,7 @@ int lpdf_mlp_fit_norm(lpdf_mlp* m, const float* feat, const float* tgt, int64_t 
 int lpdf_mlp_forward(lpdf_mlp* m, const float* feat, int64_t B, float* out, void* stream)
 {
     if (!m || B < 0 || (B > 0 && (!feat || !out))) return lpdf_set_error(LPDF_ERR_ARG, "mlp_forward: bad argument");
-    TRY(launch_mlp_forward(feat, B, m->P, m->pack, m->norm, nullptr, out, nullptr, m->error, (cudaStream_t)stream));
+    TRY(launch_mlp_forward(feat, B, m->P, m->pack, m->norm, nullptr, out, m->error, (cudaStream_t)stream));
     return LPDF_OK;
 }
 
@@ -204,9 +202,8 @@ int lpdf_mlp_gradient(lpdf_mlp* m, const float* feat, const float* tgt, int64_t 
         TRY(cudaMalloc((void**)&m->losses, sizeof(double) * 1));
         m->losses_cap = 1;
     }
-    TRY(launch_mlp_forward(feat, B, m->P, m->pack, m->norm, m->out, nullptr, m->act, m->error, st));
-    TRY(launch_mlp_backward(feat, tgt, B, m->pack, m->norm, m->out, m->act, m->part, m->grad, m->error, st));
-    TRY(launch_mlp_loss(m->out, tgt, B, m->norm, m->losses, st));
+    TRY(launch_mlp_gradient(feat, tgt, B, m->P, m->pack, m->norm, m->part, m->lpart, m->error, st));
+    TRY(launch_mlp_reduce(m->part, m->lpart, B, m->grad, m->P, m->m, m->v, 0.0f, 0, m->pack, m->losses, st));
     std::vector<float> g(kParams);
     double l = 0.0;
     TRY(cudaMemcpyAsync(g.data(), m->grad, sizeof(float) * kParams, cudaMemcpyDeviceToHost, st));
@@ -236,10 +233,9 @@ int lpdf_mlp_train(lpdf_mlp* m, const float* feat, const float* tgt, int64_t B, 
         const int64_t off = (s % nchunk) * batch;
         const float* f = feat + off * kIn;
         const float* t = tgt + off * kOut;
-        TRY(launch_mlp_forward(f, batch, m->P, m->pack, m->norm, m->out, nullptr, m->act, m->error, st));
-        TRY(launch_mlp_backward(f, t, batch, m->pack, m->norm, m->out, m->act, m->part, m->grad, m->error, st));
-        TRY(launch_mlp_loss(m->out, t, batch, m->norm, m->losses + s, st));
-        TRY(launch_mlp_adam(m->P, m->grad, m->m, m->v, lr, ++m->step, m->pack, st));
+        TRY(launch_mlp_gradient(f, t, batch, m->P, m->pack, m->norm, m->part, m->lpart, m->error, st));
+        TRY(launch_mlp_reduce(m->part, m->lpart, batch, nullptr, m->P, m->m, m->v, lr, ++m->step, m->pack,
+                              m->losses + s, st));
     }
     if (losses && steps > 0)
         TRY(cudaMemcpyAsync(losses, m->losses, sizeof(double) * steps, cudaMemcpyDeviceToHost, st));
@@ -303,7 +299,7 @@ int lpdf_surrogate_relax_solve(const lpdf_mesh* mesh, lpdf_mlp* m, const lpdf_pa
     int it[2] = {0, 0};
     if (use_net) {
         TRY(surrogate_features(*F, stats, params->ns, nullptr, params->C0, m->s_feat, nullptr, st));
-        TRY(launch_mlp_forward(m->s_feat, N, m->P, m->pack, m->norm, m->s_out, nullptr, nullptr, m->error, st));
+        TRY(launch_mlp_forward(m->s_feat, N, m->P, m->pack, m->norm, m->s_out, nullptr, m->error, st));
         const cudaError_t e = node_fields_solve(*F, stats, *params, net_fields, tol, maxit, it, st, m->s_out, m->norm);
         if (e == cudaErrorNotReady)
             return lpdf_set_error(LPDF_ERR_CG_NOCONV, "surrogate_relax_solve: pressure CG did not converge");

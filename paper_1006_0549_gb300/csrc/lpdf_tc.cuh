@@ -121,6 +121,51 @@ __device__ __forceinline__ bool mbar_wait(unsigned long long* bar, uint32_t pari
     return false;
 }
 
+// the same of 32 columns
+__device__ __forceinline__ void tmem_ld32(uint32_t taddr, float* v)
+{
+    uint32_t r[32];
+    asm volatile(
+        "tcgen05.ld.sync.aligned.32x32b.x32.b32 {%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, %15, "
+        "%16, %17, %18, %19, %20, %21, %22, %23, %24, %25, %26, %27, %28, %29, %30, %31}, [%32];"
+        : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]), "=r"(r[8]),
+          "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15]), "=r"(r[16]),
+          "=r"(r[17]), "=r"(r[18]), "=r"(r[19]), "=r"(r[20]), "=r"(r[21]), "=r"(r[22]), "=r"(r[23]), "=r"(r[24]),
+          "=r"(r[25]), "=r"(r[26]), "=r"(r[27]), "=r"(r[28]), "=r"(r[29]), "=r"(r[30]), "=r"(r[31])
+        : "r"(taddr)
+        : "memory");
+#pragma unroll
+    for (int i = 0; i < 32; ++i) v[i] = __uint_as_float(r[i]);
+}
+
+// An operand of a GEMM: a matrix [r][k] of K columns in the core-matrix layout, read as it is (K-major:
+// its rows are the operand's M or N, its columns the summation) or transposed (MN-major: its columns
+// are M or N, its rows the summation). lbo, sbo: the descriptor's byte offsets; step: the bytes from one
+// 16-deep slice of the summation to the next. K-major, no swizzle: lbo is the distance of the cores
+// along the summation (128), sbo along M or N. MN-major, no swizzle: sbo is the distance along M or N
+// (128), lbo along the summation; a core is then 8 summation rows of 8 contiguous M or N values.
+struct Operand {
+    uint32_t addr, lbo, sbo, step;
+};
+__device__ __forceinline__ Operand k_major(const void* p, int K)
+{
+    return {smem_u32(p), 128u, (uint32_t)(K / 8) * 128u, 256u};
+}
+__device__ __forceinline__ Operand mn_major(const void* p, int K)
+{
+    return {smem_u32(p), (uint32_t)(K / 8) * 128u, 128u, (uint32_t)(K / 8) * 256u};
+}
+
+// D (128 x N, FP32 in TMEM) = A B^T over `slices` slices of 16, by the calling thread; no commit
+__device__ __forceinline__ void gemm_issue_op(uint32_t d_tmem, const Operand& A, const Operand& B, int N, int slices,
+                                              bool a_mn, bool b_mn)
+{
+    const uint32_t idesc = idesc_bf16(128, N) | ((uint32_t)a_mn << 15) | ((uint32_t)b_mn << 16);
+    for (int s = 0; s < slices; ++s)
+        mma_bf16(d_tmem, smem_desc(A.addr + A.step * s, A.lbo, A.sbo), smem_desc(B.addr + B.step * s, B.lbo, B.sbo),
+                 idesc, s > 0);
+}
+
 // One GEMM tile: D (128 x N, FP32 in TMEM at d_tmem) = A (128 x K) * B (N x K)^T, both in the
 // core-matrix layout, issued by the calling (single) thread: K / 16 MMAs, then a commit.
 __device__ __forceinline__ void gemm_issue(uint32_t d_tmem, const void* A, const void* B, int N, int K,
