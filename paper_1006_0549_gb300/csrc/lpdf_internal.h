@@ -171,8 +171,8 @@ cudaError_t launch_tc_gemm(const void* A, const void* B, float* D, int M, int N,
 // P1 finite-element tables of the gridpoint solve (lpdf_solve.cu), built once per mesh.
 // DOFs are the geometric nodes with periodic partners merged (numbered in node order).
 struct Fem {
-    static constexpr int kWorkPerDof = 65;     // FP64 scratch per DOF
-    static constexpr int kDotBlocks = 1024;    // partial sums of one dot product
+    static constexpr int kWorkPerDof = 73;     // FP64 scratch per DOF
+    static constexpr int kDotBlocks = 1024;    // partial sums of one sum
     int ndof = 0, nnz = 0, E = 0, N = 0;
     int* dof = nullptr;          // geometric node -> DOF
     int* dof_node = nullptr;     // DOF -> its master node (statistics row)
@@ -188,13 +188,22 @@ struct Fem {
     int* cel = nullptr;
     double* Mval = nullptr;      // consistent mass matrix
     double* Kval = nullptr;      // stiffness matrix (unit coefficient)
+    double* Kdiag = nullptr;     // its diagonal
     double* Aval = nullptr;      // M + L^2 K of the current solve
     unsigned char* wall = nullptr;
     double* normal = nullptr;    // inward unit normal per wall DOF
     double* work = nullptr;      // kWorkPerDof * ndof + 16 * E doubles
-    double* part = nullptr;      // 12 * kDotBlocks: partial sums of up to three 4-vector dot products
-    double* scal = nullptr;      // CG scalars (device)
-    double* scal_host = nullptr; // pinned copy
+    double* part = nullptr;      // kDotBlocks partial sums
+    // the CG kernels: their grid's CTAs at most, the words of the partial sums and of z (epoch 0 at
+    // first), the epoch that the next launch starts from (a word never sees the same one twice) and
+    // the result
+    int cg_ctas = 1, max_deg = 0;    // max_deg: matrix entries of a row at most
+    void* cg_slots = nullptr;
+    ulonglong2* cg_z = nullptr;
+    unsigned long long cg_epoch = 1;
+    int* cg_out = nullptr;
+    int* cg_host = nullptr;      // pinned copy
+    std::vector<int> row_host;   // the matrix pattern's row starts
     bool has_wp = false;         // the scratch holds a previous relaxation / pressure solution
     bool has_p = false;
     // wall distance of every geometric node (inputs of the learned surrogate)
@@ -205,15 +214,6 @@ struct Fem {
     int* ncomp = nullptr;        // component of every geometric node
     int nseg = 0, n_comp = 1;
     double period = 0.0;         // x period (0: none)
-    // CUDA graphs of kCheckEvery CG iterations, one per call site (its matrix, diagonal, solution
-    // and scratch pointers, component count and wall mask)
-    struct CgGraph {
-        const void* key[4];
-        int nv, mask;
-        cudaGraphExec_t exec;
-    };
-    std::vector<CgGraph> cg_graphs;
-    cudaStream_t capture_stream = nullptr;
     double* wdist = nullptr;     // per geometric node, filled on first use: distance to the wall,
     int* wseg = nullptr;         //   the wall edge of the nearest wall point
     double* wt = nullptr;        //   and its position on that edge (0 at a, 1 at b)

@@ -30,7 +30,7 @@ namespace lpdf {
 namespace {
 
 constexpr int kDotThreads = 256;
-constexpr int kCheckEvery = 8;   // CG iterations between host-side convergence tests
+constexpr int kCheckEvery = 8;   // CG iterations between convergence tests
 
 template <class T>
 cudaError_t upload(T** d, const std::vector<T>& h)
@@ -57,68 +57,69 @@ __global__ void elem_grad_kernel(const Fem F, const double* __restrict__ f, int 
     }
 }
 
-// area-weighted average of m element values to the DOFs: out[d ld + i]
+// area-weighted average of m element values to the DOFs: out[d ld + i], a thread per value
 __global__ void recover_kernel(const Fem F, const double* __restrict__ ev, int m, double* __restrict__ out, int ld)
 {
-    const int d = blockIdx.x * blockDim.x + threadIdx.x;
-    if (d >= F.ndof) return;
-    const double inv = 1.0 / F.darea[d];
-    for (int i = 0; i < m; ++i) {
-        double s = 0.0;
-        for (int t = F.de_ptr[d]; t < F.de_ptr[d + 1]; ++t) {
-            const int e = F.de_el[t] / 3;
-            s += F.area[e] * ev[(size_t)e * m + i];
-        }
-        out[(size_t)d * ld + i] = s * inv;
+    const int64_t t0 = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    if (t0 >= (int64_t)F.ndof * m) return;
+    const int d = (int)(t0 / m), i = (int)(t0 - (int64_t)d * m);
+    double s = 0.0;
+    for (int t = F.de_ptr[d]; t < F.de_ptr[d + 1]; ++t) {
+        const int e = F.de_el[t] / 3;
+        s += F.area[e] * ev[(size_t)e * m + i];
     }
+    out[(size_t)d * ld + i] = s * (1.0 / F.darea[d]);
 }
 
-// element divergence of a recovered gradient field g (d/dx at g[d ld], d/dy at g[d ld + 1])
-__global__ void elem_div_kernel(const Fem F, const double* __restrict__ g, int ld, double* __restrict__ out)
+// element divergences of the three recovered gradients g (6 per DOF: d/dx, d/dy of each): out[3 e + i]
+__global__ void elem_div_kernel(const Fem F, const double* __restrict__ g, double* __restrict__ out)
 {
-    const int e = blockIdx.x * blockDim.x + threadIdx.x;
-    if (e >= F.E) return;
-    const double* gr = F.grad + 6 * e;
+    const int64_t t0 = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    if (t0 >= 3 * (int64_t)F.E) return;
+    const int e = (int)(t0 / 3), i = (int)(t0 - 3 * (int64_t)e);
+    const double* gr = F.grad + 6 * (size_t)e;
     double s = 0.0;
     for (int a = 0; a < 3; ++a) {
-        const size_t d = F.edof[3 * e + a];
-        s += g[d * ld] * gr[2 * a] + g[d * ld + 1] * gr[2 * a + 1];
+        const size_t d = F.edof[3 * (size_t)e + a];
+        s += g[6 * d + 2 * i] * gr[2 * a] + g[6 * d + 2 * i + 1] * gr[2 * a + 1];
     }
-    out[e] = s;
+    out[t0] = s;
 }
 
 // ---------------------------------------------------------------- per-DOF statistics
-// statistics rows (S0, means, central moments, <omega>, <phi>, ...) of the DOF's master node
-__global__ void dof_stats_kernel(const Fem F, const double* __restrict__ st, int nq, int ns, double* __restrict__ U,
-                                 double* __restrict__ R, double* __restrict__ om, double* __restrict__ phi,
-                                 double* __restrict__ k, double* __restrict__ eps)
+// statistics rows (S0, means, central moments, <omega>, <phi>, ...) of the DOF's master node, and
+// the squared relaxation length L^2, L = CL max(k^1.5/eps, Ceta nu^0.75/eps^0.25): once per DOF (an
+// element averages its three), its powers as square roots. kol = Ceta nu^0.75
+__global__ void dof_stats_kernel(const Fem F, const double* __restrict__ st, int nq, int ns, double CL, double kol,
+                                 double* __restrict__ U, double* __restrict__ R, double* __restrict__ om,
+                                 double* __restrict__ phi, double* __restrict__ k, double* __restrict__ eps,
+                                 double* __restrict__ L2)
 {
     const int d = blockIdx.x * blockDim.x + threadIdx.x;
     if (d >= F.ndof) return;
     const double* s = st + (size_t)F.dof_node[d] * nq;
-    for (int i = 0; i < 3; ++i) U[3 * d + i] = s[1 + i];
-    for (int i = 0; i < 6; ++i) R[6 * d + i] = s[4 + i];
+    for (int i = 0; i < 3; ++i) U[3 * (size_t)d + i] = s[1 + i];
+    for (int i = 0; i < 6; ++i) R[6 * (size_t)d + i] = s[4 + i];
     om[d] = s[10];
     for (int a = 0; a < ns; ++a) phi[(size_t)d * ns + a] = s[11 + a];
     const double kk = 0.5 * (s[4] + s[7] + s[9]);
+    const double e = kk * s[10];
     k[d] = kk;
-    eps[d] = kk * s[10];
+    eps[d] = e;
+    if (L2) {
+        const double ep = fmax(e, 1e-12), kp = fmax(kk, 0.0);
+        const double L = CL * fmax(kp * sqrt(kp) / ep, kol / sqrt(sqrt(ep)));
+        L2[d] = L * L;
+    }
 }
 
 // ---------------------------------------------------------------- assembly
-__global__ void elem_L2_kernel(const Fem F, const double* __restrict__ k, const double* __restrict__ eps, double CL,
-                               double Ceta, double nu, double* __restrict__ L2e)
+__global__ void elem_L2_kernel(const Fem F, const double* __restrict__ L2, double* __restrict__ L2e)
 {
     const int e = blockIdx.x * blockDim.x + threadIdx.x;
     if (e >= F.E) return;
-    const double kol = Ceta * pow(nu, 0.75);
     double s = 0.0;
-    for (int a = 0; a < 3; ++a) {
-        const int d = F.edof[3 * e + a];
-        const double ep = fmax(eps[d], 1e-12);
-        const double L = CL * fmax(pow(fmax(k[d], 0.0), 1.5) / ep, kol / pow(ep, 0.25));
-        s += L * L;
-    }
+    for (int a = 0; a < 3; ++a) s += L2[F.edof[3 * e + a]];
     L2e[e] = s / 3.0;
 }
 
@@ -141,15 +142,7 @@ __global__ void assemble_kernel(const Fem F, const double* __restrict__ L2e, dou
     }
 }
 
-__global__ void diag_kernel(const Fem F, const double* __restrict__ A, double* __restrict__ diag)
-{
-    const int i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= F.ndof) return;
-    for (int j = F.row[i]; j < F.row[i + 1]; ++j)
-        if (F.col[j] == i) diag[i] = A[j];
-}
-
-// ---------------------------------------------------------------- batched PCG (nv <= 4 vectors)
+// ---------------------------------------------------------------- batched PCG
 // vectors are stored component-major: v[c n + i]
 
 // y_c = A x_c; rows of fixed (wall) DOFs give 0 when `mask` is set
@@ -169,176 +162,562 @@ __global__ void spmv_kernel(const Fem F, const double* __restrict__ A, const dou
     for (int c = 0; c < nv; ++c) y[c * n + i] = s[c];
 }
 
-// r = b - y (0 on fixed rows); z = r / diag; p = z
-__global__ void cg_start_kernel(const Fem F, const double* __restrict__ b, const double* __restrict__ y,
-                                const double* __restrict__ diag, double* __restrict__ r, double* __restrict__ z,
-                                double* __restrict__ p, int mask, int nv)
+// Jacobi-preconditioned CG on one or two systems of the mesh's pattern (the relaxation's four
+// right-hand sides and the pressure's one) in ONE cooperative launch, all components side by side.
+//
+// What bounds it: the chain of dependent steps of an iteration, not bytes (the matrix is a few MB)
+// and not the launch any more (five launches per iteration took 20-33 us). Measured on this GPU: a
+// warp's FP64 instruction takes 65 cycles, dependent or not (an SM sub-partition works on one at a
+// time, 0.5 lanes per cycle), a division 600, a load from L2 330, a store with a fence 780. So the
+// kernels count FP64 instructions on the critical path, divide once per sum, and never fence:
+// every value that another warp reads travels as one 16-byte word (value, epoch), stored and loaded
+// whole; a reader polls until the epoch is the one it waits for. The sums' partials travel the same
+// way and are added in a fixed order, so a run gives the same bits every time.
+// A word is overwritten only after everyone has read it: the next z is stored when the sum p.Ap of
+// this iteration is known, whose partials depend on every read of the present z, and likewise for
+// the partials. Polls are bounded; a warp that gives up records it and ends, and so do then the
+// others.
+//
+// Converged when ||r_c|| <= tol ||r_c(xref)|| for every c of a system (xref NULL: the start itself),
+// tested every kCheckEvery iterations and at maxit; a converged system stops there.
+constexpr int kCgComps = 5;                       // components at most
+constexpr int kCgSmallRows = 2048, kCgDeg = 12;   // cg_small_kernel: rows, matrix entries per row at most
+constexpr int kCgSmallUnits = kCgSmallRows / 32;
+constexpr int kCgMaxThreads = 1024;               // cg_kernel
+constexpr int kCgMaxTries = 1 << 21;              // polls (of about 0.2 us) before a wait gives up
+enum { kCgIts0 = 0, kCgIts1 = 1, kCgOk = 2, kCgError = 3, kCgOut = 4 };   // kCgOk: systems converged
+
+struct CgArgs {
+    int n, nc, nv0, wpc, maxit, slice;      // slice: matrix entries per CTA in shared memory (0: none fit)
+    int mask0, mask1;
+    const int *row, *col;
+    const unsigned char* wall;
+    const double *A0, *A1, *d0, *d1, *b0, *b1, *ref0, *ref1;
+    double *x0, *x1;
+    double* state;                          // 4 nc n (r, p, q, 1/diag of cg_kernel with several rows per thread)
+    double tol;
+    unsigned long long epoch;
+    ulonglong2 *z, *slots;                  // nc n words; the partial sums' words
+    int* out;
+};
+
+__device__ __forceinline__ void word_store(ulonglong2* p, double v, unsigned long long epoch)
 {
-    const int i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= F.ndof) return;
-    const size_t n = F.ndof;
-    const bool fixed = mask && F.wall[i];
-    for (int c = 0; c < nv; ++c) {
-        const double rr = fixed ? 0.0 : b[c * n + i] - y[c * n + i];
-        r[c * n + i] = rr;
-        z[c * n + i] = rr / diag[i];
-        p[c * n + i] = rr / diag[i];
+    asm volatile(
+        "{\n\t.reg .b128 t;\n\t"
+        "mov.b128 t, {%1, %2};\n\t"
+        "st.relaxed.gpu.global.b128 [%0], t;\n\t}" ::"l"(p), "l"(__double_as_longlong(v)), "l"(epoch)
+        : "memory");
+}
+// the word's value; ok stays set only if its epoch is the expected one
+__device__ __forceinline__ double word_load(const ulonglong2* p, unsigned long long epoch, bool& ok)
+{
+    long long b;
+    unsigned long long e;
+    asm volatile(
+        "{\n\t.reg .b128 t;\n\t"
+        "ld.relaxed.gpu.global.b128 t, [%2];\n\t"
+        "mov.b128 {%0, %1}, t;\n\t}"
+        : "=l"(b), "=l"(e)
+        : "l"(p)
+        : "memory");
+    ok = ok && e == epoch;
+    return __longlong_as_double(b);
+}
+
+__device__ __forceinline__ double shfl_add(double v, int o) { return __dadd_rn(v, __shfl_down_sync(0xffffffffu, v, o)); }
+
+// a / b correctly rounded, given y = 1 / b correctly rounded (Markstein 1990): three FP64
+// instructions instead of a division
+__device__ __forceinline__ double div_by(double a, double b, double y)
+{
+    const double q = __dmul_rn(a, y);
+    return __fma_rn(__fma_rn(-q, b, a), y, q);
+}
+
+// ---- up to kCgSmallRows rows: a warp per 32 rows of a component, no CTA or grid barrier at all.
+// Unit u of a component is the rows 256 (u / 8) + u % 8 + 8 lane, whose words lie side by side (a
+// neighbouring row's is then mostly the same lane's of the next unit). Every warp polls the units'
+// partial sums itself (at most two words per lane) and adds them as a 256-thread block tree and
+// then block by block. It keeps the p of its rows' neighbours in registers and advances them
+// (p = z + beta p) from the neighbours' z, so p never travels; the z words are polled together with
+// the partials of r.z.
+__device__ __forceinline__ double cg_small_sum(double v0, double v1, int nu, int nb)
+{
+    v0 = shfl_add(shfl_add(shfl_add(v0, 4), 2), 1);
+    if (nu > 32) v1 = shfl_add(shfl_add(shfl_add(v1, 4), 2), 1);
+    double sum = __shfl_sync(0xffffffffu, v0, 0);
+    for (int b = 1; b < nb; ++b) {
+        const double t = __shfl_sync(0xffffffffu, b < 4 ? v0 : v1, (8 * b) & 31);
+        sum = __dadd_rn(sum, t);
+    }
+    return sum;
+}
+
+__device__ __forceinline__ double cg_small_total(const ulonglong2* s, int nu, int nb, unsigned long long epoch, int lane,
+                                                 bool& alive)
+{
+    double v0, v1;
+    bool ok;
+    int tries = 0;
+    do {
+        ok = true;
+        v0 = lane < nu ? word_load(s + lane, epoch, ok) : 0.0;
+        v1 = lane + 32 < nu ? word_load(s + lane + 32, epoch, ok) : 0.0;
+        ok = __all_sync(0xffffffffu, ok);
+    } while (!ok && ++tries < kCgMaxTries);
+    alive = alive && ok;
+    return cg_small_sum(v0, v1, nu, nb);
+}
+
+__device__ __forceinline__ double warp_tree(double v)
+{
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) v = shfl_add(v, o);
+    return v;   // lane 0's
+}
+
+__global__ void __launch_bounds__(32) cg_small_kernel(const __grid_constant__ CgArgs a)
+{
+    const int lane = threadIdx.x, nb = (a.n + 255) / 256, nu = 8 * nb;
+    const int c = blockIdx.x / nu, u = blockIdx.x - c * nu;
+    const bool sys = c >= a.nv0;
+    const int v = sys ? c - a.nv0 : c, c0 = sys ? a.nv0 : 0, c1 = sys ? a.nc : a.nv0;   // the system's components
+    const size_t n = a.n;
+    const int i = 256 * (u >> 3) + (u & 7) + 8 * lane;
+    const bool live = i < a.n;
+    const double* const A = sys ? a.A1 : a.A0;
+    const double* const ref = sys ? a.ref1 : a.ref0;
+    double* const x = (sys ? a.x1 : a.x0) + v * n;
+    ulonglong2* const zw = a.z + (size_t)c * 256 * nb;
+    // words of the partial sums: [p.Ap, r.z, r0.r0, r.r, r.r][component][unit]; r.r in two sets used in
+    // turn, as the components of a system only meet at the tests
+    auto slot = [&](int k, int cc) { return a.slots + ((size_t)k * kCgComps + cc) * kCgSmallUnits; };
+    const bool fixed = live && (sys ? a.mask1 : a.mask0) && a.wall[i];
+    const int rs = live ? a.row[i] : 0, deg = live ? a.row[i + 1] - rs : 0;
+    const int wdeg = __reduce_max_sync(0xffffffffu, deg);
+    int word[kCgDeg];                          // the words of the row's columns
+    int self = -1;
+    double av[kCgDeg], pn[kCgDeg], zn[kCgDeg];
+    double y = 0.0, yref = 0.0;
+#pragma unroll
+    for (int t = 0; t < kCgDeg; ++t) {
+        const int j = t < deg ? a.col[rs + t] : -1;
+        word[t] = j >= 0 ? (j & ~255) + 32 * (j & 7) + ((j & 255) >> 3) : -1;
+        self = j == i ? t : self;
+        av[t] = t < deg && !fixed ? A[rs + t] : 0.0;
+        pn[t] = 0.0;
+        if (j >= 0) {
+            y = __fma_rn(av[t], x[j], y);
+            if (ref) yref = __fma_rn(av[t], ref[v * n + j], yref);
+        }
+    }
+    const double b = live ? (sys ? a.b1 : a.b0)[v * n + i] : 0.0;
+    const double diag = live ? (sys ? a.d1 : a.d0)[i] : 1.0, dinv = 1.0 / diag;
+    double xv = live ? x[i] : 0.0;
+    double r = fixed ? 0.0 : __dsub_rn(b, y);
+    double z = div_by(r, diag, dinv), q = 0.0;
+    unsigned long long epoch = a.epoch;
+    bool alive = true;
+    auto post = [&](int k, double value) {
+        const double s = warp_tree(value);
+        if (lane == 0) word_store(slot(k, c) + u, s, epoch);
+    };
+    ulonglong2* const mine = zw + 32 * u + lane;
+    if (live) word_store(mine, z, epoch);
+    const double rref = ref ? (fixed ? 0.0 : __dsub_rn(b, yref)) : r;
+    post(1, __dmul_rn(r, z));
+    post(2, __dmul_rn(rref, rref));
+    post(3, __dmul_rn(r, r));
+    // the sum of r.z, and the z of the row's columns into zn
+    auto gather = [&]() {
+        bool ok;
+        int tries = 0;
+        auto load = [&]() {
+            ok = true;
+#pragma unroll
+            for (int t = 0; t < kCgDeg; ++t) zn[t] = word[t] >= 0 ? word_load(zw + word[t], epoch, ok) : 0.0;
+        };
+        load();
+        const double sum = cg_small_total(slot(1, c), nu, nb, epoch, lane, alive);
+        while (!__all_sync(0xffffffffu, ok) && ++tries < kCgMaxTries) load();   // mostly there by now
+        alive = alive && __all_sync(0xffffffffu, ok);
+        return sum;
+    };
+    double rz = gather();
+    double r0[4], beta = 0.0;
+#pragma unroll
+    for (int k = 0; k < 4; ++k)
+        r0[k] = c0 + k < c1 ? a.tol * sqrt(cg_small_total(slot(2, c0 + k), nu, nb, epoch, lane, alive)) : 0.0;
+    bool done = false;
+    int it = 0, set = 3;
+    for (; alive; ++it) {
+        if (it % kCheckEvery == 0 || it >= a.maxit) {
+            done = true;
+#pragma unroll
+            for (int k = 0; k < 4; ++k)
+                if (c0 + k < c1 && sqrt(cg_small_total(slot(set, c0 + k), nu, nb, epoch, lane, alive)) > r0[k]) done = false;
+            if (!alive || done || it >= a.maxit) break;
+            set = 7 - set;
+        }
+        // p of the row and its neighbours, q = A p
+        q = 0.0;
+        double p = 0.0;
+        auto advance = [&](int t) {
+            pn[t] = __fma_rn(beta, pn[t], zn[t]);
+            q = __fma_rn(av[t], pn[t], q);
+            p = self == t ? pn[t] : p;
+        };
+#pragma unroll
+        for (int t = 0; t < 7; ++t) advance(t);   // an interior row of a triangulation: 7 on average
+        if (wdeg > 7) {
+            advance(7);
+            advance(8);
+            if (wdeg > 9)
+#pragma unroll
+                for (int t = 9; t < kCgDeg; ++t) advance(t);
+        }
+        ++epoch;
+        post(0, __dmul_rn(p, q));
+        const double pq = cg_small_total(slot(0, c), nu, nb, epoch, lane, alive);
+        const double alpha = pq != 0.0 ? rz / pq : 0.0;
+        r = __fma_rn(-alpha, q, r);
+        z = div_by(r, diag, dinv);
+        if (live) word_store(mine, z, epoch);
+        post(1, __dmul_rn(r, z));
+        if ((it + 1) % kCheckEvery == 0 || it + 1 >= a.maxit) post(set, __dmul_rn(r, r));
+        xv = __fma_rn(alpha, p, xv);
+        asm volatile("" : "+d"(rz));   // the reciprocal for beta is formed here, while the sum travels
+        const double yrz = 1.0 / rz;
+        const double rznew = gather();
+        beta = rz != 0.0 ? div_by(rznew, rz, yrz) : 0.0;
+        rz = rznew;
+    }
+    if (!alive) {
+        if (lane == 0) atomicExch(a.out + kCgError, 1);
+        return;
+    }
+    if (live) x[i] = xv;
+    if (v == 0 && u == 0 && lane == 0) {
+        a.out[sys ? kCgIts1 : kCgIts0] = it;
+        if (done) atomicAdd(a.out + kCgOk, 1);
     }
 }
 
-// per-block partial sums of x_c . y_c, fixed order
-__global__ void dot_kernel(const double* __restrict__ x, const double* __restrict__ y, int n, int nv,
-                           double* __restrict__ part)
+// ---- any number of rows. CTA b owns the rows [n b / G, n (b + 1) / G) of every component; a warp
+// works on one component (wpc warps each), a lane on one row, so neighbouring lanes gather
+// neighbouring rows. kOne: at most one row per thread, so x, r, p, q and 1/diag stay in registers
+// for the whole solve; otherwise they live in global memory (touched by their thread alone). Only
+// z = r/diag is read by other CTAs: A p is carried along by q = A z + beta q, so p never travels.
+// kSmem: the CTA's slice of the matrix is staged in shared memory once.
+// A sum goes over the CTA's lanes to one word per CTA; one warp of one CTA per value collects the
+// words, divides, and publishes the coefficient, which every CTA polls: two trips through L2. (All
+// CTAs polling all words is one trip, but 152 x 152 polls of the same few lines took 12 us per
+// iteration.) kCgTasks warps of a CTA do nothing else; meanwhile the others gather the neighbours'
+// new z and form A z, which does not need beta.
+constexpr int kCgTasks = 2;
+struct CgShared {
+    double red[3][kCgMaxThreads / 32 - kCgTasks][32];   // the threads' values
+    double res[3][8];            // published sums
+    double coef[8];              // alpha or beta of every component
+    double rz[8];                // the collector's copy
+    double r0[8], rr[8];
+    unsigned active;             // components still iterating
+    int stop, fail;
+};
+
+constexpr int kCgPoll = 5;   // words polled at once by a lane
+
+// The grid sums of `nval` values of every active component, by the task warps (w of kCgTasks); mode
+// 0: res only; 1: coef = alpha = rz / sum; 2: value 0 is r.z, coef = beta. Words: partials
+// [3][kCgComps][G] and published [2][3][kCgComps], in two sets used in turn.
+__device__ __forceinline__ void cg_exchange(const CgArgs& a, CgShared& s, int w, int nval, int set,
+                                            unsigned long long epoch, int mode)
 {
-    __shared__ double sh[4][kDotThreads];
-    double s[4] = {0, 0, 0, 0};
-    for (int i = blockIdx.x * kDotThreads + threadIdx.x; i < n; i += gridDim.x * kDotThreads)
-        for (int c = 0; c < nv; ++c) s[c] += x[(size_t)c * n + i] * y[(size_t)c * n + i];
-    for (int c = 0; c < 4; ++c) sh[c][threadIdx.x] = s[c];
+    const int lane = threadIdx.x & 31;
+    const int G = gridDim.x;
+    ulonglong2* const part = a.slots + (size_t)set * 3 * kCgComps * G;
+    ulonglong2* const pub = a.slots + 2 * (size_t)3 * kCgComps * G + set * 3 * kCgComps * 2;
+    for (int t = w; t < nval * a.nc; t += kCgTasks) {
+        const int k = t / a.nc, c = t - k * a.nc;
+        if (!((s.active >> c) & 1u)) continue;
+        double v = s.red[k][c * a.wpc][lane];
+        for (int q = 1; q < a.wpc; ++q) v = __dadd_rn(v, s.red[k][c * a.wpc + q][lane]);
+        v = warp_tree(v);
+        if (lane == 0) word_store(part + (size_t)t * G + blockIdx.x, v, epoch);
+    }
+    for (int t = w; t < nval * a.nc; t += kCgTasks) {
+        const int k = t / a.nc, c = t - k * a.nc;
+        if (!((s.active >> c) & 1u) || blockIdx.x != t % G) continue;
+        double sum = 0.0;
+        bool ok = true;
+        const double y = mode == 2 && k == 0 ? 1.0 / s.rz[c] : 0.0;
+        for (int j0 = lane; j0 < G; j0 += 32 * kCgPoll) {
+            double v[kCgPoll];
+            int tries = 0;
+            do {
+                ok = true;
+#pragma unroll
+                for (int q = 0; q < kCgPoll; ++q)
+                    v[q] = j0 + 32 * q < G ? word_load(part + (size_t)t * G + j0 + 32 * q, epoch, ok) : 0.0;
+            } while (!ok && ++tries < kCgMaxTries);
+            if (!ok) s.fail = 1;
+#pragma unroll
+            for (int q = 0; q < kCgPoll; ++q) sum = __dadd_rn(sum, v[q]);
+        }
+        sum = warp_tree(sum);
+        if (lane == 0) {
+            double coef = 0.0;
+            if (mode == 1) coef = sum != 0.0 ? s.rz[c] / sum : 0.0;
+            if (mode == 2 && k == 0) coef = s.rz[c] != 0.0 ? div_by(sum, s.rz[c], y) : 0.0;
+            word_store(pub + 2 * t, coef, epoch);
+            word_store(pub + 2 * t + 1, sum, epoch);
+        }
+    }
+    // lanes 2 q and 2 q + 1 poll this warp's q-th task
+    const int t = w + kCgTasks * (lane >> 1);
+    const int k = t / a.nc, c = t - k * a.nc;
+    if (t < nval * a.nc && ((s.active >> c) & 1u)) {
+        bool ok;
+        double v;
+        int tries = 0;
+        do {
+            ok = true;
+            v = word_load(pub + 2 * t + (lane & 1), epoch, ok);
+        } while (!ok && ++tries < kCgMaxTries);
+        if (!ok) s.fail = 1;
+        if (lane & 1) s.res[k][c] = v;
+        else if (mode && k == 0) s.coef[c] = v;
+    }
+}
+
+template <bool kOne, bool kSmem>
+__global__ void __launch_bounds__(kCgMaxThreads, 1) cg_kernel(const __grid_constant__ CgArgs a)
+{
+    extern __shared__ __align__(16) unsigned char dyn[];
+    __shared__ CgShared s;
+    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+    const int task = wid - a.nc * a.wpc;          // >= 0: a task warp
+    const int c = task >= 0 ? 0 : wid / a.wpc, sub = wid - c * a.wpc;
+    const bool sys = c >= a.nv0;
+    const int v = sys ? c - a.nv0 : c;
+    const size_t n = a.n;
+    const int lo = (int)((int64_t)a.n * blockIdx.x / gridDim.x), hi = (int)((int64_t)a.n * (blockIdx.x + 1) / gridDim.x);
+    const int base = a.row[lo];
+    const double* const gA = sys ? a.A1 : a.A0;
+    double* const sA0 = reinterpret_cast<double*>(dyn);
+    double* const sA1 = sA0 + (a.nv0 > 0 ? a.slice : 0);
+    int* const scol = reinterpret_cast<int*>(sA1 + (a.nc > a.nv0 ? a.slice : 0));
+    if (kSmem) {
+        const int m = a.row[hi] - base;
+        for (int t = threadIdx.x; t < m; t += blockDim.x) {
+            if (a.nv0 > 0) sA0[t] = a.A0[base + t];
+            if (a.nc > a.nv0) sA1[t] = a.A1[base + t];
+            scol[t] = a.col[base + t];
+        }
+    }
+    if (threadIdx.x == 0) {
+        s.active = (1u << a.nc) - 1u;
+        s.stop = 0;
+        s.fail = 0;
+    }
     __syncthreads();
-    for (int o = kDotThreads / 2; o > 0; o >>= 1) {
-        if (threadIdx.x < o)
-            for (int c = 0; c < 4; ++c) sh[c][threadIdx.x] += sh[c][threadIdx.x + o];
+    const double* const sA = sys ? sA1 : sA0;
+    unsigned long long epoch = a.epoch;
+    bool bad = false;
+    // (A f) of a row; f(j) loads entry j, up to kW at once, until every word has its epoch
+    constexpr int kW = 10;
+    auto row_dot = [&](int rs, int re, auto f) {
+        double sum = 0.0;
+        for (int t = rs; t < re; t += kW) {
+            double zv[kW];
+            bool ok;
+            int tries = 0;
+            do {
+                ok = true;
+#pragma unroll
+                for (int u = 0; u < kW; ++u)
+                    zv[u] = t + u < re ? f(kSmem ? scol[t + u - base] : __ldg(a.col + t + u), ok) : 0.0;
+            } while (!ok && ++tries < kCgMaxTries);
+            bad = bad || !ok;
+#pragma unroll
+            for (int u = 0; u < kW; ++u)
+                if (t + u < re) sum = __fma_rn(kSmem ? sA[t + u - base] : __ldg(gA + t + u), zv[u], sum);
+        }
+        return sum;
+    };
+    const int mask = sys ? a.mask1 : a.mask0;
+    const double* const b = (sys ? a.b1 : a.b0) + v * n;
+    const double* const ref0 = sys ? a.ref1 : a.ref0;
+    const double* const ref = ref0 ? ref0 + v * n : nullptr;
+    const double* const diag = sys ? a.d1 : a.d0;
+    double* const x = (sys ? a.x1 : a.x0) + v * n;
+    ulonglong2* const z = a.z + c * n;
+    double* const st = a.state + 4 * c * n;
+    const int first = task >= 0 ? hi : lo + 32 * sub + lane, stride = 32 * a.wpc;   // a task warp has no rows
+    // kOne: the row's state in registers
+    double xv = 0.0, rv = 0.0, pv = 0.0, qv = 0.0, zv = 0.0, dinv = 0.0, sv = 0.0;
+    int rs = 0, re = 0;
+    double s0 = 0.0, s1 = 0.0, s2 = 0.0;
+    for (int i = first; i < hi; i += stride) {
+        rs = a.row[i];
+        re = a.row[i + 1];
+        const bool fixed = mask && a.wall[i];
+        if (ref) {
+            const double r = fixed ? 0.0 : b[i] - row_dot(rs, re, [&](int j, bool&) { return ref[j]; });
+            s2 += r * r;
+        }
+        xv = x[i];
+        rv = fixed ? 0.0 : b[i] - row_dot(rs, re, [&](int j, bool&) { return x[j]; });
+        dinv = 1.0 / diag[i];
+        zv = rv * dinv;
+        word_store(z + i, zv, epoch);
+        s0 += rv * zv;
+        s1 += rv * rv;
+        if (fixed) re = rs;   // its row of A p is zero
+        if (!kOne) {
+            st[i] = rv;
+            st[n + i] = 0.0;
+            st[2 * n + i] = 0.0;
+            st[3 * n + i] = dinv;
+        }
+    }
+    if (!ref) s2 = s1;
+    // the sums of the threads' s0 (and s1, s2) over the grid; meanwhile, when `ahead` is set, A z
+    auto zword = [&](int j, bool& have) { return word_load(z + j, epoch, have); };
+    auto exchange = [&](int nval, int set, int mode, bool ahead) {
+        if (task < 0) {
+            s.red[0][wid][lane] = s0;
+            if (nval > 1) s.red[1][wid][lane] = s1;
+            if (nval > 2) s.red[2][wid][lane] = s2;
+        }
         __syncthreads();
+        if (task >= 0) cg_exchange(a, s, task, nval, set, epoch, mode);
+        else if (kOne && ahead && first < hi) sv = row_dot(rs, re, zword);
+        if (bad) s.fail = 1;
+        __syncthreads();
+        return !s.fail;
+    };
+    bool ok = exchange(3, 1, 0, true);
+    if (threadIdx.x < a.nc) {
+        s.rz[threadIdx.x] = s.res[0][threadIdx.x];
+        s.rr[threadIdx.x] = s.res[1][threadIdx.x];
+        s.r0[threadIdx.x] = sqrt(s.res[2][threadIdx.x]);
+        s.coef[threadIdx.x] = 0.0;
     }
-    if (threadIdx.x == 0)
-        for (int c = 0; c < 4; ++c) part[(size_t)c * gridDim.x + blockIdx.x] = sh[c][0];
-}
-
-// CG scalars, kept on the device (4 slots each): rz, the last plain dot, alpha, beta,
-// |r_0|^2, |r|^2
-enum { kRZ = 0, kDot = 4, kAlpha = 8, kBeta = 12, kR0 = 16, kRR = 20, kNScal = 24 };
-
-// sum the block partials of one dot product, then per mode
-// 0: sc[slot + c] = sum; 1: alpha = rz / sum; 2: beta = sum / rz, rz = sum
-__global__ void scalar_kernel(const double* __restrict__ part, int nb, int nv, int slot, int mode,
-                              double* __restrict__ sc)
-{
-    const int c = threadIdx.x;
-    if (c >= nv) return;
-    double s = 0.0;
-    for (int b = 0; b < nb; ++b) s += part[(size_t)c * nb + b];
-    if (mode == 0) {
-        sc[slot + c] = s;
-    } else if (mode == 1) {
-        sc[kAlpha + c] = s != 0.0 ? sc[kRZ + c] / s : 0.0;
-    } else {
-        sc[kBeta + c] = sc[kRZ + c] != 0.0 ? s / sc[kRZ + c] : 0.0;
-        sc[kRZ + c] = s;
-    }
-}
-
-// x_c += alpha_c p_c ; r_c -= alpha_c q_c ; z_c = r_c / diag
-__global__ void cg_update_kernel(int n, int nv, const double* __restrict__ sc, const double* __restrict__ diag,
-                                 const double* __restrict__ p, const double* __restrict__ q, double* __restrict__ x,
-                                 double* __restrict__ r, double* __restrict__ z)
-{
-    const int i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= n) return;
-    for (int c = 0; c < nv; ++c) {
-        const size_t o = (size_t)c * n + i;
-        const double a = sc[kAlpha + c];
-        x[o] += a * p[o];
-        const double rr = r[o] - a * q[o];
-        r[o] = rr;
-        z[o] = rr / diag[i];
-    }
-}
-
-// p_c = z_c + beta_c p_c
-__global__ void cg_direction_kernel(int n, int nv, const double* __restrict__ sc, const double* __restrict__ z,
-                                    double* __restrict__ p)
-{
-    const int i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= n) return;
-    for (int c = 0; c < nv; ++c) {
-        const size_t o = (size_t)c * n + i;
-        p[o] = z[o] + sc[kBeta + c] * p[o];
-    }
-}
-
-// q_c = A p_c (0 on fixed rows) and block partials of p_c . q_c (fixed order)
-__global__ void spmv_dot_kernel(const Fem F, const double* __restrict__ A, const double* __restrict__ p,
-                                double* __restrict__ q, int mask, int nv, double* __restrict__ part)
-{
-    __shared__ double sh[4][kDotThreads];
-    const size_t n = F.ndof;
-    double acc[4] = {0, 0, 0, 0};
-    for (int i = blockIdx.x * kDotThreads + threadIdx.x; i < F.ndof; i += gridDim.x * kDotThreads) {
-        double s[4] = {0, 0, 0, 0};
-        if (!(mask && F.wall[i]))
-            for (int t = F.row[i]; t < F.row[i + 1]; ++t) {
-                const int j = F.col[t];
-                const double a = A[t];
-                for (int c = 0; c < nv; ++c) s[c] += a * p[c * n + j];
+    __syncthreads();
+    int its0 = a.maxit, its1 = a.maxit, conv = 0;   // thread 0's
+    for (int it = 0; ok; ++it) {
+        if (it % kCheckEvery == 0 || it >= a.maxit) {
+            if (wid == 0) {
+                const bool far = lane < a.nc && ((s.active >> lane) & 1u) && sqrt(s.rr[lane]) > a.tol * s.r0[lane];
+                const unsigned f = __ballot_sync(0xffffffffu, far);
+                if (lane == 0) {
+                    const unsigned m0 = (1u << a.nv0) - 1u, m1 = ((1u << a.nc) - 1u) & ~m0;
+                    unsigned act = s.active;
+                    if ((act & m0) && !(f & m0)) { act &= ~m0; its0 = it; ++conv; }
+                    if ((act & m1) && !(f & m1)) { act &= ~m1; its1 = it; ++conv; }
+                    s.active = act;
+                    s.stop = act == 0u || it >= a.maxit;
+                }
             }
-        for (int c = 0; c < nv; ++c) {
-            q[c * n + i] = s[c];
-            acc[c] += p[c * n + i] * s[c];
+            __syncthreads();
+            if (s.stop) break;
+        }
+        const bool on = task < 0 && ((s.active >> c) & 1u);
+        // r.r is only needed at the next test
+        const bool test = (it + 1) % kCheckEvery == 0 || it + 1 >= a.maxit;
+        s0 = 0.0;
+        if (on) {
+            const double beta = s.coef[c];
+            if (kOne) {
+                pv = __fma_rn(beta, pv, zv);
+                qv = __fma_rn(beta, qv, sv);
+                s0 = pv * qv;
+            } else {
+                for (int i = first; i < hi; i += stride) {
+                    const int r0 = a.row[i], r1 = mask && a.wall[i] ? r0 : a.row[i + 1];
+                    const double p = __fma_rn(beta, st[n + i], st[i] * st[3 * n + i]);
+                    const double q = __fma_rn(beta, st[2 * n + i], row_dot(r0, r1, zword));
+                    st[n + i] = p;
+                    st[2 * n + i] = q;
+                    s0 = __fma_rn(p, q, s0);
+                }
+            }
+        }
+        ++epoch;
+        ok = exchange(1, 0, 1, false);
+        if (!ok) break;
+        s0 = s1 = 0.0;
+        if (on) {
+            const double alpha = s.coef[c];
+            if (kOne) {
+                if (first < hi) {
+                    rv = __fma_rn(-alpha, qv, rv);
+                    zv = rv * dinv;
+                    word_store(z + first, zv, epoch);
+                    s0 = rv * zv;
+                    if (test) s1 = rv * rv;
+                    xv = __fma_rn(alpha, pv, xv);
+                }
+            } else {
+                for (int i = first; i < hi; i += stride) {
+                    const double r = __fma_rn(-alpha, st[2 * n + i], st[i]), zz = r * st[3 * n + i];
+                    st[i] = r;
+                    word_store(z + i, zz, epoch);
+                    s0 = __fma_rn(r, zz, s0);
+                    s1 = __fma_rn(r, r, s1);
+                    x[i] = __fma_rn(alpha, st[n + i], x[i]);
+                }
+            }
+        }
+        ok = exchange(test ? 2 : 1, 1, 2, on);
+        if (threadIdx.x < a.nc) {
+            s.rz[threadIdx.x] = s.res[0][threadIdx.x];
+            if (test) s.rr[threadIdx.x] = s.res[1][threadIdx.x];
         }
     }
-    for (int c = 0; c < 4; ++c) sh[c][threadIdx.x] = acc[c];
-    __syncthreads();
-    for (int o = kDotThreads / 2; o > 0; o >>= 1) {
-        if (threadIdx.x < o)
-            for (int c = 0; c < 4; ++c) sh[c][threadIdx.x] += sh[c][threadIdx.x + o];
-        __syncthreads();
+    if (!ok) {
+        if (threadIdx.x == 0) atomicExch(a.out + kCgError, 1);
+        return;
     }
-    if (threadIdx.x == 0)
-        for (int c = 0; c < 4; ++c) part[(size_t)c * gridDim.x + blockIdx.x] = sh[c][0];
+    if (kOne && first < hi) x[first] = xv;
+    if (blockIdx.x == 0 && threadIdx.x == 0) {
+        a.out[kCgIts0] = a.nv0 > 0 ? its0 : 0;
+        a.out[kCgIts1] = a.nc > a.nv0 ? its1 : 0;
+        a.out[kCgOk] = conv;
+    }
 }
 
-// x += alpha p; r -= alpha q; z = r / diag; block partials of r . z and r . r
-__global__ void update_dot_kernel(int n, int nv, const double* __restrict__ sc, const double* __restrict__ diag,
-                                  const double* __restrict__ p, const double* __restrict__ q, double* __restrict__ x,
-                                  double* __restrict__ r, double* __restrict__ z, double* __restrict__ part_rz,
-                                  double* __restrict__ part_rr)
+// block partials of the sum of x, fixed order: a tree over 256 values
+__global__ void sum_kernel(const double* __restrict__ x, int n, double* __restrict__ part)
 {
-    __shared__ double sh[8][kDotThreads];
-    double a_rz[4] = {0, 0, 0, 0}, a_rr[4] = {0, 0, 0, 0};
-    for (int i = blockIdx.x * kDotThreads + threadIdx.x; i < n; i += gridDim.x * kDotThreads)
-        for (int c = 0; c < nv; ++c) {
-            const size_t o = (size_t)c * n + i;
-            const double al = sc[kAlpha + c];
-            x[o] += al * p[o];
-            const double rr = r[o] - al * q[o];
-            r[o] = rr;
-            const double zz = rr / diag[i];
-            z[o] = zz;
-            a_rz[c] += rr * zz;
-            a_rr[c] += rr * rr;
-        }
-    for (int c = 0; c < 4; ++c) {
-        sh[c][threadIdx.x] = a_rz[c];
-        sh[4 + c][threadIdx.x] = a_rr[c];
-    }
+    __shared__ double sh[kDotThreads];
+    double s = 0.0;
+    for (int i = blockIdx.x * kDotThreads + threadIdx.x; i < n; i += gridDim.x * kDotThreads) s += x[i];
+    sh[threadIdx.x] = s;
     __syncthreads();
     for (int o = kDotThreads / 2; o > 0; o >>= 1) {
-        if (threadIdx.x < o)
-            for (int c = 0; c < 8; ++c) sh[c][threadIdx.x] += sh[c][threadIdx.x + o];
+        if (threadIdx.x < o) sh[threadIdx.x] += sh[threadIdx.x + o];
         __syncthreads();
     }
-    if (threadIdx.x == 0)
-        for (int c = 0; c < 4; ++c) {
-            part_rz[(size_t)c * gridDim.x + blockIdx.x] = sh[c][0];
-            part_rr[(size_t)c * gridDim.x + blockIdx.x] = sh[4 + c][0];
-        }
+    if (threadIdx.x == 0) part[blockIdx.x] = sh[0];
 }
 
-// beta = rz_new / rz, rz = rz_new, rr (for the convergence test)
-__global__ void scalar_beta_kernel(const double* __restrict__ part_rz, const double* __restrict__ part_rr, int nb,
-                                   int nv, double* __restrict__ sc)
+constexpr size_t kCgSmemMax = 96 * 1024;
+
+// words of the partial sums (cg_small_kernel's, cg_kernel's with its published sums)
+size_t cg_slot_words(int ctas)
 {
-    const int c = threadIdx.x;
-    if (c >= nv) return;
-    double rz = 0.0, rr = 0.0;
-    for (int b = 0; b < nb; ++b) {
-        rz += part_rz[(size_t)c * nb + b];
-        rr += part_rr[(size_t)c * nb + b];
-    }
-    sc[kBeta + c] = sc[kRZ + c] != 0.0 ? rz / sc[kRZ + c] : 0.0;
-    sc[kRZ + c] = rz;
-    sc[kRR + c] = rr;
+    return std::max((size_t)5 * kCgComps * kCgSmallUnits, 2 * (size_t)3 * kCgComps * ctas + 2 * 3 * kCgComps * 2);
+}
+
+cudaError_t cg_configure()
+{
+    cudaError_t e = cudaFuncSetAttribute(cg_kernel<true, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kCgSmemMax);
+    if (e == cudaSuccess)
+        e = cudaFuncSetAttribute(cg_kernel<false, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kCgSmemMax);
+    return e;
 }
 
 // ---------------------------------------------------------------- right-hand sides
@@ -395,16 +774,23 @@ __global__ void pressure_rhs_kernel(const Fem F, const double* __restrict__ gT, 
     b[d] = s;
 }
 
-__global__ void fill_kernel(int n, double v, double* __restrict__ x)
+__global__ void subtract_mean_kernel(int n, const double* __restrict__ part, int nb, double* __restrict__ x)
 {
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i < n) x[i] = v;
+    double sum = 0.0;
+    for (int b = 0; b < nb; ++b) sum += part[b];
+    if (i < n) x[i] -= sum / n;
 }
 
-__global__ void subtract_mean_kernel(int n, const double* __restrict__ sum, double* __restrict__ x)
+// the converged solutions, kept as the next solve's start
+__global__ void keep_solution_kernel(const int* __restrict__ cg_out, int systems, int n4, const double* __restrict__ wp,
+                                     double* __restrict__ wp_prev, int n, const double* __restrict__ p,
+                                     double* __restrict__ p_prev)
 {
+    if (cg_out[kCgOk] != systems) return;
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i < n) x[i] -= sum[0] / n;
+    if (i < n4) wp_prev[i] = wp[i];
+    if (i < n) p_prev[i] = p[i];
 }
 
 // ---------------------------------------------------------------- the output fields
@@ -414,10 +800,12 @@ __global__ void fields_kernel(const Fem F, int ns, int nfp, const double* __rest
                               const double* __restrict__ gU, const double* __restrict__ lapU,
                               const double* __restrict__ gp, const double* __restrict__ wp, int gmodel, double C0,
                               double Comega1, double Comega2, double dpdx0, double dpdy0,
-                              const float* __restrict__ surr, const float* __restrict__ snorm, float* __restrict__ out)
+                              const float* __restrict__ surr, const float* __restrict__ snorm,
+                              const int* __restrict__ cg_out, int systems, float* __restrict__ out)
 {
     const int nd = blockIdx.x * blockDim.x + threadIdx.x;
     if (nd >= F.N) return;
+    if (cg_out && cg_out[kCgOk] != systems) return;   // a CG did not converge: the caller's fields stay
     const int d = F.dof[nd];
     const size_t n = F.ndof;
     const double* r = R + 6 * (size_t)d;       // uu, uv, uw, vv, vw, ww
@@ -643,7 +1031,7 @@ cudaError_t fem_build(const double* node_xy, int N, const int32_t* tri, int E, c
         for (int a = 0; a < 3; ++a)
             for (int b = 0; b < 3; ++b) rows[edof[3 * e + a]][edof[3 * e + b]].push_back(9 * e + 3 * a + b);
     std::vector<int> row(ndof + 1, 0), col, cptr(1, 0), cel;
-    std::vector<double> Mval, Kval;
+    std::vector<double> Mval, Kval, Kdiag(ndof, 0.0);
     for (int i = 0; i < ndof; ++i) {
         for (const auto& kv : rows[i]) {
             col.push_back(kv.first);
@@ -658,6 +1046,7 @@ cudaError_t fem_build(const double* node_xy, int N, const int32_t* tri, int E, c
             cptr.push_back((int)cel.size());
             Mval.push_back(m);
             Kval.push_back(kk);
+            if (kv.first == i) Kdiag[i] = kk;
         }
         row[i + 1] = (int)col.size();
     }
@@ -709,6 +1098,9 @@ cudaError_t fem_build(const double* node_xy, int N, const int32_t* tri, int E, c
     F->nseg = (int)(seg.size() / 4);
     F->n_comp = n_comp;
     F->period = period;
+    F->row_host = row;
+    for (int i = 0; i < ndof; ++i) F->max_deg = std::max(F->max_deg, row[i + 1] - row[i]);
+    F->cg_ctas = sm_count();
     if (seg.empty()) {
         seg.assign(4, 0.0);
         segn.assign(2, 0);
@@ -718,16 +1110,20 @@ cudaError_t fem_build(const double* node_xy, int N, const int32_t* tri, int E, c
         (e = upload(&F->area, area)) || (e = upload(&F->grad, grad)) || (e = upload(&F->de_ptr, de_ptr)) ||
         (e = upload(&F->de_el, de_el)) || (e = upload(&F->darea, darea)) || (e = upload(&F->row, row)) ||
         (e = upload(&F->col, col)) || (e = upload(&F->cptr, cptr)) || (e = upload(&F->cel, cel)) ||
-        (e = upload(&F->Mval, Mval)) || (e = upload(&F->Kval, Kval)) || (e = upload(&F->wall, wall)) ||
+        (e = upload(&F->Mval, Mval)) || (e = upload(&F->Kval, Kval)) || (e = upload(&F->Kdiag, Kdiag)) || (e = upload(&F->wall, wall)) ||
         (e = upload(&F->normal, normal)) || (e = upload(&F->xy, xy)) || (e = upload(&F->seg, seg)) ||
         (e = upload(&F->segn, segn)) || (e = upload(&F->seg_off, seg_off)) || (e = upload(&F->ncomp, ncomp_v)) || (e = cudaMalloc((void**)&F->wdist, sizeof(double) * std::max(1, N))) ||
         (e = cudaMalloc((void**)&F->wseg, sizeof(int) * std::max(1, N))) ||
         (e = cudaMalloc((void**)&F->wt, sizeof(double) * std::max(1, N))) ||
         (e = cudaMalloc((void**)&F->Aval, sizeof(double) * std::max(1, F->nnz))) ||
         (e = cudaMalloc((void**)&F->work, sizeof(double) * (Fem::kWorkPerDof * (size_t)ndof + 16 * (size_t)E))) ||
-        (e = cudaMalloc((void**)&F->part, sizeof(double) * 12 * Fem::kDotBlocks)) ||
-        (e = cudaMalloc((void**)&F->scal, sizeof(double) * kNScal)) ||
-        (e = cudaMallocHost((void**)&F->scal_host, sizeof(double) * kNScal))) {
+        (e = cudaMalloc((void**)&F->part, sizeof(double) * Fem::kDotBlocks)) ||
+        (e = cudaMalloc(&F->cg_slots, sizeof(ulonglong2) * cg_slot_words(F->cg_ctas))) ||
+        (e = cudaMemset(F->cg_slots, 0, sizeof(ulonglong2) * cg_slot_words(F->cg_ctas))) ||
+        (e = cudaMalloc((void**)&F->cg_z, sizeof(ulonglong2) * kCgComps * ((size_t)ndof + 255))) ||
+        (e = cudaMemset(F->cg_z, 0, sizeof(ulonglong2) * kCgComps * ((size_t)ndof + 255))) ||
+        (e = cudaMalloc((void**)&F->cg_out, sizeof(int) * kCgOut)) ||
+        (e = cudaMallocHost((void**)&F->cg_host, sizeof(int) * kCgOut)) || (e = cg_configure())) {
         fem_free(F);
         return e;
     }
@@ -739,111 +1135,48 @@ void fem_free(Fem* F)
 {
     if (!F) return;
     void* ps[] = {F->dof, F->dof_node, F->edof, F->area, F->grad, F->de_ptr, F->de_el, F->darea, F->row, F->col,
-                  F->cptr, F->cel, F->Mval, F->Kval, F->Aval, F->wall, F->normal, F->work, F->part, F->scal,
+                  F->cptr, F->cel, F->Mval, F->Kval, F->Kdiag, F->Aval, F->wall, F->normal, F->work, F->part, F->cg_slots, F->cg_z, F->cg_out,
                   F->xy, F->seg, F->segn, F->seg_off, F->ncomp, F->wdist, F->wseg, F->wt};
     for (void* p : ps) cudaFree(p);
-    cudaFreeHost(F->scal_host);
-    for (auto& g : F->cg_graphs) cudaGraphExecDestroy(g.exec);
-    if (F->capture_stream) cudaStreamDestroy(F->capture_stream);
+    cudaFreeHost(F->cg_host);
     delete F;
 }
 
 namespace {
 
-void launch_dot(const Fem& F, const double* x, const double* y, int nv, int slot, int mode, cudaStream_t st)
+// One cooperative launch of the CG on the systems that `a` names (its matrices, right-hand sides,
+// starts, component counts and scratch set). At least 32 rows per CTA: fewer CTAs have fewer
+// partial sums to exchange. The line between the kernels lies where the small one's warps poll two
+// words per lane; it needs rows of at most kCgDeg entries.
+cudaError_t launch_cg(Fem& F, CgArgs& a, cudaStream_t st)
 {
-    const int nb = (int)std::min<unsigned>(Fem::kDotBlocks, blocks(F.ndof, kDotThreads));
-    dot_kernel<<<nb, kDotThreads, 0, st>>>(x, y, F.ndof, nv, F.part + 8 * Fem::kDotBlocks);
-    scalar_kernel<<<1, 32, 0, st>>>(F.part + 8 * Fem::kDotBlocks, nb, nv, slot, mode, F.scal);
-}
-
-// Jacobi-preconditioned CG on nv <= 4 systems with the same matrix A (diagonal `diag`).
-// x holds the start vector, with the fixed values in place on the wall rows when `mask` is set
-// (those rows are not solved for). Converged when ||r_c|| <= tol ||r_c(xref)|| for every c, the
-// residual of the reference start xref (xref = NULL: x itself); tested on the host every
-// kCheckEvery iterations. Five launches per iteration: q = A p with p.q, alpha, the update with
-// r.z and r.r, beta, the new direction. Returns cudaErrorNotReady if not converged.
-cudaError_t pcg(const Fem& F, const double* A, const double* diag, const double* b, double* x, const double* xref,
-                int nv, int mask, double tol, int maxit, int* iters, double* scratch, cudaStream_t st)
-{
-    const size_t n = F.ndof;
-    double* r = scratch;
-    double* z = r + 4 * n;
-    double* p = z + 4 * n;
-    double* q = p + 4 * n;
-    const unsigned g = blocks((int64_t)n);
-    const int nb = (int)std::min<unsigned>(Fem::kDotBlocks, blocks(F.ndof, kDotThreads));
-    double* part_rz = F.part;
-    double* part_rr = F.part + 4 * Fem::kDotBlocks;
-    if (xref) {
-        spmv_kernel<<<g, 256, 0, st>>>(F, A, xref, q, mask, nv);
-        cg_start_kernel<<<g, 256, 0, st>>>(F, b, q, diag, r, z, p, mask, nv);
-        launch_dot(F, r, r, nv, kR0, 0, st);
-    }
-    spmv_kernel<<<g, 256, 0, st>>>(F, A, x, q, mask, nv);
-    cg_start_kernel<<<g, 256, 0, st>>>(F, b, q, diag, r, z, p, mask, nv);
-    if (!xref) launch_dot(F, r, r, nv, kR0, 0, st);
-    launch_dot(F, r, r, nv, kRR, 0, st);
-    launch_dot(F, r, z, nv, kRZ, 0, st);
-    // one CG iteration: five launches (SpMV with the p.q dot, alpha, update with the r.z and r.r
-    // dots, beta, new direction)
-    auto iteration = [&](cudaStream_t s) {
-        spmv_dot_kernel<<<nb, kDotThreads, 0, s>>>(F, A, p, q, mask, nv, F.part);
-        scalar_kernel<<<1, 32, 0, s>>>(F.part, nb, nv, kDot, 1, F.scal);          // alpha = rz / pq
-        update_dot_kernel<<<nb, kDotThreads, 0, s>>>((int)n, nv, F.scal, diag, p, q, x, r, z, part_rz, part_rr);
-        scalar_beta_kernel<<<1, 32, 0, s>>>(part_rz, part_rr, nb, nv, F.scal);    // beta, rz, rr
-        cg_direction_kernel<<<g, 256, 0, s>>>((int)n, nv, F.scal, z, p);
-    };
-    // kCheckEvery iterations between two convergence tests replay one CUDA graph, captured once per
-    // call site (the scalars live on the device, so a replay needs no host work)
-    cudaGraphExec_t exec = nullptr;
-    for (const auto& cg : F.cg_graphs)
-        if (cg.key[0] == A && cg.key[1] == diag && cg.key[2] == x && cg.key[3] == scratch && cg.nv == nv &&
-            cg.mask == mask)
-            exec = cg.exec;
-    if (!exec) {
-        Fem& Fm = const_cast<Fem&>(F);
-        cudaError_t e = cudaSuccess;
-        if (!Fm.capture_stream) e = cudaStreamCreateWithFlags(&Fm.capture_stream, cudaStreamNonBlocking);
-        if (e == cudaSuccess) e = cudaStreamBeginCapture(Fm.capture_stream, cudaStreamCaptureModeThreadLocal);
-        if (e == cudaSuccess) {
-            for (int k = 0; k < kCheckEvery; ++k) iteration(Fm.capture_stream);
-            cudaGraph_t graph = nullptr;
-            e = cudaStreamEndCapture(Fm.capture_stream, &graph);
-            if (e == cudaSuccess) e = cudaGraphInstantiate(&exec, graph, 0);
-            if (graph) cudaGraphDestroy(graph);
-        }
-        if (e != cudaSuccess) return e;
-        Fm.cg_graphs.push_back({{A, diag, x, scratch}, nv, mask, exec});
-    }
-    double r0[4] = {0, 0, 0, 0};
-    int it = 0;
-    bool done = false;
-    for (;;) {
-        if (it % kCheckEvery == 0 || it >= maxit) {
-            cudaError_t e = cudaMemcpyAsync(F.scal_host, F.scal, sizeof(double) * kNScal, cudaMemcpyDeviceToHost, st);
-            if (e == cudaSuccess) e = cudaStreamSynchronize(st);
-            if (e != cudaSuccess) return e;
-            if (it == 0)
-                for (int c = 0; c < nv; ++c) r0[c] = std::sqrt(F.scal_host[kR0 + c]);
-            done = true;
-            for (int c = 0; c < nv; ++c)
-                if (std::sqrt(F.scal_host[kRR + c]) > tol * r0[c]) done = false;
-            if (done || it >= maxit) break;
-        }
-        if (it % kCheckEvery == 0 && it + kCheckEvery <= maxit) {
-            const cudaError_t e = cudaGraphLaunch(exec, st);
-            if (e != cudaSuccess) return e;
-            it += kCheckEvery;
-        } else {
-            iteration(st);
-            ++it;
-        }
-    }
-    *iters = it;
-    cudaError_t e = cudaGetLastError();
+    const int n = F.ndof;
+    a.n = n;
+    a.row = F.row;
+    a.col = F.col;
+    a.wall = F.wall;
+    a.slots = static_cast<ulonglong2*>(F.cg_slots);
+    a.out = F.cg_out;
+    a.epoch = F.cg_epoch;
+    F.cg_epoch += (unsigned long long)a.maxit + 4ull;
+    const cudaError_t e = cudaMemsetAsync(F.cg_out, 0, sizeof(int) * kCgOut, st);
     if (e != cudaSuccess) return e;
-    return done ? cudaSuccess : cudaErrorNotReady;
+    void* args[] = {&a};
+    if (n <= kCgSmallRows && F.max_deg <= kCgDeg)
+        return cudaLaunchCooperativeKernel((const void*)cg_small_kernel, dim3(8 * ((n + 255) / 256) * a.nc), dim3(32),
+                                           args, 0, st);
+    const int G = std::max(1, std::min(F.cg_ctas, (n + 31) / 32));
+    const int rows = (n + G - 1) / G;
+    a.wpc = std::min((kCgMaxThreads / 32 - kCgTasks) / a.nc, (rows + 31) / 32);
+    int slice = 0;
+    for (int b = 0; b < G; ++b)
+        slice = std::max(slice, F.row_host[(int64_t)n * (b + 1) / G] - F.row_host[(int64_t)n * b / G]);
+    const size_t entry = sizeof(int) + sizeof(double) * ((a.nv0 > 0) + (a.nc > a.nv0));
+    const bool one = rows <= 32 * a.wpc, smem = slice * entry <= kCgSmemMax;
+    a.slice = smem ? slice : 0;
+    const void* fn = one ? (smem ? (const void*)cg_kernel<true, true> : (const void*)cg_kernel<true, false>)
+                         : (smem ? (const void*)cg_kernel<false, true> : (const void*)cg_kernel<false, false>);
+    return cudaLaunchCooperativeKernel(fn, dim3(G), dim3(32 * (a.nc * a.wpc + kCgTasks)), args, smem ? slice * entry : 0, st);
 }
 
 }  // namespace
@@ -866,69 +1199,97 @@ cudaError_t node_fields_solve(Fem& F, const double* stats, const lpdf_params& P,
     double* lapU = w;   w += 3 * n;
     double* gp = w;     w += 2 * n;
     double* wp = w;     w += 4 * n;
+    double* p = w;      w += n;
     double* diag = w;   w += n;
-    double* rhs = w;    w += 4 * n;
+    double* rhs = w;    w += 5 * n;       // the relaxation's four, the pressure's
     double* tmp = w;    w += 4 * n;
-    double* cgs = w;    w += 16 * n;      // r, z, p, q of the CG
-    double* xref = w;   w += 4 * n;       // the zero-interior start (reference of the test)
+    double* L2 = w;     w += n;
+    double* cgs = w;    w += 20 * n;      // scratch of the CG
+    double* xref = w;   w += 5 * n;       // the zero-interior start (reference of the test)
     double* wp_prev = w; w += 4 * n;      // previous solutions (warm start)
     double* p_prev = w; w += n;
     double* ew = F.work + Fem::kWorkPerDof * n;   // element scratch, 16 per element
     const unsigned gd = blocks((int64_t)n), ge = blocks(F.E);
     iters[0] = iters[1] = 0;
-    dof_stats_kernel<<<gd, 256, 0, st>>>(F, stats, nq, ns, U, R, om, phi, k, eps);
+    const bool relax = P.gmodel == 0 && !surr, press = P.pressure_solve != 0;
+    dof_stats_kernel<<<gd, 256, 0, st>>>(F, stats, nq, ns, P.CL, P.Ceta * std::pow(P.nu, 0.75), U, R, om, phi, k, eps,
+                                         relax ? L2 : nullptr);
     // recovered gradients of the mean velocity, then their recovered divergences
     elem_grad_kernel<<<ge, 256, 0, st>>>(F, U, 3, 3, ew);
-    recover_kernel<<<gd, 256, 0, st>>>(F, ew, 6, gU, 6);
-    for (int i = 0; i < 3; ++i) {
-        elem_div_kernel<<<ge, 256, 0, st>>>(F, gU + 2 * i, 6, ew);
-        recover_kernel<<<gd, 256, 0, st>>>(F, ew, 1, lapU + i, 3);
-    }
-    if (P.gmodel == 0 && !surr) {
-        elem_L2_kernel<<<ge, 256, 0, st>>>(F, k, eps, P.CL, P.Ceta, P.nu, ew);
+    recover_kernel<<<blocks(6 * (int64_t)n), 256, 0, st>>>(F, ew, 6, gU, 6);
+    elem_div_kernel<<<blocks(3 * (int64_t)F.E), 256, 0, st>>>(F, gU, ew);
+    recover_kernel<<<blocks(3 * (int64_t)n), 256, 0, st>>>(F, ew, 3, lapU, 3);
+    CgArgs a{};
+    a.tol = tol;
+    a.maxit = maxit;
+    a.z = F.cg_z;
+    a.state = cgs;
+    if (relax) {
+        elem_L2_kernel<<<ge, 256, 0, st>>>(F, L2, ew);
         assemble_kernel<<<gd, 256, 0, st>>>(F, ew, F.Aval, diag);
         const bool warm = P.cg_warm_start && F.has_wp;
         er_setup_kernel<<<gd, 256, 0, st>>>(F, eps, P.C0, tmp, wp, warm ? wp_prev : nullptr, xref);
         spmv_kernel<<<gd, 256, 0, st>>>(F, F.Mval, tmp, rhs, 0, 4);     // b = M wp^h
-        cudaError_t e = pcg(F, F.Aval, diag, rhs, wp, xref, 4, 1, tol, maxit, &iters[0], cgs, st);
-        if (e != cudaSuccess) return e;
-        e = cudaMemcpyAsync(wp_prev, wp, sizeof(double) * 4 * n, cudaMemcpyDeviceToDevice, st);
-        if (e != cudaSuccess) return e;
-        F.has_wp = true;
+        a.A0 = F.Aval;
+        a.d0 = diag;
+        a.b0 = rhs;
+        a.x0 = wp;
+        a.ref0 = xref;
+        a.mask0 = 1;
+        a.nv0 = 4;
     }
-    if (P.pressure_solve) {
+    a.nc = a.nv0;
+    if (press) {
         pressure_T_kernel<<<gd, 256, 0, st>>>(F, U, R, tmp);
         elem_grad_kernel<<<ge, 256, 0, st>>>(F, tmp, 4, 4, ew);
-        pressure_rhs_kernel<<<gd, 256, 0, st>>>(F, ew, rhs);
-        diag_kernel<<<gd, 256, 0, st>>>(F, F.Kval, diag);
-        double* p = tmp;
-        const bool warm = P.cg_warm_start && F.has_p;
-        if (warm) {
-            cudaError_t e = cudaMemcpyAsync(p, p_prev, sizeof(double) * n, cudaMemcpyDeviceToDevice, st);
-            if (e != cudaSuccess) return e;
-        } else {
-            fill_kernel<<<gd, 256, 0, st>>>((int)n, 0.0, p);
-        }
+        pressure_rhs_kernel<<<gd, 256, 0, st>>>(F, ew, rhs + 4 * n);
         // consistent singular system (the right-hand side sums to zero): CG stays in the range up
         // to rounding; the constant is removed afterwards. Reference start: zero.
-        fill_kernel<<<gd, 256, 0, st>>>((int)n, 0.0, xref);
-        cudaError_t e = pcg(F, F.Kval, diag, rhs, p, warm ? xref : nullptr, 1, 0, tol, maxit, &iters[1], cgs, st);
+        const bool warm = P.cg_warm_start && F.has_p;
+        cudaError_t e = warm ? cudaMemcpyAsync(p, p_prev, sizeof(double) * n, cudaMemcpyDeviceToDevice, st)
+                             : cudaMemsetAsync(p, 0, sizeof(double) * n, st);
+        if (e == cudaSuccess && warm) e = cudaMemsetAsync(xref + 4 * n, 0, sizeof(double) * n, st);
         if (e != cudaSuccess) return e;
-        double* ones = rhs + n;
-        fill_kernel<<<gd, 256, 0, st>>>((int)n, 1.0, ones);
-        launch_dot(F, p, ones, 1, kDot, 0, st);
-        subtract_mean_kernel<<<gd, 256, 0, st>>>((int)n, F.scal + kDot, p);
-        e = cudaMemcpyAsync(p_prev, p, sizeof(double) * n, cudaMemcpyDeviceToDevice, st);
+        a.A1 = F.Kval;
+        a.d1 = F.Kdiag;
+        a.b1 = rhs + 4 * n;
+        a.x1 = p;
+        a.ref1 = warm ? xref + 4 * n : nullptr;
+        ++a.nc;
+    }
+    if (a.nc > 0) {
+        const cudaError_t e = launch_cg(F, a, st);
         if (e != cudaSuccess) return e;
-        F.has_p = true;
+    }
+    if (press) {
+        const int nb = (int)std::min<unsigned>(Fem::kDotBlocks, blocks((int64_t)n, kDotThreads));   // fixed order
+        sum_kernel<<<nb, kDotThreads, 0, st>>>(p, (int)n, F.part);
+        subtract_mean_kernel<<<gd, 256, 0, st>>>((int)n, F.part, nb, p);
         elem_grad_kernel<<<ge, 256, 0, st>>>(F, p, 1, 1, ew);
-        recover_kernel<<<gd, 256, 0, st>>>(F, ew, 2, gp, 2);
+        recover_kernel<<<blocks(2 * (int64_t)n), 256, 0, st>>>(F, ew, 2, gp, 2);
     } else {
-        fill_kernel<<<blocks(2 * (int64_t)n), 256, 0, st>>>(2 * (int)n, 0.0, gp);
+        const cudaError_t e = cudaMemsetAsync(gp, 0, sizeof(double) * 2 * n, st);
+        if (e != cudaSuccess) return e;
     }
     fields_kernel<<<blocks(F.N), 256, 0, st>>>(F, ns, nfp, U, R, om, phi, k, eps, gU, lapU, gp, wp, P.gmodel, P.C0,
-                                               P.Comega1, P.Comega2, P.dpdx0, P.dpdy0, surr, surr_norm, out);
-    return cudaGetLastError();
+                                               P.Comega1, P.Comega2, P.dpdx0, P.dpdy0, surr, surr_norm,
+                                               a.nc > 0 ? F.cg_out : nullptr, relax + press, out);
+    if (a.nc == 0) return cudaGetLastError();
+    // everything is enqueued: the one synchronisation reads how the CGs ended
+    const int n4 = relax ? 4 * (int)n : 0, n1 = press ? (int)n : 0;
+    keep_solution_kernel<<<blocks(std::max(n4, n1)), 256, 0, st>>>(F.cg_out, relax + press, n4, wp, wp_prev, n1, p, p_prev);
+    cudaError_t e = cudaGetLastError();
+    if (e == cudaSuccess)
+        e = cudaMemcpyAsync(F.cg_host, F.cg_out, sizeof(int) * kCgOut, cudaMemcpyDeviceToHost, st);
+    if (e == cudaSuccess) e = cudaStreamSynchronize(st);
+    if (e != cudaSuccess) return e;
+    if (F.cg_host[kCgError]) return cudaErrorLaunchTimeout;   // a bounded wait of the CG kernel gave up
+    iters[0] = F.cg_host[kCgIts0];
+    iters[1] = F.cg_host[kCgIts1];
+    if (F.cg_host[kCgOk] != relax + press) return cudaErrorNotReady;
+    F.has_wp = F.has_wp || relax;
+    F.has_p = F.has_p || press;
+    return cudaSuccess;
 }
 
 cudaError_t surrogate_features(Fem& F, const double* stats, int ns, const float* fields, double C0, float* feat,
