@@ -400,11 +400,12 @@ int build_mesh(const double* node_xy, int32_t n_nodes, const int32_t* tri, int32
     m->box[0] = x0; m->box[1] = x1; m->box[2] = y0; m->box[3] = y1;
     std::vector<float> ew(16 * (size_t)n_tri, 0.0f);
     for (int e = 0; e < n_tri; ++e) {
-        for (int q = 0; q < 4; ++q) {
-            ew[16 * (size_t)e + q] = ea[4 * (size_t)e + q];
-            ew[16 * (size_t)e + 4 + q] = eb[4 * (size_t)e + q];
-            std::memcpy(&ew[16 * (size_t)e + 8 + q], &en[4 * (size_t)e + q], sizeof(float));
-        }
+        float* w = &ew[16 * (size_t)e];
+        for (int q = 0; q < 4; ++q) w[q] = ea[4 * (size_t)e + q];
+        w[4] = eb[4 * (size_t)e];
+        w[5] = eb[4 * (size_t)e + 1];
+        for (int q = 0; q < 3; ++q) std::memcpy(w + 6 + q, &en[4 * (size_t)e + (q + 1) % 3], sizeof(float));
+        w[9] = eb[4 * (size_t)e + 2];
     }
     cudaError_t ce = cudaSuccess;
     if ((ce = dalloc(&d.ex, n_tri)) != cudaSuccess || (ce = dalloc(&d.ey, n_tri)) != cudaSuccess ||

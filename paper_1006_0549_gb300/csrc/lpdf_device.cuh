@@ -325,41 +325,38 @@ static __device__ __noinline__ int fast_wall_exit(float l0, float l1, float l2, 
 // domain can lie beyond the line of some wall edge, never beyond every negative edge's line.
 // Bound: with u = 2^-24, dx = fl(px - x_v0) (x_v0 exact in FP32) and the coefficients rounded
 // from FP64, |lambda_a' - lambda_a| <= 4.01 u (|b_a dx| + |g_a dy|) for a = 1, 2, and for
-// lambda_0 = 1 - lambda_1 - lambda_2 that sum plus 2 u (1 + |lambda_1| + |lambda_2|); the
-// constants below carry a margin for the rounding of the bounds themselves.
+// lambda_0 = 1 - lambda_1 - lambda_2 that sum plus 2 u (1 + |lambda_1| + |lambda_2|). One bound serves
+// all three: with T the sum of the four |b_a dx|, |g_a dy| (|lambda_1| + |lambda_2| <= T within its
+// rounding), 6.01 u T + 2 u covers each; the constants carry a margin for the rounding of the bound
+// itself. A hop is about half instructions and half L1 traffic: three separate bounds and the
+// bookkeeping of the smallest weight were 15 instructions more, and the record (coefficients, the
+// neighbours in the order of the opposite vertices, the centroid) is 40 bytes.
 template <bool kWalls = false>
 __device__ __forceinline__ int walk_test_fast(const DevMesh& M, int e, float px, float py, int& next)
 {
     const float4* W = M.ew + 4 * (size_t)e;
     const float4 A = __ldg(W);
     const float4 B = __ldg(W + 1);
-    const int4 N = __ldg(reinterpret_cast<const int4*>(W + 2));
-    if (M.periodic && fabsf(B.z - px) > 0.5f * M.period) return -1;
+    const float2 C = __ldg(reinterpret_cast<const float2*>(W + 2));   // neighbour opposite vertex 2, centroid x
+    if (M.periodic && fabsf(C.y - px) > 0.5f * M.period) return -1;
     const float dx = __fsub_rn(px, A.x), dy = __fsub_rn(py, A.y);
     const float t1 = A.z * dx, s1 = A.w * dy, t2 = B.x * dx, s2 = B.y * dy;
     const float l1 = t1 + s1, l2 = t2 + s2;
     const float l0 = (1.0f - l1) - l2;
-    const float E1 = 3.0e-7f * (fabsf(t1) + fabsf(s1)) + 1e-30f;
-    const float E2 = 3.0e-7f * (fabsf(t2) + fabsf(s2)) + 1e-30f;
-    const float E0 = E1 + E2 + 1.5e-7f * (1.0f + fabsf(l1) + fabsf(l2));
-    if (l0 > E0 && l1 > E1 && l2 > E2) return 1;
-    // the most negative lambda, lowest index on ties; vertex a is opposite edge (a + 1) % 3
-    // (edge k runs from vertex k to vertex k + 1)
-    int a = 0;
-    float lm = l0;
-    if (l1 < lm) { a = 1; lm = l1; }
-    if (l2 < lm) { a = 2; lm = l2; }
-    const float Ea = a == 0 ? E0 : (a == 1 ? E1 : E2);
-    if (!(lm < -Ea)) return -1;
-    next = a == 0 ? N.y : (a == 1 ? N.z : N.x);
-    if (next >= 0) return 0;
-    if (kWalls) {
-        const int c = fast_wall_exit(l0, l1, l2, E0, E1, E2, N, a);
+    const float E = fmaf(4.6e-7f, (fabsf(t1) + fabsf(s1)) + (fabsf(t2) + fabsf(s2)), 1.55e-7f);
+    const float lm = fminf(fminf(l0, l1), l2);
+    if (lm > E) return 1;
+    if (!(lm < -E)) return -1;
+    // the most negative lambda, lowest index on ties
+    next = __float_as_int(l0 == lm ? B.z : (l1 == lm ? B.w : C.x));
+    if (kWalls && next < 0) {
+        // vertex a is opposite edge (a + 1) % 3 (edge k runs from vertex k to vertex k + 1)
+        const int a = l0 == lm ? 0 : (l1 == lm ? 1 : 2);
+        const int4 N = make_int4(__float_as_int(C.x), __float_as_int(B.z), __float_as_int(B.w), 0);
+        const int c = fast_wall_exit(l0, l1, l2, E, E, E, N, a);
         if (c == kWalkUndecided) return -1;
         next = c;
-        return 0;
     }
-    next = -1 - (a == 2 ? 0 : a + 1);   // a wall: -1 - (the exit edge)
     return 0;
 }
 
