@@ -18,7 +18,8 @@
  *     the library owns the objects it creates (lpdf_mesh, lpdf_ctx) and their device memory.
  *   - `stream` is a cudaStream_t passed as void* (NULL = legacy default stream). Calls marked
  *     "async" only enqueue work on that stream; calls marked "sync" return after the work ends.
- *   - Floating-point particle state is FP32 structure-of-arrays; gridpoint moment sums are FP64.
+ *   - Floating-point particle state is FP32, one array per field at the interface; gridpoint moment sums
+ *     are FP64.
  */
 #ifndef LPDF_H
 #define LPDF_H
@@ -166,7 +167,8 @@ int lpdf_mesh_load_multi(const double* node_xy, int32_t n_nodes, const int32_t* 
 
 /* ---------------------------------------------------------------------------------------
  * lpdf_ctx_create -- particle ensemble on one mesh with room for `capacity` particles
- * (device SoA state x, y, u, v, w, omega, psi[ns], elem, pid, plus the moment accumulators).
+ * (device state x, y, u, v, w, omega, psi[ns], elem, pid, in the library's own layout, plus the moment
+ * accumulators).
  * params->ns must be in 1..LPDF_MAX_SCALARS. sync. The mesh must outlive the context.
  * ------------------------------------------------------------------------------------- */
 int lpdf_ctx_create(const lpdf_mesh* mesh, const lpdf_params* params, int64_t capacity, lpdf_ctx** out);
@@ -204,7 +206,7 @@ int lpdf_particles_init(lpdf_ctx* ctx, int32_t n_per_elem, const float* node_ini
                         void* stream);
 
 /* ---------------------------------------------------------------------------------------
- * lpdf_set_state / lpdf_get_state -- copy the SoA state in or out. `on_device` = 1: the
+ * lpdf_set_state / lpdf_get_state -- copy the state in or out of the caller's arrays, one per field. `on_device` = 1: the
  * pointers are device memory, 0: host memory. psi is ns rows of n values. set_state sets the
  * ensemble size to n (n <= capacity). async (a host copy is synchronous w.r.t. the host only
  * when the host memory is pageable).

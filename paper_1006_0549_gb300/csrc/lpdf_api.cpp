@@ -506,21 +506,18 @@ int lpdf_ctx_create(const lpdf_mesh* mesh, const lpdf_params* params, int64_t ca
     c->mesh = mesh;
     c->params = *params;
     c->ns = params->ns;
-    DevState& s = c->s;
+    Particles& s = c->s;
     s.n = 0;
     s.cap = cap;
     const int nq = nquant(c->ns);
     cudaError_t ce = cudaSuccess;
-    DevState& s2 = c->s2;
+    Particles& s2 = c->s2;
     s2.n = 0;
     s2.cap = cap;
     const size_t E = (size_t)mesh->d.n_tri;
-    if ((ce = dalloc(&s.x, cap)) || (ce = dalloc(&s.y, cap)) || (ce = dalloc(&s.u, cap)) || (ce = dalloc(&s.v, cap)) ||
-        (ce = dalloc(&s.w, cap)) || (ce = dalloc(&s.om, cap)) || (ce = dalloc(&s.psi, cap * c->ns)) ||
-        (ce = dalloc(&s.elem, cap)) || (ce = dalloc(&s.pid, cap)) ||
-        (ce = dalloc(&s2.x, cap)) || (ce = dalloc(&s2.y, cap)) || (ce = dalloc(&s2.u, cap)) || (ce = dalloc(&s2.v, cap)) ||
-        (ce = dalloc(&s2.w, cap)) || (ce = dalloc(&s2.om, cap)) || (ce = dalloc(&s2.psi, cap * c->ns)) ||
-        (ce = dalloc(&s2.elem, cap)) || (ce = dalloc(&s2.pid, cap)) ||
+    const size_t rest = (size_t)cap * rest_words(c->ns);
+    if ((ce = dalloc(&s.rec, 8 * cap)) || (ce = dalloc(&s.elem, cap)) || (rest && (ce = dalloc(&s.rest, rest))) ||
+        (ce = dalloc(&s2.rec, 8 * cap)) || (ce = dalloc(&s2.elem, cap)) || (rest && (ce = dalloc(&s2.rest, rest))) ||
         (ce = dalloc(&c->sort.cnt, E + 1)) || (ce = dalloc(&c->sort.cursor, E + 1)) ||
         (ce = dalloc(&c->sort.start, E + 2)) || (ce = dalloc(&c->sort.perm, cap)) ||
         (ce = dalloc(&c->node_acc, (size_t)mesh->d.n_nodes * nq)) || (ce = dalloc(&c->status, 4)) ||
@@ -552,9 +549,10 @@ int lpdf_ctx_create(const lpdf_mesh* mesh, const lpdf_params* params, int64_t ca
 void lpdf_ctx_free(lpdf_ctx* c)
 {
     if (!c) return;
-    for (DevState* s : {&c->s, &c->s2}) {
-        cudaFree(s->x); cudaFree(s->y); cudaFree(s->u); cudaFree(s->v); cudaFree(s->w); cudaFree(s->om);
-        cudaFree(s->psi); cudaFree(s->elem); cudaFree(s->pid);
+    for (Particles* s : {&c->s, &c->s2}) {
+        cudaFree(s->rec);
+        cudaFree(s->rest);
+        cudaFree(s->elem);
     }
     cudaFree(c->sort.cnt); cudaFree(c->sort.cursor); cudaFree(c->sort.start); cudaFree(c->sort.perm);
     for (auto& q : c->ev_pending)
@@ -670,26 +668,43 @@ int lpdf_particles_init_multi(lpdf_ctx* c, const int32_t* n_per_elem, const floa
                      (cudaStream_t)stream);
 }
 
-static int copy_state(lpdf_ctx* c, int64_t n, bool in, float* x, float* y, float* u, float* v, float* w, float* om,
-                      float* psi, int32_t* elem, uint32_t* pid, int on_device, cudaStream_t st)
+// The user's arrays into the records or back. Device arrays: one kernel. Host arrays: by way of a
+// stream-ordered staging buffer of at most kStage particles at a time (given back at the end).
+static int copy_state(lpdf_ctx* c, int64_t n, bool in, const UserArrays& user, int on_device, cudaStream_t st)
 {
-    const cudaMemcpyKind k = on_device ? cudaMemcpyDeviceToDevice : (in ? cudaMemcpyHostToDevice : cudaMemcpyDeviceToHost);
-    DevState& s = c->s;
-    struct Item { void* dev; void* usr; size_t bytes; };
-    const size_t fb = sizeof(float) * (size_t)n;
-    Item items[] = {{s.x, x, fb}, {s.y, y, fb}, {s.u, u, fb}, {s.v, v, fb}, {s.w, w, fb}, {s.om, om, fb},
-                    {s.elem, elem, sizeof(int32_t) * (size_t)n}, {s.pid, pid, sizeof(uint32_t) * (size_t)n}};
     if (n == 0) return LPDF_OK;
-    for (auto& it : items) {
-        if (!it.usr) continue;
-        CUDA_TRY(in ? cudaMemcpyAsync(it.dev, it.usr, it.bytes, k, st) : cudaMemcpyAsync(it.usr, it.dev, it.bytes, k, st));
+    const int ns = c->ns;
+    if (on_device) {
+        CUDA_TRY(in ? launch_pack_state(c->s, 0, n, ns, user, st) : launch_unpack_state(c->s, 0, n, ns, user, st));
+        return LPDF_OK;
     }
-    if (psi)
-        for (int a = 0; a < c->ns; ++a) {
-            float* dev = s.psi + (size_t)a * s.cap;
-            float* usr = psi + (size_t)a * n;
-            CUDA_TRY(in ? cudaMemcpyAsync(dev, usr, fb, k, st) : cudaMemcpyAsync(usr, dev, fb, k, st));
+    constexpr int64_t kStage = 1 << 22;
+    const int64_t m = std::min(n, kStage);
+    const int rows = 8 + ns;
+    float* stage = nullptr;
+    CUDA_TRY(cudaMallocAsync((void**)&stage, sizeof(float) * (size_t)m * rows, st));
+    // the staging rows x, y, u, v, w, omega, elem, pid, psi_0, ...; a row the caller left out is skipped
+    const UserArrays dev{stage, stage + m, stage + 2 * m, stage + 3 * m, stage + 4 * m, stage + 5 * m, stage + 8 * m,
+                         reinterpret_cast<int*>(stage + 6 * m), reinterpret_cast<uint32_t*>(stage + 7 * m), m};
+    char* host[8] = {(char*)user.x, (char*)user.y, (char*)user.u, (char*)user.v, (char*)user.w, (char*)user.om,
+                     (char*)user.elem, (char*)user.pid};
+    cudaError_t e = cudaSuccess;
+    for (int64_t i0 = 0; i0 < n && e == cudaSuccess; i0 += m) {
+        const int64_t k = std::min(m, n - i0);
+        if (!in) e = launch_unpack_state(c->s, i0, k, ns, dev, st);
+        for (int r = 0; r < rows && e == cudaSuccess; ++r) {
+            char* h = r < 8 ? host[r] : (user.psi ? (char*)(user.psi + (int64_t)(r - 8) * n) : nullptr);
+            if (!h) continue;
+            h += sizeof(float) * (size_t)i0;
+            float* d = stage + r * m;
+            e = in ? cudaMemcpyAsync(d, h, sizeof(float) * (size_t)k, cudaMemcpyHostToDevice, st)
+                   : cudaMemcpyAsync(h, d, sizeof(float) * (size_t)k, cudaMemcpyDeviceToHost, st);
         }
+        if (in && e == cudaSuccess) e = launch_pack_state(c->s, i0, k, ns, dev, st);
+    }
+    const cudaError_t f = cudaFreeAsync(stage, st);
+    CUDA_TRY(e);
+    CUDA_TRY(f);
     return LPDF_OK;
 }
 
@@ -703,8 +718,9 @@ int lpdf_set_state(lpdf_ctx* c, int64_t n, const float* x, const float* y, const
     if (n > 0 && (!x || !y || !u || !v || !w || !om || !psi || !elem || !pid))
         return fail(LPDF_ERR_ARG, "set_state needs every array");
     c->s.n = n;
-    const int rc = copy_state(c, n, true, (float*)x, (float*)y, (float*)u, (float*)v, (float*)w, (float*)om,
-                              (float*)psi, (int32_t*)elem, (uint32_t*)pid, on_device, (cudaStream_t)stream);
+    const UserArrays user{(float*)x, (float*)y, (float*)u, (float*)v, (float*)w, (float*)om, (float*)psi, (int*)elem,
+                          (uint32_t*)pid, n};
+    const int rc = copy_state(c, n, true, user, on_device, (cudaStream_t)stream);
     if (rc) return rc;
     // any order is valid input; the first step brings the ensemble into element order
     CUDA_TRY(launch_iota(c->pipe.perm, n, (cudaStream_t)stream));
@@ -715,8 +731,8 @@ int lpdf_get_state(const lpdf_ctx* c, float* x, float* y, float* u, float* v, fl
                    int32_t* elem, uint32_t* pid, int on_device, void* stream)
 {
     if (!c) return fail(LPDF_ERR_ARG, "ctx is NULL");
-    return copy_state(const_cast<lpdf_ctx*>(c), c->s.n, false, x, y, u, v, w, om, psi, elem, pid, on_device,
-                      (cudaStream_t)stream);
+    const UserArrays user{x, y, u, v, w, om, psi, elem, pid, c->s.n};
+    return copy_state(const_cast<lpdf_ctx*>(c), c->s.n, false, user, on_device, (cudaStream_t)stream);
 }
 
 int lpdf_sort(lpdf_ctx* c, void* stream)
@@ -772,7 +788,7 @@ static int capture_steps(lpdf_ctx* c, const float* fields, int slot)
     (void)sm_count();   // device queries stay outside the capture
     CUDA_TRY(cudaStreamBeginCapture(cs, cudaStreamCaptureModeThreadLocal));
     const int nq = nquant(c->ns);
-    DevState a = c->s, b = c->s2;
+    Particles a = c->s, b = c->s2;
     PipeScratch w = c->pipe;
     cudaError_t e = cudaSuccess;
     for (int k = 0; k < 2 && e == cudaSuccess; ++k) {
@@ -802,7 +818,7 @@ static int capture_steps(lpdf_ctx* c, const float* fields, int slot)
         return fail(LPDF_ERR_CUDA, "pdf_steps: graph capture: %s", cudaGetErrorString(e));
     }
     c->graph_fields[slot] = fields;
-    c->graph_state[slot] = c->s.x;
+    c->graph_state[slot] = c->s.rec;
     c->graph_perm[slot] = c->pipe.perm;
     return LPDF_OK;
 }
@@ -816,7 +832,7 @@ int lpdf_pdf_steps(lpdf_ctx* c, const float* node_fields, uint64_t step0, int32_
     if (pairs > 0 && c->s.n > 0) {
         int slot = -1;
         for (int k = 0; k < 2; ++k)
-            if (c->graph[k] && c->graph_fields[k] == node_fields && c->graph_state[k] == c->s.x &&
+            if (c->graph[k] && c->graph_fields[k] == node_fields && c->graph_state[k] == c->s.rec &&
                 c->graph_perm[k] == c->pipe.perm)
                 slot = k;
         if (slot < 0) {

@@ -534,6 +534,47 @@ struct ParticleState {
     uint32_t pid;
 };
 
+// one record, 32 bytes in one instruction: read once and not kept in L1; read and kept; written through
+__device__ __forceinline__ void rec_load_stream(const float* p, float (&r)[8])
+{
+    asm("ld.global.nc.L1::no_allocate.v8.f32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];"
+        : "=f"(r[0]), "=f"(r[1]), "=f"(r[2]), "=f"(r[3]), "=f"(r[4]), "=f"(r[5]), "=f"(r[6]), "=f"(r[7])
+        : "l"(p));
+}
+__device__ __forceinline__ void rec_store_stream(float* p, const float (&r)[8])
+{
+    asm volatile("st.global.cs.v8.f32 [%0], {%1, %2, %3, %4, %5, %6, %7, %8};" ::"l"(p), "f"(r[0]), "f"(r[1]), "f"(r[2]),
+                 "f"(r[3]), "f"(r[4]), "f"(r[5]), "f"(r[6]), "f"(r[7])
+                 : "memory");
+}
+
+// the scalars from psi_1 on
+template <int NS>
+__device__ __forceinline__ void rest_load(const float* rest, int64_t j, float* psi)
+{
+    if (NS == 2) psi[1] = __ldcs(rest + j);
+    if (NS == 3) {
+        const float2 v = __ldcs(reinterpret_cast<const float2*>(rest) + j);
+        psi[1] = v.x;
+        psi[NS > 2 ? 2 : 0] = v.y;
+    }
+    if (NS == 4) {
+        const float4 v = __ldcs(reinterpret_cast<const float4*>(rest) + j);
+        psi[NS > 1 ? 1 : 0] = v.x;
+        psi[NS > 2 ? 2 : 0] = v.y;
+        psi[NS > 3 ? 3 : 0] = v.z;
+    }
+}
+template <int NS>
+__device__ __forceinline__ void rest_store(float* rest, int64_t j, const float* psi)
+{
+    if (NS == 2) __stcs(rest + j, psi[1]);
+    if (NS == 3) __stcs(reinterpret_cast<float2*>(rest) + j, make_float2(psi[1], psi[NS > 2 ? 2 : 0]));
+    if (NS == 4)
+        __stcs(reinterpret_cast<float4*>(rest) + j,
+               make_float4(psi[NS > 1 ? 1 : 0], psi[NS > 2 ? 2 : 0], psi[NS > 3 ? 3 : 0], 0.0f));
+}
+
 __device__ __forceinline__ bool in_source(float px, float py, float sx, float sy, float r)
 {
     const float dx = __fsub_rn(px, sx), dy = __fsub_rn(py, sy);

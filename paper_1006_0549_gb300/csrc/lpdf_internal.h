@@ -89,6 +89,19 @@ struct DevState {
     int64_t n, cap;
 };
 
+// A context's particles: a 32-byte record each (x, y, u, v, w, omega, psi_0, pid as bits), one sector of
+// memory, so that a gather in element order moves no byte that it does not use, however the wanted
+// records are spread (as separate arrays the 32 values of a warp's gather lay in 10-25 sectors, eight
+// arrays over); the element, which the re-bucketing streams, is an array of its own, and so are the
+// scalars from psi_1 on (rest_words(ns) words a particle).
+struct Particles {
+    float* rec;
+    float* rest;
+    int* elem;
+    int64_t n, cap;
+};
+__host__ __device__ constexpr int rest_words(int ns) { return ns <= 3 ? ns - 1 : 4; }   // ns = 4: a float4, one unused
+
 // Status words (device): [0] error bits, [1] lost count, [2] one lost pid, [3] total hops
 enum : unsigned { kErrLost = 1u, kErrNonFinite = 2u, kErrOverflow = 4u, kErrTimeout = 8u, kErrCheck = 16u };
 
@@ -105,8 +118,18 @@ struct InitLayout {
     const uint32_t* key;
     int n_comp;
 };
-cudaError_t launch_particles_init(const DevMesh& m, const DevState& s, int ns, const InitLayout& L, int64_t P,
+cudaError_t launch_particles_init(const DevMesh& m, const Particles& s, int ns, const InitLayout& L, int64_t P,
                                   const float* node_init, int m_erlang, unsigned long long* status, cudaStream_t st);
+// user arrays (device; ns rows of `ld` values for psi) -> particles [i0, i0 + n) and back (a NULL array
+// is skipped)
+struct UserArrays {
+    float *x, *y, *u, *v, *w, *om, *psi;
+    int* elem;
+    uint32_t* pid;
+    int64_t ld;
+};
+cudaError_t launch_pack_state(const Particles& s, int64_t i0, int64_t n, int ns, const UserArrays& a, cudaStream_t st);
+cudaError_t launch_unpack_state(const Particles& s, int64_t i0, int64_t n, int ns, const UserArrays& a, cudaStream_t st);
 cudaError_t launch_grid_statistics(const DevMesh& m, int ns, const unsigned long long* node_acc, double* out,
                                    int raw, cudaStream_t st);
 
@@ -117,7 +140,7 @@ struct SortScratch {
     int* start = nullptr;
     int* perm = nullptr;
 };
-cudaError_t launch_sort(const DevMesh& m, const DevState& s, int ns, const DevState& dst, SortScratch& w,
+cudaError_t launch_sort(const DevMesh& m, const Particles& s, int ns, const Particles& dst, SortScratch& w,
                         unsigned long long* status, cudaStream_t st);
 
 // scratch of the step pipeline (lpdf_pipeline.cu)
@@ -148,7 +171,7 @@ struct StepTune {
     int adv = 0, mom = 0;
 };
 constexpr int kAdvVariants = 6, kMomVariants = 4;
-cudaError_t launch_pdf_step_pipeline(const DevMesh& m, const DevState& cur, const DevState& nxt, int ns,
+cudaError_t launch_pdf_step_pipeline(const DevMesh& m, const Particles& cur, const Particles& nxt, int ns,
                                      const float* fields, const StepParams& p, PipeScratch& w,
                                      unsigned long long* node_acc, unsigned long long* status, cudaStream_t st,
                                      const cudaEvent_t* ev, const StepTune& tune,
@@ -299,8 +322,8 @@ struct lpdf_mesh {
 struct lpdf_ctx {
     const lpdf_mesh* mesh;
     lpdf_params params;
-    lpdf::DevState s;                         // current particle state
-    lpdf::DevState s2;                        // second buffer (written by the step and the re-bucketing)
+    lpdf::Particles s;                        // current particle state
+    lpdf::Particles s2;                        // second buffer (written by the step and the re-bucketing)
     lpdf::SortScratch sort;
     lpdf::PipeScratch pipe;
     unsigned long long* node_acc = nullptr;   // n_nodes x nq fixed-point sums

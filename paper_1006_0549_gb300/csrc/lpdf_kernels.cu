@@ -12,7 +12,7 @@ namespace lpdf {
 // element of its element range, with ids counted from 0 and its own Philox key.
 // ------------------------------------------------------------------------------------------
 template <int NS>
-__global__ void particles_init_kernel(const __grid_constant__ DevMesh M, const __grid_constant__ DevState S,
+__global__ void particles_init_kernel(const __grid_constant__ DevMesh M, const __grid_constant__ Particles S,
                                       const __grid_constant__ InitLayout L, const float* __restrict__ init,
                                       int m_erlang, unsigned long long* status)
 {
@@ -68,20 +68,17 @@ __global__ void particles_init_kernel(const __grid_constant__ DevMesh M, const _
         const uint32_t ew[6] = {b.z, b.w, c.x, c.y, c.z, c.w};
         float sum = 0.0f;
         for (int k = 0; k < m_erlang; ++k) sum += -logf(u01(ew[k]));
-        S.x[i] = px; S.y[i] = py;
-        S.u[i] = Fi[0] + Fi[3] * z0;
-        S.v[i] = Fi[1] + Fi[3] * z1;
-        S.w[i] = Fi[2] + Fi[3] * z2;
-        S.om[i] = Fi[4] * sum / (float)m_erlang;
-#pragma unroll
-        for (int q = 0; q < NS; ++q) S.psi[(size_t)q * S.cap + i] = 0.0f;
+        const float r[8] = {px, py, Fi[0] + Fi[3] * z0, Fi[1] + Fi[3] * z1, Fi[2] + Fi[3] * z2,
+                            Fi[4] * sum / (float)m_erlang, 0.0f, __uint_as_float(pid)};
+        rec_store_stream(S.rec + 8 * i, r);
+        const float psi[NS] = {};
+        rest_store<NS>(S.rest, i, psi);
         S.elem[i] = ne;
-        S.pid[i] = pid;
     }
     if (err) atomicOr(&status[0], (unsigned long long)err);
 }
 
-cudaError_t launch_particles_init(const DevMesh& m, const DevState& s, int ns, const InitLayout& L, int64_t P,
+cudaError_t launch_particles_init(const DevMesh& m, const Particles& s, int ns, const InitLayout& L, int64_t P,
                                   const float* node_init, int m_erlang, unsigned long long* status, cudaStream_t st)
 {
     const unsigned grid = (unsigned)((P + 255) / 256);
@@ -92,6 +89,70 @@ cudaError_t launch_particles_init(const DevMesh& m, const DevState& s, int ns, c
         case 3: particles_init_kernel<3><<<grid, 256, 0, st>>>(m, s, L, node_init, m_erlang, status); break;
         case 4: particles_init_kernel<4><<<grid, 256, 0, st>>>(m, s, L, node_init, m_erlang, status); break;
         default: return cudaErrorInvalidValue;
+    }
+    return cudaGetLastError();
+}
+
+// ------------------------------------------------------------------------------------------
+// The user's arrays and the records: particle i0 + i and entry i of the arrays
+// ------------------------------------------------------------------------------------------
+template <int NS>
+__global__ void pack_state_kernel(const __grid_constant__ Particles S, int64_t i0, int64_t n, const __grid_constant__ UserArrays A)
+{
+    const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    if (i >= n) return;
+    float psi[NS];
+#pragma unroll
+    for (int a = 0; a < NS; ++a) psi[a] = A.psi[a * A.ld + i];
+    const float r[8] = {A.x[i], A.y[i], A.u[i], A.v[i], A.w[i], A.om[i], psi[0], __uint_as_float(A.pid[i])};
+    rec_store_stream(S.rec + 8 * (i0 + i), r);
+    rest_store<NS>(S.rest, i0 + i, psi);
+    S.elem[i0 + i] = A.elem[i];
+}
+
+template <int NS>
+__global__ void unpack_state_kernel(const __grid_constant__ Particles S, int64_t i0, int64_t n,
+                                    const __grid_constant__ UserArrays A)
+{
+    const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    if (i >= n) return;
+    float r[8], psi[NS];
+    rec_load_stream(S.rec + 8 * (i0 + i), r);
+    psi[0] = r[6];
+    rest_load<NS>(S.rest, i0 + i, psi);
+    float* const out[6] = {A.x, A.y, A.u, A.v, A.w, A.om};
+#pragma unroll
+    for (int k = 0; k < 6; ++k)
+        if (out[k]) out[k][i] = r[k];
+    if (A.psi)
+#pragma unroll
+        for (int a = 0; a < NS; ++a) A.psi[a * A.ld + i] = psi[a];
+    if (A.elem) A.elem[i] = S.elem[i0 + i];
+    if (A.pid) A.pid[i] = __float_as_uint(r[7]);
+}
+
+cudaError_t launch_pack_state(const Particles& s, int64_t i0, int64_t n, int ns, const UserArrays& a, cudaStream_t st)
+{
+    if (n == 0) return cudaSuccess;
+    const unsigned g = (unsigned)((n + 255) / 256);
+    switch (ns) {
+        case 1: pack_state_kernel<1><<<g, 256, 0, st>>>(s, i0, n, a); break;
+        case 2: pack_state_kernel<2><<<g, 256, 0, st>>>(s, i0, n, a); break;
+        case 3: pack_state_kernel<3><<<g, 256, 0, st>>>(s, i0, n, a); break;
+        default: pack_state_kernel<4><<<g, 256, 0, st>>>(s, i0, n, a); break;
+    }
+    return cudaGetLastError();
+}
+
+cudaError_t launch_unpack_state(const Particles& s, int64_t i0, int64_t n, int ns, const UserArrays& a, cudaStream_t st)
+{
+    if (n == 0) return cudaSuccess;
+    const unsigned g = (unsigned)((n + 255) / 256);
+    switch (ns) {
+        case 1: unpack_state_kernel<1><<<g, 256, 0, st>>>(s, i0, n, a); break;
+        case 2: unpack_state_kernel<2><<<g, 256, 0, st>>>(s, i0, n, a); break;
+        case 3: unpack_state_kernel<3><<<g, 256, 0, st>>>(s, i0, n, a); break;
+        default: unpack_state_kernel<4><<<g, 256, 0, st>>>(s, i0, n, a); break;
     }
     return cudaGetLastError();
 }

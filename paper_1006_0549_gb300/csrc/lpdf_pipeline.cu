@@ -53,25 +53,12 @@ __device__ __forceinline__ unsigned rec_hash(int key) { return ((unsigned)key * 
 // The state streams through once per step: its loads skip L1 (which keeps the element field
 // rows and mesh records that the particles of an element share) and its stores are marked
 // streaming.
-__device__ __forceinline__ float ld_stream(const float* p)
-{
-    float v;
-    asm("ld.global.nc.L1::no_allocate.f32 %0, [%1];" : "=f"(v) : "l"(p));
-    return v;
-}
 __device__ __forceinline__ int ld_stream(const int* p)
 {
     int v;
     asm("ld.global.nc.L1::no_allocate.s32 %0, [%1];" : "=r"(v) : "l"(p));
     return v;
 }
-__device__ __forceinline__ uint32_t ld_stream(const uint32_t* p)
-{
-    uint32_t v;
-    asm("ld.global.nc.L1::no_allocate.u32 %0, [%1];" : "=r"(v) : "l"(p));
-    return v;
-}
-
 // The rest of a walk that has met a wall edge (edge walls): mirror the position across the wall
 // edge (U <- 2 U_w - U, U_w = (lid_u, 0, 0) on a moving wall), go on walking from the same
 // element, at most kReflCap mirrorings and kHopCap hops in all. Returns the owner, or -1 (lost).
@@ -120,7 +107,7 @@ static __device__ __noinline__ int walk_mirroring(const DevMesh& M, float lid_u,
 
 // one particle, its state loaded: advanced, located and written to position i of the next buffer
 template <int NS, int kKind>
-__device__ __forceinline__ void advance_store(const DevMesh& M, const DevState& nxt, const float* __restrict__ EF,
+__device__ __forceinline__ void advance_store(const DevMesh& M, const Particles& nxt, const float* __restrict__ EF,
                                               const StepParams& P, unsigned long long* __restrict__ status,
                                               int64_t i, ParticleState<NS>& p, unsigned& err, int& hops)
 {
@@ -176,37 +163,33 @@ __device__ __forceinline__ void advance_store(const DevMesh& M, const DevState& 
         atomicAdd(&status[1], 1ull);
         atomicCAS(&status[2], ~0ull, (unsigned long long)p.pid);
     }
-    __stcs(nxt.x + i, p.x);
-    __stcs(nxt.y + i, p.y);
-    __stcs(nxt.u + i, p.u);
-    __stcs(nxt.v + i, p.v);
-    __stcs(nxt.w + i, p.w);
-    __stcs(nxt.om + i, p.om);
-#pragma unroll
-    for (int a = 0; a < NS; ++a) __stcs(nxt.psi + (size_t)a * nxt.cap + i, p.psi[a]);
+    const float r[8] = {p.x, p.y, p.u, p.v, p.w, p.om, p.psi[0], __uint_as_float(p.pid)};
+    rec_store_stream(nxt.rec + 8 * i, r);
+    rest_store<NS>(nxt.rest, i, p.psi);
     __stcs(nxt.elem + i, ne);
-    __stcs(nxt.pid + i, p.pid);
 }
 
 // one particle: position i of the next buffer takes particle perm[i] of the current one
 template <int NS, int kKind>
-__device__ __forceinline__ void advance_one(const DevMesh& M, const DevState& cur, const DevState& nxt,
+__device__ __forceinline__ void advance_one(const DevMesh& M, const Particles& cur, const Particles& nxt,
                                             const int* __restrict__ perm, const float* __restrict__ EF,
                                             const StepParams& P, unsigned long long* __restrict__ status, int64_t i,
                                             unsigned& err, int& hops)
 {
     const int src = ld_stream(perm + i);
     ParticleState<NS> p;
-    p.x = ld_stream(cur.x + src);
-    p.y = ld_stream(cur.y + src);
-    p.u = ld_stream(cur.u + src);
-    p.v = ld_stream(cur.v + src);
-    p.w = ld_stream(cur.w + src);
-    p.om = ld_stream(cur.om + src);
-#pragma unroll
-    for (int a = 0; a < NS; ++a) p.psi[a] = ld_stream(cur.psi + (size_t)a * cur.cap + src);
+    float r[8];
+    rec_load_stream(cur.rec + 8 * (int64_t)src, r);
     p.elem = ld_stream(cur.elem + src);
-    p.pid = ld_stream(cur.pid + src);
+    p.x = r[0];
+    p.y = r[1];
+    p.u = r[2];
+    p.v = r[3];
+    p.w = r[4];
+    p.om = r[5];
+    p.psi[0] = r[6];
+    p.pid = __float_as_uint(r[7]);
+    rest_load<NS>(cur.rest, src, p.psi);
     advance_store<NS, kKind>(M, nxt, EF, P, status, i, p, err, hops);
 }
 
@@ -221,8 +204,8 @@ __device__ __forceinline__ void advance_one(const DevMesh& M, const DevState& cu
 constexpr int kQChunk = 64;
 template <int NS, int kKind, int ABLK, int MINB, int kGrid>
 __global__ void __launch_bounds__(ABLK, MINB)
-advance_kernel(const __grid_constant__ DevMesh M, const __grid_constant__ DevState cur,
-               const __grid_constant__ DevState nxt, const int* __restrict__ perm, const float* __restrict__ EF,
+advance_kernel(const __grid_constant__ DevMesh M, const __grid_constant__ Particles cur,
+               const __grid_constant__ Particles nxt, const int* __restrict__ perm, const float* __restrict__ EF,
                const __grid_constant__ StepParams P, unsigned long long* __restrict__ status,
                unsigned* __restrict__ tiles)
 {
@@ -623,23 +606,27 @@ struct QGroup {
     }
 };
 
+// the position and the group's fields of particle j
 template <int NS, int G>
-__device__ __forceinline__ void gather_fields(const DevState& S, int j, float* f)
+__device__ __forceinline__ void gather_fields(const Particles& S, int j, float& x, float& y, float* f)
 {
-    if (G == 0) {
-        f[0] = S.u[j];
-        f[1] = S.v[j];
-        f[2] = S.w[j];
-        f[3] = S.om[j];
-    } else if (G == 1) {
+    const float4* r = reinterpret_cast<const float4*>(S.rec + 8 * (int64_t)j);
+    const float4 a = __ldg(r);
+    x = a.x;
+    y = a.y;
+    float psi[NS];
+    if (G != 1) {
+        f[0] = a.z;
+        f[1] = a.w;
+    }
+    const float4 b = __ldg(r + 1);
+    if (G != 1) f[2] = b.x;
+    if (G == 0) f[3] = b.y;
+    if (G != 0) {
+        psi[0] = b.z;
+        rest_load<NS>(S.rest, j, psi);
 #pragma unroll
-        for (int a = 0; a < NS; ++a) f[a] = S.psi[(size_t)a * S.cap + j];
-    } else {
-        f[0] = S.u[j];
-        f[1] = S.v[j];
-        f[2] = S.w[j];
-#pragma unroll
-        for (int a = 0; a < NS; ++a) f[3 + a] = S.psi[(size_t)a * S.cap + j];
+        for (int a_ = 0; a_ < NS; ++a_) f[(G == 2 ? 3 : 0) + a_] = psi[a_];
     }
 }
 
@@ -746,7 +733,7 @@ __device__ __forceinline__ long long to_fixed64(double v, unsigned& err)
 // the warp; the FP64 coefficients of the element combine them in FP64 and each node sum gets one
 // 64-bit fixed-point add per quantity.
 template <int NS, int G>
-__device__ __forceinline__ void moment_group(const DevState& S, const int* __restrict__ perm, int base, int end,
+__device__ __forceinline__ void moment_group(const Particles& S, const int* __restrict__ perm, int base, int end,
                                             float X0, float Y0, const double4& co, const int4& mv, int lane,
                                             unsigned long long* __restrict__ node_acc, unsigned& err)
 {
@@ -766,18 +753,14 @@ __device__ __forceinline__ void moment_group(const DevState& S, const int* __res
     int j2 = pos + 32 < end ? perm[pos + 32] : -1;
     float cx = 0.0f, cy = 0.0f, cf[NF];
     if (j1 >= 0) {
-        cx = S.x[j1];
-        cy = S.y[j1];
-        gather_fields<NS, G>(S, j1, cf);
+        gather_fields<NS, G>(S, j1, cx, cy, cf);
     }
 #pragma unroll 1
     for (; j1 >= 0; pos += 32) {
         const int j3 = pos + 64 < end ? perm[pos + 64] : -1;
         float nx = 0.0f, ny = 0.0f, nf[NF];
         if (j2 >= 0) {
-            nx = S.x[j2];
-            ny = S.y[j2];
-            gather_fields<NS, G>(S, j2, nf);
+            gather_fields<NS, G>(S, j2, nx, ny, nf);
         }
         // (dx, dy) = p - vertex 0 as exact double-floats (dh + dl), x and y packed
         float2 dh, dl;
@@ -845,7 +828,7 @@ __device__ __forceinline__ void moment_group(const DevState& S, const int* __res
 // (IECM) into their own accumulators instead
 template <int NS, int MBLK, int MMINB, bool kFlux = false>
 __global__ void __launch_bounds__(MBLK, MMINB) moments_kernel_df(const __grid_constant__ DevMesh M,
-                                                      const __grid_constant__ DevState S,
+                                                      const __grid_constant__ Particles S,
                                                       const int* __restrict__ perm, const int* __restrict__ kstart,
                                                       unsigned long long* __restrict__ node_acc,
                                                       unsigned long long* __restrict__ status)
@@ -923,7 +906,7 @@ __device__ __forceinline__ void warp_reduce_scatter(const float (&acc)[NK], int 
 
 template <int NS, int MBLK, int MMINB, bool kFlux = false>
 __global__ void __launch_bounds__(MBLK, MMINB) moments_kernel_f32(const __grid_constant__ DevMesh M,
-                                                      const __grid_constant__ DevState S,
+                                                      const __grid_constant__ Particles S,
                                                       const int* __restrict__ perm, const int* __restrict__ kstart,
                                                       unsigned long long* __restrict__ node_acc,
                                                       unsigned long long* __restrict__ status)
@@ -962,14 +945,16 @@ __global__ void __launch_bounds__(MBLK, MMINB) moments_kernel_f32(const __grid_c
 #pragma unroll
             for (int k = 0; k < MB; ++k) {
                 const int j = idx[k0 + k] >= 0 ? idx[k0 + k] : 0;
-                bx[buf][k] = S.x[j];
-                by[buf][k] = S.y[j];
-                bu[buf][k] = S.u[j];
-                bv[buf][k] = S.v[j];
-                bw[buf][k] = S.w[j];
-                if (!kFlux) bo[buf][k] = S.om[j];
-#pragma unroll
-                for (int a = 0; a < NS; ++a) bp[buf][k][a] = S.psi[(size_t)a * S.cap + j];
+                const float4* r = reinterpret_cast<const float4*>(S.rec + 8 * (int64_t)j);
+                const float4 ra = __ldg(r), rb = __ldg(r + 1);
+                bx[buf][k] = ra.x;
+                by[buf][k] = ra.y;
+                bu[buf][k] = ra.z;
+                bv[buf][k] = ra.w;
+                bw[buf][k] = rb.x;
+                bo[buf][k] = rb.y;
+                bp[buf][k][0] = rb.z;
+                rest_load<NS>(S.rest, j, bp[buf][k]);
             }
         };
         if constexpr (NB == 2) gather(0, 0);
@@ -1084,7 +1069,7 @@ __device__ __forceinline__ void half_reduce_scatter(const float (&acc)[NK], int 
 // the reduction's shuffles span the warp.
 template <int NS, int MBLK, int MMINB>
 __global__ void __launch_bounds__(MBLK, MMINB) moments_kernel_f32h(const __grid_constant__ DevMesh M,
-                                                       const __grid_constant__ DevState S,
+                                                       const __grid_constant__ Particles S,
                                                        const int* __restrict__ perm, const int* __restrict__ kstart,
                                                        unsigned long long* __restrict__ node_acc,
                                                        unsigned long long* __restrict__ status)
@@ -1132,14 +1117,16 @@ __global__ void __launch_bounds__(MBLK, MMINB) moments_kernel_f32h(const __grid_
 #pragma unroll
             for (int k = 0; k < MB; ++k) {
                 const int j = idx[k0 + k] >= 0 ? idx[k0 + k] : 0;
-                bx[buf][k] = S.x[j];
-                by[buf][k] = S.y[j];
-                bu[buf][k] = S.u[j];
-                bv[buf][k] = S.v[j];
-                bw[buf][k] = S.w[j];
-                bo[buf][k] = S.om[j];
-#pragma unroll
-                for (int a = 0; a < NS; ++a) bp[buf][k][a] = S.psi[(size_t)a * S.cap + j];
+                const float4* r = reinterpret_cast<const float4*>(S.rec + 8 * (int64_t)j);
+                const float4 ra = __ldg(r), rb = __ldg(r + 1);
+                bx[buf][k] = ra.x;
+                by[buf][k] = ra.y;
+                bu[buf][k] = ra.z;
+                bv[buf][k] = ra.w;
+                bw[buf][k] = rb.x;
+                bo[buf][k] = rb.y;
+                bp[buf][k][0] = rb.z;
+                rest_load<NS>(S.rest, j, bp[buf][k]);
             }
         };
         if (base < end) {
@@ -1235,7 +1222,7 @@ int sm_count_cached()
 }
 
 template <int NS, int kKind, int ABLK, int MINB, int kGrid>
-void launch_advance_v(const DevMesh& m, const DevState& cur, const DevState& nxt, const int* perm, const float* ef,
+void launch_advance_v(const DevMesh& m, const Particles& cur, const Particles& nxt, const int* perm, const float* ef,
                       const StepParams& p, unsigned long long* status, unsigned* tiles, cudaStream_t st)
 {
     const int64_t ntiles = (cur.n + ABLK - 1) / ABLK;
@@ -1245,7 +1232,7 @@ void launch_advance_v(const DevMesh& m, const DevState& cur, const DevState& nxt
 }
 
 template <int NS, int kKind>
-void launch_advance(int v, const DevMesh& m, const DevState& cur, const DevState& nxt, const int* perm,
+void launch_advance(int v, const DevMesh& m, const Particles& cur, const Particles& nxt, const int* perm,
                     const float* ef, const StepParams& p, unsigned long long* status, unsigned* tiles,
                     cudaStream_t st)
 {
@@ -1260,7 +1247,7 @@ void launch_advance(int v, const DevMesh& m, const DevState& cur, const DevState
 }
 
 template <int NS>
-void launch_moments(int v, int mode, const DevMesh& m, const DevState& s, const int* perm, const int* kstart,
+void launch_moments(int v, int mode, const DevMesh& m, const Particles& s, const int* perm, const int* kstart,
                     unsigned long long* node_acc, unsigned long long* status, cudaStream_t st)
 {
     const int64_t threads = (int64_t)m.n_tri * 32;
@@ -1294,7 +1281,7 @@ void launch_moments(int v, int mode, const DevMesh& m, const DevState& s, const 
 }
 
 template <int NS>
-cudaError_t run_pipeline(const DevMesh& m, const DevState& cur, const DevState& nxt, const float* fields,
+cudaError_t run_pipeline(const DevMesh& m, const Particles& cur, const Particles& nxt, const float* fields,
                          const StepParams& p, PipeScratch& w, unsigned long long* node_acc, unsigned long long* status,
                          cudaStream_t st, const cudaEvent_t* ev, const StepTune& tune, unsigned long long* flux_acc)
 {
@@ -1342,7 +1329,7 @@ cudaError_t run_pipeline(const DevMesh& m, const DevState& cur, const DevState& 
 
 }  // namespace
 
-cudaError_t launch_pdf_step_pipeline(const DevMesh& m, const DevState& cur, const DevState& nxt, int ns,
+cudaError_t launch_pdf_step_pipeline(const DevMesh& m, const Particles& cur, const Particles& nxt, int ns,
                                      const float* fields, const StepParams& p, PipeScratch& w,
                                      unsigned long long* node_acc, unsigned long long* status, cudaStream_t st,
                                      const cudaEvent_t* ev, const StepTune& tune, unsigned long long* flux_acc)

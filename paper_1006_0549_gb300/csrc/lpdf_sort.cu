@@ -113,6 +113,10 @@ __global__ void segment_sort_kernel(const int* __restrict__ start, int* __restri
     for (int i = threadIdx.x; i < len; i += blockDim.x) perm[b + i] = v[i];
 }
 
+struct Rec {
+    float4 a, b;
+};
+
 template <class T>
 __global__ void gather_kernel(const T* __restrict__ src, T* __restrict__ dst, const int* __restrict__ perm, int64_t n)
 {
@@ -122,7 +126,7 @@ __global__ void gather_kernel(const T* __restrict__ src, T* __restrict__ dst, co
 
 }  // namespace
 
-cudaError_t launch_sort(const DevMesh& m, const DevState& s, int ns, const DevState& dst, SortScratch& w,
+cudaError_t launch_sort(const DevMesh& m, const Particles& s, int ns, const Particles& dst, SortScratch& w,
                         unsigned long long* status, cudaStream_t st)
 {
     if (s.n == 0) return cudaSuccess;
@@ -138,16 +142,16 @@ cudaError_t launch_sort(const DevMesh& m, const DevState& s, int ns, const DevSt
     segment_sort_kernel<<<E + 1, 256, 0, st>>>(w.start, w.perm, status);
     const int64_t nblk = (s.n + 255) / 256;
     const unsigned gg = (unsigned)(nblk < 152 * 16 ? nblk : 152 * 16);
-    gather_kernel<float><<<gg, 256, 0, st>>>(s.x, dst.x, w.perm, s.n);
-    gather_kernel<float><<<gg, 256, 0, st>>>(s.y, dst.y, w.perm, s.n);
-    gather_kernel<float><<<gg, 256, 0, st>>>(s.u, dst.u, w.perm, s.n);
-    gather_kernel<float><<<gg, 256, 0, st>>>(s.v, dst.v, w.perm, s.n);
-    gather_kernel<float><<<gg, 256, 0, st>>>(s.w, dst.w, w.perm, s.n);
-    gather_kernel<float><<<gg, 256, 0, st>>>(s.om, dst.om, w.perm, s.n);
-    for (int a = 0; a < ns; ++a)
-        gather_kernel<float><<<gg, 256, 0, st>>>(s.psi + (size_t)a * s.cap, dst.psi + (size_t)a * dst.cap, w.perm, s.n);
+    // the records as 16-byte halves; the remaining scalars by their words
+    gather_kernel<Rec><<<gg, 256, 0, st>>>(reinterpret_cast<const Rec*>(s.rec), reinterpret_cast<Rec*>(dst.rec), w.perm, s.n);
+    if (rest_words(ns) == 1) gather_kernel<float><<<gg, 256, 0, st>>>(s.rest, dst.rest, w.perm, s.n);
+    if (rest_words(ns) == 2)
+        gather_kernel<float2><<<gg, 256, 0, st>>>(reinterpret_cast<const float2*>(s.rest), reinterpret_cast<float2*>(dst.rest),
+                                                  w.perm, s.n);
+    if (rest_words(ns) == 4)
+        gather_kernel<float4><<<gg, 256, 0, st>>>(reinterpret_cast<const float4*>(s.rest), reinterpret_cast<float4*>(dst.rest),
+                                                  w.perm, s.n);
     gather_kernel<int><<<gg, 256, 0, st>>>(s.elem, dst.elem, w.perm, s.n);
-    gather_kernel<uint32_t><<<gg, 256, 0, st>>>(s.pid, dst.pid, w.perm, s.n);
     return cudaGetLastError();
 }
 
