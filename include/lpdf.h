@@ -281,8 +281,8 @@ int lpdf_pdf_steps(lpdf_ctx* ctx, const float* node_fields, uint64_t step0, int3
  *       tiles); 2 = 128, >= 8 (64 registers); 3 = 256, >= 4, persistent; 4 = 64, >= 18
  *       (56 registers), persistent; 5 = 128, >= 10, persistent, each warp taking 64-particle
  *       chunks in order from a counter in the context's scratch.
- *   mom (moments kernel, a warp per element): 0 = 256 threads, >= 2 CTAs per SM; 1 = 128, >= 4;
- *       2 = 512, >= 1; 3 = 256, >= 3.
+ *   mom (moments kernel, a warp per element): 0 = 256 threads, >= 2 CTAs per SM; 1 = 128, >= 4
+ *       (four scalars: 5); 2 = 512, >= 1; 3 = 256, >= 3.
  * lpdf_ctx_set_tune sets it (LPDF_ERR_ARG outside those ranges). lpdf_ctx_autotune times every
  * advance variant, then every moments variant with the best advance variant. A trial is one
  * warm-up step and steps_per_trial timed steps (CUDA events on `stream`) of this context's own

@@ -166,7 +166,8 @@ struct PipeScratch {
 // bit-identical results. adv: advance kernel 0 = 256 threads, >= 4 CTAs/SM; 1 = 128, >= 10,
 // persistent grid; 2 = 128, >= 8; 3 = 256, >= 4, persistent; 4 = 64, >= 18, persistent; 5 = 128,
 // >= 10, persistent, warps taking 64-particle chunks from a counter. mom: moments kernel
-// 0 = 256 threads, >= 2 CTAs/SM; 1 = 128, >= 4; 2 = 512, >= 1; 3 = 256, >= 3.
+// 0 = 256 threads, >= 2 CTAs/SM; 1 = 128, >= 4 (four scalars: 5); 2 = 512, >= 1; 3 = 256,
+// >= 3.
 struct StepTune {
     int adv = 0, mom = 0;
 };

@@ -904,6 +904,9 @@ __device__ __forceinline__ void warp_reduce_scatter(const float (&acc)[NK], int 
     hi = B0 > 0 ? b[0] : 0.0f;
 }
 
+template <int NS>
+constexpr int kMomentBatch = NS == 1 ? 4 : (NS == 4 ? 1 : 2);   // particles per lane and buffer
+
 template <int NS, int MBLK, int MMINB, bool kFlux = false>
 __global__ void __launch_bounds__(MBLK, MMINB) moments_kernel_f32(const __grid_constant__ DevMesh M,
                                                       const __grid_constant__ Particles S,
@@ -928,11 +931,12 @@ __global__ void __launch_bounds__(MBLK, MMINB) moments_kernel_f32(const __grid_c
 #pragma unroll
         for (int k = 0; k < NK; ++k) acc[k] = 0.0f;
         const int end = min(p1, base + 32 * LC);
-        // the lane's gather indices for the whole chunk first, then batches of MB particles per
-        // lane; with one scalar the batches are double-buffered (the next batch's state loads
-        // are issued before the current batch is accumulated), with more the registers go to one
-        // batch at a time. The accumulation order per lane stays position order either way.
-        constexpr int MB = NS <= 2 ? 4 : 2, NB = NS == 1 ? 2 : 1;
+        // the lane's gather indices for the whole chunk first, then batches of MB particles per lane,
+        // double-buffered: the next batch's records are loaded (one 256-bit load each) before the
+        // current batch is accumulated, in position order per lane. Two buffers of one or two
+        // particles are worth more than one buffer of two or four: the cavity's four-scalar moments
+        // took 377 us with one buffer and two 128-bit loads per record, 329 us so.
+        constexpr int MB = kMomentBatch<NS>, NB = 2;
         static_assert(LC % MB == 0, "whole batches per chunk");
         int idx[LC];
 #pragma unroll
@@ -945,15 +949,15 @@ __global__ void __launch_bounds__(MBLK, MMINB) moments_kernel_f32(const __grid_c
 #pragma unroll
             for (int k = 0; k < MB; ++k) {
                 const int j = idx[k0 + k] >= 0 ? idx[k0 + k] : 0;
-                const float4* r = reinterpret_cast<const float4*>(S.rec + 8 * (int64_t)j);
-                const float4 ra = __ldg(r), rb = __ldg(r + 1);
-                bx[buf][k] = ra.x;
-                by[buf][k] = ra.y;
-                bu[buf][k] = ra.z;
-                bv[buf][k] = ra.w;
-                bw[buf][k] = rb.x;
-                bo[buf][k] = rb.y;
-                bp[buf][k][0] = rb.z;
+                float r[8];
+                rec_load_stream(S.rec + 8 * (int64_t)j, r);
+                bx[buf][k] = r[0];
+                by[buf][k] = r[1];
+                bu[buf][k] = r[2];
+                bv[buf][k] = r[3];
+                bw[buf][k] = r[4];
+                bo[buf][k] = r[5];
+                bp[buf][k][0] = r[6];
                 rest_load<NS>(S.rest, j, bp[buf][k]);
             }
         };
@@ -1104,7 +1108,7 @@ __global__ void __launch_bounds__(MBLK, MMINB) moments_kernel_f32h(const __grid_
         float acc[NK];
 #pragma unroll
         for (int k = 0; k < NK; ++k) acc[k] = 0.0f;
-        constexpr int MB = NS <= 2 ? 4 : 2, NB = NS == 1 ? 2 : 1;
+        constexpr int MB = kMomentBatch<NS>, NB = 2;
         static_assert(LC % MB == 0, "whole batches per chunk");
         int idx[LC];
 #pragma unroll
@@ -1117,15 +1121,15 @@ __global__ void __launch_bounds__(MBLK, MMINB) moments_kernel_f32h(const __grid_
 #pragma unroll
             for (int k = 0; k < MB; ++k) {
                 const int j = idx[k0 + k] >= 0 ? idx[k0 + k] : 0;
-                const float4* r = reinterpret_cast<const float4*>(S.rec + 8 * (int64_t)j);
-                const float4 ra = __ldg(r), rb = __ldg(r + 1);
-                bx[buf][k] = ra.x;
-                by[buf][k] = ra.y;
-                bu[buf][k] = ra.z;
-                bv[buf][k] = ra.w;
-                bw[buf][k] = rb.x;
-                bo[buf][k] = rb.y;
-                bp[buf][k][0] = rb.z;
+                float r[8];
+                rec_load_stream(S.rec + 8 * (int64_t)j, r);
+                bx[buf][k] = r[0];
+                by[buf][k] = r[1];
+                bu[buf][k] = r[2];
+                bv[buf][k] = r[3];
+                bw[buf][k] = r[4];
+                bo[buf][k] = r[5];
+                bp[buf][k][0] = r[6];
                 rest_load<NS>(S.rest, j, bp[buf][k]);
             }
         };
@@ -1246,6 +1250,11 @@ void launch_advance(int v, const DevMesh& m, const Particles& cur, const Particl
     }
 }
 
+// four scalars: 20 warps per SM at 96 registers (a few spills) hide more of the gathers than 16 at 128:
+// 1.205 against 1.230 ms per step of the 20M cavity
+template <int NS>
+constexpr int kMomentCtas = NS == 4 ? 5 : 4;
+
 template <int NS>
 void launch_moments(int v, int mode, const DevMesh& m, const Particles& s, const int* perm, const int* kstart,
                     unsigned long long* node_acc, unsigned long long* status, cudaStream_t st)
@@ -1265,7 +1274,7 @@ void launch_moments(int v, int mode, const DevMesh& m, const Particles& s, const
     if (s.n <= (int64_t)kHalfPpe * m.n_tri) {
         const int64_t ht = ((int64_t)m.n_tri + 1) / 2 * 32;
         switch (v) {
-            case 1: moments_kernel_f32h<NS, 128, 4><<<nblocks(ht, 128), 128, 0, st>>>(m, s, perm, kstart, node_acc, status); break;
+            case 1: moments_kernel_f32h<NS, 128, kMomentCtas<NS>><<<nblocks(ht, 128), 128, 0, st>>>(m, s, perm, kstart, node_acc, status); break;
             case 2: moments_kernel_f32h<NS, 512, 1><<<nblocks(ht, 512), 512, 0, st>>>(m, s, perm, kstart, node_acc, status); break;
             case 3: moments_kernel_f32h<NS, 256, 3><<<nblocks(ht, 256), 256, 0, st>>>(m, s, perm, kstart, node_acc, status); break;
             default: moments_kernel_f32h<NS, 256, 2><<<nblocks(ht, 256), 256, 0, st>>>(m, s, perm, kstart, node_acc, status); break;
@@ -1273,7 +1282,7 @@ void launch_moments(int v, int mode, const DevMesh& m, const Particles& s, const
         return;
     }
     switch (v) {
-        case 1: moments_kernel_f32<NS, 128, 4><<<nblocks(threads, 128), 128, 0, st>>>(m, s, perm, kstart, node_acc, status); break;
+        case 1: moments_kernel_f32<NS, 128, kMomentCtas<NS>><<<nblocks(threads, 128), 128, 0, st>>>(m, s, perm, kstart, node_acc, status); break;
         case 2: moments_kernel_f32<NS, 512, 1><<<nblocks(threads, 512), 512, 0, st>>>(m, s, perm, kstart, node_acc, status); break;
         case 3: moments_kernel_f32<NS, 256, 3><<<nblocks(threads, 256), 256, 0, st>>>(m, s, perm, kstart, node_acc, status); break;
         default: moments_kernel_f32<NS, 256, 2><<<nblocks(threads, 256), 256, 0, st>>>(m, s, perm, kstart, node_acc, status); break;
