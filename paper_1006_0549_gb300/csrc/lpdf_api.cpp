@@ -516,7 +516,7 @@ int lpdf_ctx_create(const lpdf_mesh* mesh, const lpdf_params* params, int64_t ca
     s2.cap = cap;
     const size_t E = (size_t)mesh->d.n_tri;
     const size_t rest = (size_t)cap * rest_words(c->ns);
-    if ((ce = dalloc(&s.rec, 8 * cap)) || (ce = dalloc(&s.elem, cap)) || (rest && (ce = dalloc(&s.rest, rest))) ||
+    if ((ce = pipeline_configure()) || (ce = dalloc(&s.rec, 8 * cap)) || (ce = dalloc(&s.elem, cap)) || (rest && (ce = dalloc(&s.rest, rest))) ||
         (ce = dalloc(&s2.rec, 8 * cap)) || (ce = dalloc(&s2.elem, cap)) || (rest && (ce = dalloc(&s2.rest, rest))) ||
         (ce = dalloc(&c->sort.cnt, E + 1)) || (ce = dalloc(&c->sort.cursor, E + 1)) ||
         (ce = dalloc(&c->sort.start, E + 2)) || (ce = dalloc(&c->sort.perm, cap)) ||
@@ -751,13 +751,14 @@ int lpdf_pdf_step(lpdf_ctx* c, const float* node_fields, uint64_t step, void* st
     if (!c || !node_fields) return fail(LPDF_ERR_ARG, "pdf_step: NULL argument");
     const cudaStream_t st = (cudaStream_t)stream;
     ++c->nsteps;
-    const int nq = nquant(c->ns);
-    CUDA_TRY(cudaMemsetAsync(c->node_acc, 0, sizeof(unsigned long long) * (size_t)c->mesh->d.n_nodes * nq, st));
+    if (c->s.n == 0) {   // the step's first kernel zeroes the sums, but there is none
+        const size_t nodes = (size_t)c->mesh->d.n_nodes;
+        CUDA_TRY(cudaMemsetAsync(c->node_acc, 0, sizeof(unsigned long long) * nodes * nquant(c->ns), st));
+        if (c->flux_acc) CUDA_TRY(cudaMemsetAsync(c->flux_acc, 0, sizeof(unsigned long long) * nodes * 3 * c->ns, st));
+    }
     StepParams p = make_step_params(c->params, c->mesh, step);
     p.comp = c->mesh->d.n_comp > 1 ? c->comp : nullptr;
     p.beta = c->params.mixing == 1 ? c->iecm_beta : nullptr;
-    if (c->flux_acc)
-        CUDA_TRY(cudaMemsetAsync(c->flux_acc, 0, sizeof(unsigned long long) * (size_t)c->mesh->d.n_nodes * 3 * c->ns, st));
     c->s2.n = c->s.n;
     std::array<cudaEvent_t, 4> ev{};
     if (c->timing) {
@@ -787,14 +788,10 @@ static int capture_steps(lpdf_ctx* c, const float* fields, int slot)
     const cudaStream_t cs = c->graph_stream;
     (void)sm_count();   // device queries stay outside the capture
     CUDA_TRY(cudaStreamBeginCapture(cs, cudaStreamCaptureModeThreadLocal));
-    const int nq = nquant(c->ns);
     Particles a = c->s, b = c->s2;
     PipeScratch w = c->pipe;
     cudaError_t e = cudaSuccess;
     for (int k = 0; k < 2 && e == cudaSuccess; ++k) {
-        e = cudaMemsetAsync(c->node_acc, 0, sizeof(unsigned long long) * (size_t)c->mesh->d.n_nodes * nq, cs);
-        if (e == cudaSuccess && c->flux_acc)
-            e = cudaMemsetAsync(c->flux_acc, 0, sizeof(unsigned long long) * (size_t)c->mesh->d.n_nodes * 3 * c->ns, cs);
         StepParams p = make_step_params(c->params, c->mesh, 0);
         p.comp = c->mesh->d.n_comp > 1 ? c->comp : nullptr;
         p.beta = c->params.mixing == 1 ? c->iecm_beta : nullptr;

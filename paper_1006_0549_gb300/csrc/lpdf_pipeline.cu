@@ -246,14 +246,20 @@ advance_kernel(const __grid_constant__ DevMesh M, const __grid_constant__ Partic
 }
 
 // ------------------------------------------------------------------------------------------
-// T: thread (e, q) writes float4 q of the three rows of element e
+// T: thread (e, q) writes float4 q of the three rows of element e; the step's counters and sums are
+// zeroed on the way (a memset each was a launch each)
 // ------------------------------------------------------------------------------------------
 template <int NS>
 __global__ void element_fields_kernel(const __grid_constant__ DevMesh M, const float* __restrict__ F,
-                                      float* __restrict__ EF)
+                                      float* __restrict__ EF, int* __restrict__ kwork, int nk,
+                                      unsigned long long* __restrict__ acc, int64_t na,
+                                      unsigned long long* __restrict__ flux, int64_t nf)
 {
     constexpr int NFP = (22 + NS + 3) / 4 * 4, NQ4 = NFP / 4;
-    const int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    const int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x, nt = (int64_t)gridDim.x * blockDim.x;
+    for (int64_t i = t; i < nk; i += nt) kwork[i] = 0;
+    for (int64_t i = t; i < na; i += nt) acc[i] = 0ull;
+    for (int64_t i = t; i < nf; i += nt) flux[i] = 0ull;
     if (t >= (int64_t)M.n_tri * NQ4) return;
     const int e = (int)(t / NQ4), q = (int)(t - (int64_t)e * NQ4);
     const int4 V = __ldg(&M.ev[e]);
@@ -272,32 +278,30 @@ __global__ void element_fields_kernel(const __grid_constant__ DevMesh M, const f
 }
 
 // ------------------------------------------------------------------------------------------
-// H: one warp per record block of kBlk positions, warp-synchronous (no block barriers)
+// H: one warp per record block (blk) of kBlk positions, warp-synchronous (no block barriers)
 // ------------------------------------------------------------------------------------------
 constexpr int kHWarps = 8;             // warps (record blocks) per CTA
 constexpr int kRows = kBlk / 32;       // rows of 32 positions in a record block
 constexpr int kWHash = 256;            // per-warp hash slots (a block has at most kBlk elements)
 static_assert(kWHash == 256 && kWHash >= kBlk, "rec_hash gives 8 bits; a block has at most kBlk elements");
 
-__global__ void __launch_bounds__(32 * kHWarps) histogram_kernel(const int* __restrict__ elem, int64_t n,
-                                                               uint16_t* __restrict__ rrank,
-                                                               int* __restrict__ rec_key, int* __restrict__ rec_cnt,
-                                                               int* __restrict__ nrec, int* __restrict__ kcnt,
-                                                               int* __restrict__ krc, unsigned long long* __restrict__ status)
+struct HistShared {               // a warp's
+    int hkey[kWHash];
+    unsigned short hcnt[kWHash];
+    unsigned char hrec[kWHash];
+    short used[kBlk];             // slot of each record, in insertion order
+};
+
+__device__ __forceinline__ void histogram_block(HistShared& sh, const int* elem, int64_t n, int64_t blk, uint16_t* rrank,
+                                                int* rec_key, int* rec_cnt, int* nrec, int* kcnt, int* krc,
+                                                unsigned long long* status)
 {
-    __shared__ int hkey_s[kHWarps][kWHash];
-    __shared__ unsigned short hcnt_s[kHWarps][kWHash];
-    __shared__ unsigned char hrec_s[kHWarps][kWHash];
-    __shared__ short used_s[kHWarps][kBlk];   // slot of each record, in insertion order
-    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+    const int lane = threadIdx.x & 31;
     const unsigned lt = (1u << lane) - 1u;
-    const int64_t blk = (int64_t)blockIdx.x * kHWarps + wid;     // the record block of this warp
-    const int64_t nblk = (n + kBlk - 1) / kBlk;
-    if (blk >= nblk) return;
-    int* const hkey = hkey_s[wid];
-    unsigned short* const hcnt = hcnt_s[wid];
-    unsigned char* const hrec = hrec_s[wid];
-    short* const used = used_s[wid];
+    int* const hkey = sh.hkey;
+    unsigned short* const hcnt = sh.hcnt;
+    unsigned char* const hrec = sh.hrec;
+    short* const used = sh.used;
     for (int s = lane; s < kWHash; s += 32) hkey[s] = -1;
     const int64_t base = blk * kBlk;
     int key[kRows];
@@ -372,6 +376,19 @@ __global__ void __launch_bounds__(32 * kHWarps) histogram_kernel(const int* __re
     if (lane == 0 && e_or) atomicOr(&status[0], (unsigned long long)e_or);
 }
 
+__global__ void __launch_bounds__(32 * kHWarps) histogram_kernel(const int* __restrict__ elem, int64_t n,
+                                                               uint16_t* __restrict__ rrank,
+                                                               int* __restrict__ rec_key, int* __restrict__ rec_cnt,
+                                                               int* __restrict__ nrec, int* __restrict__ kcnt,
+                                                               int* __restrict__ krc, unsigned long long* __restrict__ status)
+{
+    __shared__ HistShared sh[kHWarps];
+    const int wid = threadIdx.x >> 5;
+    const int64_t blk = (int64_t)blockIdx.x * kHWarps + wid;     // the record block of this warp
+    if (blk >= (n + kBlk - 1) / kBlk) return;
+    histogram_block(sh[wid], elem, n, blk, rrank, rec_key, rec_cnt, nrec, kcnt, krc, status);
+}
+
 // ------------------------------------------------------------------------------------------
 // S1: exclusive scan of two int arrays of length n (blockIdx.y picks the array)
 // ------------------------------------------------------------------------------------------
@@ -436,6 +453,38 @@ __global__ void __launch_bounds__(kScanThreads) scan_tiles_kernel(ScanPair sp, i
     if (threadIdx.x == 0) sp.tot(a)[blockIdx.x] = total;
 }
 
+// the same in one launch for few tiles: every block first adds up all that lies before its tile
+// (at most kScanOneTiles - 1 tiles: 60 KB from L2) instead of waiting for the others
+constexpr int kScanOneTiles = 16;
+
+__global__ void __launch_bounds__(kScanThreads) scan_one_kernel(ScanPair sp, int n)
+{
+    __shared__ int wsum[33];
+    const int a = blockIdx.y;
+    const int* const in = sp.src(a);
+    const int64_t tile0 = (int64_t)blockIdx.x * kScanTile;
+    int before = 0;
+#pragma unroll 8
+    for (int64_t j = threadIdx.x; j < tile0; j += kScanThreads) before += in[j];
+    int carry;
+    block_scan_1024(before, wsum, carry);
+    const int64_t base = tile0 + (int64_t)threadIdx.x * kScanItems;
+    int v[kScanItems];
+    int sum = 0;
+#pragma unroll
+    for (int k = 0; k < kScanItems; ++k) {
+        v[k] = base + k < n ? in[base + k] : 0;
+        sum += v[k];
+    }
+    int total;
+    int run = carry + block_scan_1024(sum, wsum, total);
+#pragma unroll
+    for (int k = 0; k < kScanItems; ++k) {
+        if (base + k < n) sp.dst(a)[base + k] = run;
+        run += v[k];
+    }
+}
+
 // the tile totals (at most kScanTile of them) scanned in place
 __global__ void __launch_bounds__(kScanThreads) scan_parts_kernel(ScanPair sp, int ntiles)
 {
@@ -469,31 +518,31 @@ __global__ void scan_add_kernel(ScanPair sp, int n)
 // S2, S3, S4
 // ------------------------------------------------------------------------------------------
 // a warp per record block (a block holds a few records: one per distinct element)
-__global__ void __launch_bounds__(256) record_scatter_kernel(const int* __restrict__ nrec, const int* __restrict__ rec_key,
-                                                            const int* __restrict__ krstart, int* __restrict__ kcur,
-                                                            int* __restrict__ klist, int64_t nblk)
+__device__ __forceinline__ void record_scatter_block(int64_t blk, const int* nrec, const int* rec_key, const int* krstart,
+                                                     int* kcur, int* klist)
 {
-    const int64_t blk = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-    if (blk >= nblk) return;
-    const int lane = threadIdx.x & 31;
     const int nr = nrec[blk];
-    for (int t = lane; t < nr; t += 32) {
+    for (int t = threadIdx.x & 31; t < nr; t += 32) {
         const int rid = (int)blk * kBlk + t;
         const int key = rec_key[rid];
         klist[krstart[key] + atomicAdd(&kcur[key], 1)] = rid;
     }
 }
 
+__global__ void __launch_bounds__(256) record_scatter_kernel(const int* __restrict__ nrec, const int* __restrict__ rec_key,
+                                                            const int* __restrict__ krstart, int* __restrict__ kcur,
+                                                            int* __restrict__ klist, int64_t nblk)
+{
+    const int64_t blk = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
+    if (blk < nblk) record_scatter_block(blk, nrec, rec_key, krstart, kcur, klist);
+}
+
 // a warp per element: its records in block order (a record id is block * kBlk + slot, and an
 // element has at most one record per block), then the running offsets
-__global__ void __launch_bounds__(256) key_offsets_kernel(int n_keys, const int* __restrict__ kstart,
-                                                          const int* __restrict__ krstart,
-                                                          const int* __restrict__ klist, int* __restrict__ klist2,
-                                                          const int* __restrict__ rec_cnt, int* __restrict__ rec_off)
+__device__ __forceinline__ void key_offsets_elem(int e, const int* kstart, const int* krstart, const int* klist, int* klist2,
+                                                 const int* rec_cnt, int* rec_off)
 {
-    const int e = (int)(((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5);
     const int lane = threadIdx.x & 31;
-    if (e >= n_keys) return;
     const int r0 = krstart[e], r1 = krstart[e + 1], nr = r1 - r0;
     if (nr == 0) return;
     if (nr == 1) {
@@ -524,6 +573,15 @@ __global__ void __launch_bounds__(256) key_offsets_kernel(int n_keys, const int*
     }
 }
 
+__global__ void __launch_bounds__(256) key_offsets_kernel(int n_keys, const int* __restrict__ kstart,
+                                                          const int* __restrict__ krstart,
+                                                          const int* __restrict__ klist, int* __restrict__ klist2,
+                                                          const int* __restrict__ rec_cnt, int* __restrict__ rec_off)
+{
+    const int e = (int)(((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5);
+    if (e < n_keys) key_offsets_elem(e, kstart, krstart, klist, klist2, rec_cnt, rec_off);
+}
+
 constexpr int kScatterPer = 4;   // particles per thread of the particle scatter
 
 __global__ void particle_scatter_kernel(int64_t n, const uint16_t* __restrict__ rrank, const int* __restrict__ rec_off,
@@ -546,6 +604,66 @@ __global__ void particle_scatter_kernel(int64_t n, const uint16_t* __restrict__ 
     for (int k = 0; k < kScatterPer; ++k) {
         const int64_t i = i0 + (int64_t)k * blockDim.x;
         if (i < n) perm_new[off[k] + (pk[k] & 255u)] = (int)i;
+    }
+}
+
+// The whole re-bucketing (H, S1, S2, S3, S4) of a small ensemble in one launch: a cluster of
+// kSmallCtas CTAs that meet at the hardware's cluster barrier between the phases. Seven launches of
+// 3-5 us of latency each took 32 us at 50,000 particles, however little there is to do. One cluster is
+// 5 % of the GPU: up to kSmallN particles its phases still take less than the launches would.
+constexpr int kSmallCtas = 8, kSmallThreads = 1024, kSmallN = 1 << 17, kSmallKeys = 8 * kSmallThreads;
+constexpr size_t kSmallSmem = sizeof(HistShared) * (kSmallThreads / 32);
+
+__device__ __forceinline__ void cluster_sync()
+{
+    asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
+}
+
+__global__ void __launch_bounds__(kSmallThreads, 1) rebucket_small_kernel(const int* elem, int n, int E, PipeScratch w,
+                                                                          unsigned long long* status)
+{
+    extern __shared__ __align__(16) unsigned char dyn[];
+    __shared__ int wsum[33];
+    HistShared* const sh = reinterpret_cast<HistShared*>(dyn);
+    const int wid = threadIdx.x >> 5, gw = (int)(blockIdx.x * (kSmallThreads / 32)) + wid;
+    constexpr int kWarpsAll = kSmallCtas * kSmallThreads / 32;
+    int* const kcnt = w.kwork;
+    int* const krc = w.kwork + (E + 1);
+    int* const kcur = w.kwork + 2 * (E + 1);
+    const int nblk = (n + kBlk - 1) / kBlk;
+    for (int blk = gw; blk < nblk; blk += kWarpsAll) {
+        histogram_block(sh[wid], elem, n, blk, w.rrank, w.rec_key, w.rec_cnt, w.nrec, kcnt, krc, status);
+        __syncwarp();
+    }
+    cluster_sync();
+    if (blockIdx.x < 2) {
+        // S1: CTA 0 scans the particles, CTA 1 the records per element
+        const int* const in = blockIdx.x ? krc : kcnt;
+        int* const out = blockIdx.x ? w.krstart : w.kstart;
+        constexpr int kPer = kSmallKeys / kSmallThreads;
+        const int base = threadIdx.x * kPer;
+        int v[kPer], sum = 0;
+#pragma unroll
+        for (int k = 0; k < kPer; ++k) {
+            v[k] = base + k <= E ? __ldcg(in + base + k) : 0;
+            sum += v[k];
+        }
+        int total;
+        int run = block_scan_1024(sum, wsum, total);
+#pragma unroll
+        for (int k = 0; k < kPer; ++k) {
+            if (base + k <= E) out[base + k] = run;
+            run += v[k];
+        }
+    }
+    cluster_sync();
+    for (int blk = gw; blk < nblk; blk += kWarpsAll) record_scatter_block(blk, w.nrec, w.rec_key, w.krstart, kcur, w.klist);
+    cluster_sync();
+    for (int e = gw; e < E; e += kWarpsAll) key_offsets_elem(e, w.kstart, w.krstart, w.klist, w.klist2, w.rec_cnt, w.rec_off);
+    cluster_sync();
+    for (int i = (int)(blockIdx.x * kSmallThreads + threadIdx.x); i < n; i += kSmallCtas * kSmallThreads) {
+        const unsigned pk = w.rrank[i];
+        w.perm_new[w.rec_off[(i / kBlk) * kBlk + (pk >> 8)] + (pk & 255u)] = i;
     }
 }
 
@@ -1204,6 +1322,10 @@ cudaError_t scan_pair(const int* in0, int* out0, const int* in1, int* out1, int 
     const int ntiles = (n + kScanTile - 1) / kScanTile;
     if (ntiles > kScanTile) return cudaErrorInvalidValue;
     ScanPair sp{{in0, in1}, {out0, out1}, {part, part + kScanTile}};
+    if (ntiles <= kScanOneTiles) {
+        scan_one_kernel<<<dim3(ntiles, 2), kScanThreads, 0, st>>>(sp, n);
+        return cudaGetLastError();
+    }
     scan_tiles_kernel<<<dim3(ntiles, 2), kScanThreads, 0, st>>>(sp, n);
     scan_parts_kernel<<<dim3(1, 2), kScanThreads, 0, st>>>(sp, ntiles);
     scan_add_kernel<<<dim3(nblocks(n, 256), 2), 256, 0, st>>>(sp, n);
@@ -1289,6 +1411,23 @@ void launch_moments(int v, int mode, const DevMesh& m, const Particles& s, const
     }
 }
 
+cudaError_t launch_rebucket_small(const int* elem, int n, int E, const PipeScratch& w, unsigned long long* status,
+                                  cudaStream_t st)
+{
+    cudaLaunchConfig_t cfg{};
+    cfg.gridDim = dim3(kSmallCtas);
+    cfg.blockDim = dim3(kSmallThreads);
+    cfg.dynamicSmemBytes = kSmallSmem;
+    cfg.stream = st;
+    cudaLaunchAttribute at{};
+    at.id = cudaLaunchAttributeClusterDimension;
+    at.val.clusterDim.x = kSmallCtas;
+    at.val.clusterDim.y = at.val.clusterDim.z = 1;
+    cfg.attrs = &at;
+    cfg.numAttrs = 1;
+    return cudaLaunchKernelEx(&cfg, rebucket_small_kernel, elem, n, E, w, status);
+}
+
 template <int NS>
 cudaError_t run_pipeline(const DevMesh& m, const Particles& cur, const Particles& nxt, const float* fields,
                          const StepParams& p, PipeScratch& w, unsigned long long* node_acc, unsigned long long* status,
@@ -1298,15 +1437,15 @@ cudaError_t run_pipeline(const DevMesh& m, const Particles& cur, const Particles
     if (n == 0) return cudaSuccess;
     const int E = m.n_tri;
     const int64_t nblk = (n + kBlk - 1) / kBlk;
-    cudaError_t e = cudaMemsetAsync(w.kwork, 0, sizeof(int) * (3 * (size_t)(E + 1) + 1), st);
-    if (e != cudaSuccess) return e;
     int* kcnt = w.kwork;
     int* krc = w.kwork + (E + 1);
     int* kcur = w.kwork + 2 * (E + 1);
     unsigned* tiles = reinterpret_cast<unsigned*>(w.kwork + 3 * (E + 1));
     if (ev) cudaEventRecord(ev[0], st);
     constexpr int NQ4 = (22 + NS + 3) / 4;
-    element_fields_kernel<NS><<<nblocks((int64_t)E * NQ4, 256), 256, 0, st>>>(m, fields, w.efields);
+    element_fields_kernel<NS><<<nblocks((int64_t)E * NQ4, 256), 256, 0, st>>>(
+        m, fields, w.efields, w.kwork, 3 * (E + 1) + 1, node_acc, (int64_t)m.n_nodes * (11 + 2 * NS), flux_acc,
+        flux_acc ? (int64_t)m.n_nodes * 3 * NS : 0);
     // the kernel with the least code that covers the mesh and the model: walls off the frame,
     // IECM or reactions (kind 2); several components (kind 1); the plain step (kind 0)
     if (m.edge_walls || p.beta || p.react_k > 0.0f)
@@ -1314,14 +1453,19 @@ cudaError_t run_pipeline(const DevMesh& m, const Particles& cur, const Particles
     else if (m.n_comp > 1) launch_advance<NS, 1>(tune.adv, m, cur, nxt, w.perm, w.efields, p, status, tiles, st);
     else launch_advance<NS, 0>(tune.adv, m, cur, nxt, w.perm, w.efields, p, status, tiles, st);
     if (ev) cudaEventRecord(ev[1], st);
-    histogram_kernel<<<(unsigned)((nblk + kHWarps - 1) / kHWarps), 32 * kHWarps, 0, st>>>(
-        nxt.elem, n, w.rrank, w.rec_key, w.rec_cnt, w.nrec, kcnt, krc, status);
-    e = scan_pair(kcnt, w.kstart, krc, w.krstart, E + 1, w.scan_part, st);
-    if (e != cudaSuccess) return e;
-    record_scatter_kernel<<<nblocks(nblk * 32, 256), 256, 0, st>>>(w.nrec, w.rec_key, w.krstart, kcur, w.klist, nblk);
-    key_offsets_kernel<<<nblocks((int64_t)E * 32, 256), 256, 0, st>>>(E, w.kstart, w.krstart, w.klist, w.klist2,
-                                                                       w.rec_cnt, w.rec_off);
-    particle_scatter_kernel<<<nblocks(n, 256 * kScatterPer), 256, 0, st>>>(n, w.rrank, w.rec_off, w.perm_new);
+    if (n <= kSmallN && E < kSmallKeys) {
+        const cudaError_t e = launch_rebucket_small(nxt.elem, (int)n, E, w, status, st);
+        if (e != cudaSuccess) return e;
+    } else {
+        histogram_kernel<<<(unsigned)((nblk + kHWarps - 1) / kHWarps), 32 * kHWarps, 0, st>>>(
+            nxt.elem, n, w.rrank, w.rec_key, w.rec_cnt, w.nrec, kcnt, krc, status);
+        const cudaError_t e = scan_pair(kcnt, w.kstart, krc, w.krstart, E + 1, w.scan_part, st);
+        if (e != cudaSuccess) return e;
+        record_scatter_kernel<<<nblocks(nblk * 32, 256), 256, 0, st>>>(w.nrec, w.rec_key, w.krstart, kcur, w.klist, nblk);
+        key_offsets_kernel<<<nblocks((int64_t)E * 32, 256), 256, 0, st>>>(E, w.kstart, w.krstart, w.klist, w.klist2,
+                                                                           w.rec_cnt, w.rec_off);
+        particle_scatter_kernel<<<nblocks(n, 256 * kScatterPer), 256, 0, st>>>(n, w.rrank, w.rec_off, w.perm_new);
+    }
     if (ev) cudaEventRecord(ev[2], st);
     launch_moments<NS>(tune.mom, p.moment_sums, m, nxt, w.perm_new, w.kstart, node_acc, status, st);
     if (flux_acc) {
@@ -1353,6 +1497,11 @@ cudaError_t launch_pdf_step_pipeline(const DevMesh& m, const Particles& cur, con
 }
 
 int sm_count() { return sm_count_cached(); }
+
+cudaError_t pipeline_configure()
+{
+    return cudaFuncSetAttribute(rebucket_small_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmallSmem);
+}
 
 cudaError_t launch_step_counter(unsigned long long* c, unsigned long long set, unsigned long long add, cudaStream_t st)
 {
