@@ -49,6 +49,7 @@ struct Smem {
     static constexpr int NF = 8 + NS;         // x, y, u, v, w, omega, psi[NS], elem, pid
     static constexpr int NQ = 11 + 2 * NS;
     static constexpr int NT = 128;            // node-table slots
+    static constexpr unsigned char kOne = 255;
     static constexpr int F_X = 0, F_Y = 1, F_U = 2, F_V = 3, F_W = 4, F_OM = 5, F_PSI = 6, F_ELEM = 6 + NS,
                          F_PID = 7 + NS;
     alignas(128) float tile[NF][kT];          // bulk-copy rows (16-byte aligned)
@@ -63,7 +64,8 @@ struct Smem {
     unsigned short ustart[kMaxBins + 1];
     short cslot[kMaxBins][3];                 // node-table slot of each bin's corners (-1: global)
     int wsum[kWarps];
-    int nbins, nunits, tfill, abort;
+    unsigned char qa[NQ], qb[NQ];             // a quantity as the product of two rows (kOne: 1)
+    int nbins, nunits, tfill, abort, hfill, ndirect;
     NodeTable<NQ, NT> table;
     unsigned long long bar;
 };
@@ -106,22 +108,23 @@ __device__ __forceinline__ int block_scan(int v, int* wsum, int& total)
     return off + incl - v;
 }
 
-// The exact walk test with its weights returned by value (a small struct travels through the
-// call's parameter space): the walk's own variables never have their address taken, so they are
-// not given a home in local memory.
-struct WalkLam {
-    int code;   // kWalkIn, or the exit as walk_test's `next`
-    float l0, l1, l2;
-};
-static __device__ __noinline__ WalkLam walk_test_lam(const DevMesh& M, int e, float px, float py)
+// The barycentric weights of (px, py) in e, from the orientation values (the FP32 values of orient_sign:
+// Kahan's FMA determinant of differences from each edge's first vertex) and the element's 1 / (2 area)
+__device__ __forceinline__ void orientation_weights(const DevMesh& M, int e, float px, float py, float* lam)
 {
-    float lam[3] = {0.0f, 0.0f, 0.0f};
-    WalkLam r;
-    r.code = walk_decide(M, e, px, py, lam);
-    r.l0 = lam[0];
-    r.l1 = lam[1];
-    r.l2 = lam[2];
-    return r;
+    const float4 X = __ldg(&M.ex[e]);
+    const float4 Y = __ldg(&M.ey[e]);
+    const float xs[3] = {X.x, X.y, X.z}, ys[3] = {Y.x, Y.y, Y.z};
+#pragma unroll
+    for (int k = 0; k < 3; ++k) {
+        const int b = (k + 1) % 3;
+        const float dx1 = __fsub_rn(xs[b], xs[k]), dy1 = __fsub_rn(ys[b], ys[k]);
+        const float dx2 = __fsub_rn(px, xs[k]), dy2 = __fsub_rn(py, ys[k]);
+        const float w = dy1 * dx2;
+        const float err = fmaf(-dy1, dx2, w);
+        const float f = fmaf(dx1, dy2, -w);
+        lam[(k + 2) % 3] = (f + err) * Y.w;   // edge k is opposite vertex k + 2
+    }
 }
 
 __device__ __forceinline__ unsigned hash_slot(int key) { return ((unsigned)key * 2654435761u) >> 24; }   // 8 bits
@@ -240,6 +243,21 @@ pdf_step_kernel(const __grid_constant__ DevMesh M, const __grid_constant__ DevSt
     const unsigned lt = (1u << lane) - 1u;
     for (int i = tid; i < NT; i += kThreads) sm.table.key[i] = -1;
     for (int i = tid; i < NT * NQ; i += kThreads) (&sm.table.acc[0][0])[i] = 0ull;
+    if (tid < NQ) {
+        // 1, u, v, w, uu, uv, uw, vv, vw, ww, omega, psi_a, psi_a^2
+        const int k = tid, a = k - 11;
+        int ra = SM::kOne, rb = SM::kOne;
+        if (k >= 1 && k <= 3) ra = SM::F_U + k - 1;
+        if (k >= 4 && k <= 9) {
+            ra = SM::F_U + (k < 7 ? 0 : (k < 9 ? 1 : 2));
+            rb = SM::F_U + (k < 7 ? k - 4 : (k < 9 ? k - 6 : 2));
+        }
+        if (k == 10) ra = SM::F_OM;
+        if (k >= 11) ra = SM::F_PSI + (a < NS ? a : a - NS);
+        if (k >= 11 + NS) rb = ra;
+        sm.qa[k] = (unsigned char)ra;
+        sm.qb[k] = (unsigned char)rb;
+    }
     if (tid == 0) {
         sm.tfill = 0;
         sm.abort = 0;
@@ -333,7 +351,7 @@ pdf_step_kernel(const __grid_constant__ DevMesh M, const __grid_constant__ DevSt
                 }
             };
             // one test of walk w; on a stop, record the particle and start the next one
-            auto step = [&](Walk& w, bool found, int next, float* lam) {
+            auto step = [&](Walk& w, bool found, int next) {
                 if (!(found || next < 0 || w.h >= kHopCap)) {
                     w.e = next;
                     ++w.h;
@@ -343,7 +361,10 @@ pdf_step_kernel(const __grid_constant__ DevMesh M, const __grid_constant__ DevSt
                 int ne = w.e;
                 bool lost = !found;
                 hops += found ? w.h : (next < 0 ? w.h : kHopCap + 1);
-                if (lost) {
+                float lam[3];
+                if (found) {
+                    orientation_weights(M, ne, w.px, w.py, lam);
+                } else {
                     ne = w.e0;
                     barycentric(__ldg(&M.ex[ne]), __ldg(&M.ey[ne]), w.px, w.py, lam[0], lam[1], lam[2]);
                 }
@@ -368,21 +389,27 @@ pdf_step_kernel(const __grid_constant__ DevMesh M, const __grid_constant__ DevSt
             start(B);
 #pragma unroll 1
             while (A.j >= 0 || B.j >= 0) {
-                WalkLam ra = {kWalkIn, 0.0f, 0.0f, 0.0f}, rb = ra;
-                if (A.j >= 0) ra = walk_test_lam(M, A.e, A.px, A.py);
-                if (B.j >= 0) rb = walk_test_lam(M, B.e, B.px, B.py);
+                // the certified test; the exact one where it is undecided (kWalkIn: inside, else the exit)
+                int ca = kWalkIn, cb = kWalkIn, next = -1;
                 if (A.j >= 0) {
-                    float la[3] = {ra.l0, ra.l1, ra.l2};
-                    step(A, ra.code == kWalkIn, ra.code == kWalkIn ? -1 : ra.code, la);
+                    const int r = walk_test_fast(M, A.e, A.px, A.py, next);
+                    ca = r > 0 ? kWalkIn : (r == 0 ? next : walk_test_code(M, A.e, A.px, A.py));
                 }
                 if (B.j >= 0) {
-                    float lb[3] = {rb.l0, rb.l1, rb.l2};
-                    step(B, rb.code == kWalkIn, rb.code == kWalkIn ? -1 : rb.code, lb);
+                    const int r = walk_test_fast(M, B.e, B.px, B.py, next);
+                    cb = r > 0 ? kWalkIn : (r == 0 ? next : walk_test_code(M, B.e, B.px, B.py));
                 }
+                if (A.j >= 0) step(A, ca == kWalkIn, ca);
+                if (B.j >= 0) step(B, cb == kWalkIn, cb);
             }
         }
         // ---- 3a. insert the new elements into the bin hash (one insert per distinct key of a row)
+        // an ensemble that no one sorts ends with as many elements as particles in a sub-tile: once the
+        // hash is full (kHash distinct elements or more) the sub-tile is not binned at all, its
+        // particles all take the direct path (a search of the full hash by every particle took most
+        // of the step there)
         for (int i = tid; i < kHash; i += kThreads) sm.hkey[i] = -1;
+        if (tid == 0) sm.hfill = sm.ndirect = 0;
         __syncthreads();
 #pragma unroll
         for (int j = 0; j < kPPT; ++j) {
@@ -393,12 +420,14 @@ pdf_step_kernel(const __grid_constant__ DevMesh M, const __grid_constant__ DevSt
 #pragma unroll 1
                 for (int p = 0; p < kHash; ++p) {
                     const int s = (h0 + p) & (kHash - 1);
-                    const int cur = sm.hkey[s];
+                    const int cur = *(volatile int*)&sm.hkey[s];
                     if (cur == k) break;
                     if (cur == -1) {
                         const int old = atomicCAS(&sm.hkey[s], -1, k);
+                        if (old == -1) atomicAdd(&sm.hfill, 1);
                         if (old == -1 || old == k) break;
                     }
+                    if ((p & 7) == 7 && *(volatile int*)&sm.hfill >= kHash) break;
                 }
             }
         }
@@ -418,7 +447,10 @@ pdf_step_kernel(const __grid_constant__ DevMesh M, const __grid_constant__ DevSt
             }
         }
         // ---- 3b. bins: the distinct new elements in ascending order -------------------------------
-        {
+        const bool binned = sm.hfill < kHash;   // (after the barrier above)
+        if (!binned) {
+            if (tid == 0) sm.nbins = 0;
+        } else {
             int* const list = reinterpret_cast<int*>(sm.perm);   // kHash ints fit in perm
             const int s0 = 2 * tid, s1 = 2 * tid + 1;
             const int k0 = sm.hkey[s0], k1 = sm.hkey[s1];
@@ -458,7 +490,7 @@ pdf_step_kernel(const __grid_constant__ DevMesh M, const __grid_constant__ DevSt
         for (int j = 0; j < kPPT; ++j) {
             const int k = mykey[j];
             unsigned short b = kNoBin;
-            if (k >= 0) {
+            if (k >= 0 && binned) {
                 const unsigned h0 = hash_slot(k);
 #pragma unroll 1
                 for (int p = 0; p < kHash; ++p) {
@@ -515,7 +547,11 @@ pdf_step_kernel(const __grid_constant__ DevMesh M, const __grid_constant__ DevSt
 #pragma unroll
             for (int j = 0; j < kPPT; ++j) {
                 const unsigned short b = mybin[j];
-                if (b == kNoBin) continue;
+                if (b == kNoBin) {
+                    // the list of the particles without a bin, from the end of perm
+                    if (mykey[j] >= 0) sm.perm[kT - 1 - atomicAdd(&sm.ndirect, 1)] = (unsigned short)(j * kThreads + tid);
+                    continue;
+                }
                 const int pos = sm.wcnt[b][wid] + myrank[j];
                 if (consistent(pos < kT, err)) sm.perm[pos] = (unsigned short)(j * kThreads + tid);
             }
@@ -588,22 +624,21 @@ pdf_step_kernel(const __grid_constant__ DevMesh M, const __grid_constant__ DevSt
                         table_add(sm.table, (int)sm.cslot[b][c], bin_node(sm, M, b, c), k,
                                   to_fixed(acc[c * NQ + k], err), node_acc);
             }
-            // particles without a bin (more than kMaxBins distinct elements in the sub-tile)
-#pragma unroll 1
-            for (int j = 0; j < kPPT; ++j) {
-                const int t = j * kThreads + tid;
-                if (mybin[j] != kNoBin || mykey[j] < 0) continue;
-                const int4 mv = __ldg(&M.em[mykey[j]]);
-                const int nd[3] = {mv.x, mv.y, mv.z};
-                float q[NQ];
-                quantities<NS>(sm, t, q);
-                for (int c = 0; c < 3; ++c) {
-                    const float l = sm.lam[c][t];
-                    for (int k = 0; k < NQ; ++k) {
-                        const long long v = to_fixed(l * q[k], err);
-                        if (v != 0) atomicAdd(&node_acc[(size_t)nd[c] * NQ + k], (unsigned long long)v);
-                    }
-                }
+            // particles without a bin (more than kMaxBins distinct elements in the sub-tile): a lane per
+            // (particle, corner, quantity), neighbouring lanes on neighbouring sums of one node, so that
+            // a warp's atomics fall in a few sectors (a particle per lane scattered each of its 3 NQ)
+            const int nitems = sm.ndirect * NK;
+#pragma unroll 4
+            for (int i = tid; i < nitems; i += kThreads) {
+                const int d = i / NK, k = i - d * NK;
+                const int c = k / NQ, q = k - c * NQ;
+                const int t = sm.perm[kT - 1 - d];
+                if (!consistent(t < kT, err)) continue;
+                const int node = __ldg(reinterpret_cast<const int*>(M.em + __float_as_int(sm.tile[SM::F_ELEM][t])) + c);
+                const int ra = sm.qa[q], rb = sm.qb[q];
+                const float fa = ra == SM::kOne ? 1.0f : sm.tile[ra][t], fb = rb == SM::kOne ? 1.0f : sm.tile[rb][t];
+                const long long v = to_fixed(sm.lam[c][t] * (fa * fb), err);
+                if (v != 0) atomicAdd(&node_acc[(size_t)node * NQ + q], (unsigned long long)v);
             }
             // the first kThreads units: one per thread
             int b = -1;
