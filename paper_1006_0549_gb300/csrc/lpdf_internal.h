@@ -228,8 +228,16 @@ struct Fem {
     // first), the epoch that the next launch starts from (a word never sees the same one twice) and
     // the result
     int cg_ctas = 1, max_deg = 0;    // max_deg: matrix entries of a row at most
+    // per CTA of cg_kernel the other CTAs' rows that its rows refer to (halo, CSR over the CTAs), and the
+    // matrix's columns as indices into (the CTA's rows, its halo)
+    int *lcol = nullptr, *halo_ptr = nullptr, *halo = nullptr;
+    int max_halo = 0;
     void* cg_slots = nullptr;
     ulonglong2* cg_z = nullptr;
+    unsigned long long* cg_zf = nullptr;   // the preconditioner's 8-byte words, and their epochs
+    unsigned cg_epoch32 = 1;
+    float* lmax = nullptr;       // bounds of the spectra of D^-1 A (device) and D^-1 K
+    float lmaxK = 0.0f;
     unsigned long long cg_epoch = 1;
     int* cg_out = nullptr;
     int* cg_host = nullptr;      // pinned copy

@@ -124,11 +124,13 @@ __global__ void elem_L2_kernel(const Fem F, const double* __restrict__ L2, doubl
 }
 
 // A = M + sum_e L2_e K_e (fixed contribution order per CSR entry); diag = its diagonal
+// (and the largest row sum of |D^-1 A| of the rows that are solved for, a bound of its spectrum)
 __global__ void assemble_kernel(const Fem F, const double* __restrict__ L2e, double* __restrict__ A,
-                                double* __restrict__ diag)
+                                double* __restrict__ diag, float* __restrict__ lmax)
 {
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= F.ndof) return;
+    float total = 0.0f;
     for (int j = F.row[i]; j < F.row[i + 1]; ++j) {
         double s = 0.0;
         for (int t = F.cptr[j]; t < F.cptr[j + 1]; ++t) {
@@ -138,8 +140,11 @@ __global__ void assemble_kernel(const Fem F, const double* __restrict__ L2e, dou
             s += L2e[e] * (F.area[e] * (g[2 * a] * g[2 * b] + g[2 * a + 1] * g[2 * b + 1]));
         }
         A[j] = F.Mval[j] + s;
+        total += fabsf((float)A[j]);
         if (F.col[j] == i) diag[i] = A[j];
     }
+    // positive floats compare like their bits
+    if (!F.wall[i]) atomicMax(reinterpret_cast<int*>(lmax), __float_as_int(total / (float)diag[i]));
 }
 
 // ---------------------------------------------------------------- batched PCG
@@ -195,9 +200,15 @@ struct CgArgs {
     const double *A0, *A1, *d0, *d1, *b0, *b1, *ref0, *ref1;
     double *x0, *x1;
     double* state;                          // 4 nc n (r, p, q, 1/diag of cg_kernel with several rows per thread)
+    const int *lcol, *halo_ptr, *halo;      // cg_kernel: see Fem
+    int width;                              // its rows and halo, at most
+    const float* lmax0;                     // bounds of the spectra of D^-1 A (device) and D^-1 K
+    float lmax1;
     double tol;
     unsigned long long epoch;
+    unsigned epoch32;                       // of the 8-byte words zf
     ulonglong2 *z, *slots;                  // nc n words; the partial sums' words
+    unsigned long long* zf;                 // 2 nc n words
     int* out;
 };
 
@@ -208,6 +219,18 @@ __device__ __forceinline__ void word_store(ulonglong2* p, double v, unsigned lon
         "mov.b128 t, {%1, %2};\n\t"
         "st.relaxed.gpu.global.b128 [%0], t;\n\t}" ::"l"(p), "l"(__double_as_longlong(v)), "l"(epoch)
         : "memory");
+}
+__device__ __forceinline__ ulonglong2 word_raw(const ulonglong2* p)
+{
+    ulonglong2 w;
+    asm volatile(
+        "{\n\t.reg .b128 t;\n\t"
+        "ld.relaxed.gpu.global.b128 t, [%2];\n\t"
+        "mov.b128 {%0, %1}, t;\n\t}"
+        : "=l"(w.x), "=l"(w.y)
+        : "l"(p)
+        : "memory");
+    return w;
 }
 // the word's value; ok stays set only if its epoch is the expected one
 __device__ __forceinline__ double word_load(const ulonglong2* p, unsigned long long epoch, bool& ok)
@@ -404,12 +427,43 @@ __global__ void __launch_bounds__(32) cg_small_kernel(const __grid_constant__ Cg
     }
 }
 
+// The preconditioner of cg_kernel with one row per thread and the matrix in shared memory: kCheb steps of
+// the Chebyshev iteration for D^-1 A z = D^-1 r on [lmax / kChebRatio, lmax] (Golub & Varga 1961), lmax a
+// Gershgorin bound: a fixed symmetric positive polynomial in D^-1 A, in FP32. A step has no sum over the
+// grid and no FP64: a CTA stores its rows' z as 8-byte words (value, epoch), polls the words of its halo
+// (the other CTAs' rows that its rows refer to) into shared memory, and gathers from there after a barrier
+// of the component's warps. What bounds it is that trip through L2: 1.3 us a step, while an FP64
+// iteration with its two grid sums takes 7. (Every thread polling its row's columns itself, up to ten
+// words, took 3 us: 30 warps x 10 uncoalesced loads a try.) Two buffers are used in turn: a thread
+// overwrites what it stored two steps ago, which its neighbours' CTAs read before they stored what its
+// own has read since; the pattern is symmetric. r is scaled by a power of two near 1/|r_0| first. What
+// FP32 rounds away changes the search directions a little, not the residual or the solution: those stay
+// FP64, and so does the test. 25,351 nodes: the relaxation 16 iterations instead of 176, the pressure 64
+// instead of 740, the solve 2.63 ms instead of 7.44; error against a 64-bit direct solve 2.5e-8 as
+// before. (degree, ratio) = (8, 64) 3.10 ms, (12, 144) 2.90, (16, 256) 2.63, (20, 400) 2.76, (28, 784) 2.75;
+// 2,760 nodes 1.80, 1.69, 1.54, 1.82, 1.52 ms, without it 3.95.
+constexpr int kCheb = 16;
+constexpr float kChebRatio = 256.0f;
+
+__device__ __forceinline__ void word32_store(unsigned long long* p, float v, unsigned epoch)
+{
+    const unsigned long long w = ((unsigned long long)epoch << 32) | __float_as_uint(v);
+    asm volatile("st.relaxed.gpu.global.b64 [%0], %1;" ::"l"(p), "l"(w) : "memory");
+}
+__device__ __forceinline__ unsigned long long word32_load(const unsigned long long* p)
+{
+    unsigned long long w;
+    asm volatile("ld.relaxed.gpu.global.b64 %0, [%1];" : "=l"(w) : "l"(p) : "memory");
+    return w;
+}
+
 // ---- any number of rows. CTA b owns the rows [n b / G, n (b + 1) / G) of every component; a warp
 // works on one component (wpc warps each), a lane on one row, so neighbouring lanes gather
 // neighbouring rows. kOne: at most one row per thread, so x, r, p, q and 1/diag stay in registers
-// for the whole solve; otherwise they live in global memory (touched by their thread alone). Only
-// z = r/diag is read by other CTAs: A p is carried along by q = A z + beta q, so p never travels.
-// kSmem: the CTA's slice of the matrix is staged in shared memory once.
+// for the whole solve; otherwise they live in global memory (touched by their thread alone). Only z
+// is read by other CTAs: A p is carried along by q = A z + beta q, so p never travels.
+// kSmem: the CTA's slice of the matrix is staged in shared memory once. With both (up to 29,184 rows of
+// the five components, 145,920 of the pressure alone) z = P(D^-1 r) as above, otherwise z = r/diag.
 // A sum goes over the CTA's lanes to one word per CTA; one warp of one CTA per value collects the
 // words, divides, and publishes the coefficient, which every CTA polls: two trips through L2. (All
 // CTAs polling all words is one trip, but 152 x 152 polls of the same few lines took 12 us per
@@ -424,6 +478,7 @@ struct CgShared {
     double r0[8], rr[8];
     unsigned active;             // components still iterating
     int stop, fail;
+    float ch[2][2 * kCheb + 1];  // per system: 1 / theta, then the two coefficients of every step
 };
 
 constexpr int kCgPoll = 5;   // words polled at once by a lane
@@ -507,13 +562,41 @@ __global__ void __launch_bounds__(kCgMaxThreads, 1) cg_kernel(const __grid_const
     const double* const gA = sys ? a.A1 : a.A0;
     double* const sA0 = reinterpret_cast<double*>(dyn);
     double* const sA1 = sA0 + (a.nv0 > 0 ? a.slice : 0);
-    int* const scol = reinterpret_cast<int*>(sA1 + (a.nc > a.nv0 ? a.slice : 0));
+    constexpr bool kPoly = kOne && kSmem;
+    double* const szd = sA1 + (a.nc > a.nv0 ? a.slice : 0);                 // kPoly: [nc][width] of z
+    int* const scol = reinterpret_cast<int*>(szd + (kPoly ? a.nc * a.width : 0));   // kPoly: indices into a z vector
+    float* const sF0 = reinterpret_cast<float*>(scol + a.slice);            // kPoly: the matrices in FP32
+    float* const sF1 = sF0 + (a.nv0 > 0 ? a.slice : 0);
+    float* const szf = sF1 + (a.nc > a.nv0 ? a.slice : 0);                  // kPoly: [nc][2][width] of the polynomial
+    int* const shalo = reinterpret_cast<int*>(szf + 2 * a.nc * a.width);    // kPoly: the other CTAs' rows read here
+    int halo = 0;
     if (kSmem) {
         const int m = a.row[hi] - base;
         for (int t = threadIdx.x; t < m; t += blockDim.x) {
             if (a.nv0 > 0) sA0[t] = a.A0[base + t];
             if (a.nc > a.nv0) sA1[t] = a.A1[base + t];
-            scol[t] = a.col[base + t];
+            scol[t] = kPoly ? a.lcol[base + t] : a.col[base + t];
+            if (kPoly) {
+                if (a.nv0 > 0) sF0[t] = (float)a.A0[base + t];
+                if (a.nc > a.nv0) sF1[t] = (float)a.A1[base + t];
+            }
+        }
+    }
+    if (kPoly) {
+        halo = a.halo_ptr[blockIdx.x + 1] - a.halo_ptr[blockIdx.x];
+        for (int t = threadIdx.x; t < halo; t += blockDim.x) shalo[t] = a.halo[a.halo_ptr[blockIdx.x] + t];
+    }
+    if (kPoly && threadIdx.x < 2) {
+        const float lmax = 1.01f * (threadIdx.x ? a.lmax1 : (a.nv0 > 0 ? *a.lmax0 : 1.0f)), lmin = lmax / kChebRatio;
+        const float theta = 0.5f * (lmax + lmin), delta = 0.5f * (lmax - lmin), sigma = theta / delta;
+        float* const ch = s.ch[threadIdx.x];
+        ch[0] = 1.0f / theta;
+        float rho = 1.0f / sigma;
+        for (int k = 0; k < kCheb; ++k) {
+            const float next = 1.0f / (2.0f * sigma - rho);
+            ch[1 + 2 * k] = next * rho;
+            ch[2 + 2 * k] = 2.0f * next / delta;
+            rho = next;
         }
     }
     if (threadIdx.x == 0) {
@@ -537,12 +620,51 @@ __global__ void __launch_bounds__(kCgMaxThreads, 1) cg_kernel(const __grid_const
                 ok = true;
 #pragma unroll
                 for (int u = 0; u < kW; ++u)
-                    zv[u] = t + u < re ? f(kSmem ? scol[t + u - base] : __ldg(a.col + t + u), ok) : 0.0;
+                    zv[u] = t + u < re ? f(kSmem && !kPoly ? scol[t + u - base] : __ldg(a.col + t + u), ok) : 0.0;
             } while (!ok && ++tries < kCgMaxTries);
             bad = bad || !ok;
 #pragma unroll
             for (int u = 0; u < kW; ++u)
                 if (t + u < re) sum = __fma_rn(kSmem ? sA[t + u - base] : __ldg(gA + t + u), zv[u], sum);
+        }
+        return sum;
+    };
+    // kPoly: fills the other CTAs' entries of a vector of the component (a thread at most every T-th, two at
+    // once, the last one in place of one that is not there), then waits for all of its threads
+    const int T = 32 * a.wpc, tid = 32 * sub + lane, width = a.width;
+    auto gather_halo = [&](auto&& load, auto&& good, auto&& put) {
+        for (int h = tid; h < halo; h += 2 * T) {
+            const int h1 = min(h + T, halo - 1), j0 = shalo[h], j1 = shalo[h1];
+            auto w0 = load(j0), w1 = load(j1);
+            int tries = bad ? kCgMaxTries : 0;
+            while (!(good(w0) && good(w1))) {
+                if (++tries >= kCgMaxTries) {
+                    bad = true;
+                    break;
+                }
+                w0 = load(j0);
+                w1 = load(j1);
+            }
+            put(hi - lo + h, w0);
+            put(hi - lo + h1, w1);
+        }
+        __syncwarp();
+        asm volatile("bar.sync %0, %1;" ::"r"(1 + c), "r"(T) : "memory");
+    };
+    // A times such a vector, eight entries of the row at once
+    auto row_dot_local = [&](auto zero, const auto* A, const auto* zl, int rs, int re) {
+        constexpr int kB = 8;
+        auto sum = zero;
+        for (int t = rs - base; t < re - base; t += kB) {
+            decltype(zero) zz[kB], aa[kB];
+#pragma unroll
+            for (int u = 0; u < kB; ++u) {
+                const int at = min(t + u, re - base - 1);
+                zz[u] = zl[scol[at]];
+                aa[u] = A[at];
+            }
+#pragma unroll
+            for (int u = 0; u < kB; ++u) sum = t + u < re - base ? fma(aa[u], zz[u], sum) : sum;
         }
         return sum;
     };
@@ -555,6 +677,35 @@ __global__ void __launch_bounds__(kCgMaxThreads, 1) cg_kernel(const __grid_const
     ulonglong2* const z = a.z + c * n;
     double* const st = a.state + 4 * c * n;
     const int first = task >= 0 ? hi : lo + 32 * sub + lane, stride = 32 * a.wpc;   // a task warp has no rows
+    unsigned epoch32 = a.epoch32;
+    double up = 1.0, down = 1.0;                   // kPoly: the scale of r and back
+    unsigned long long* const zf = a.zf + 2 * c * n;
+    const float* const sF = sys ? sF1 : sF0;
+    const bool mine = first < hi;
+    // kPoly: z = P(D^-1 r) of the thread's row, jz = its r / diag (all threads of the component take part;
+    // a fixed row's z stays 0)
+    auto polynomial = [&](double jz, float dinvf, int rs, int re) {
+        const float* const ch = s.ch[sys];
+        const float rt = (float)(jz * up);
+        float d = ch[0] * rt, z32 = d;
+#pragma unroll 1
+        for (int k = 0; k < kCheb; ++k) {
+            const unsigned ep = epoch32 + k;
+            unsigned long long* const w = zf + (k & 1) * n;
+            float* const zl = szf + (2 * c + (k & 1)) * width;
+            if (mine) {
+                word32_store(w + first, z32, ep);
+                zl[first - lo] = z32;
+            }
+            gather_halo([&](int j) { return word32_load(w + j); },
+                        [&](unsigned long long x) { return (unsigned)(x >> 32) == ep; },
+                        [&](int at, unsigned long long x) { zl[at] = __uint_as_float((unsigned)x); });
+            d = fmaf(ch[1 + 2 * k], d, ch[2 + 2 * k] * fmaf(-dinvf, row_dot_local(0.0f, sF, zl, rs, re), rt));
+            z32 += d;
+        }
+        epoch32 += kCheb;
+        return (double)z32 * down;
+    };
     // kOne: the row's state in registers
     double xv = 0.0, rv = 0.0, pv = 0.0, qv = 0.0, zv = 0.0, dinv = 0.0, sv = 0.0;
     int rs = 0, re = 0;
@@ -571,7 +722,7 @@ __global__ void __launch_bounds__(kCgMaxThreads, 1) cg_kernel(const __grid_const
         rv = fixed ? 0.0 : b[i] - row_dot(rs, re, [&](int j, bool&) { return x[j]; });
         dinv = 1.0 / diag[i];
         zv = rv * dinv;
-        word_store(z + i, zv, epoch);
+        if (!kPoly) word_store(z + i, zv, epoch);
         s0 += rv * zv;
         s1 += rv * rv;
         if (fixed) re = rs;   // its row of A p is zero
@@ -593,12 +744,34 @@ __global__ void __launch_bounds__(kCgMaxThreads, 1) cg_kernel(const __grid_const
         }
         __syncthreads();
         if (task >= 0) cg_exchange(a, s, task, nval, set, epoch, mode);
-        else if (kOne && ahead && first < hi) sv = row_dot(rs, re, zword);
+        else if (kPoly && ahead) {
+            double* const zl = szd + c * width;
+            if (mine) zl[first - lo] = zv;
+            gather_halo([&](int j) { return word_raw(z + j); }, [&](const ulonglong2& x) { return x.y == epoch; },
+                        [&](int at, const ulonglong2& x) { zl[at] = __longlong_as_double((long long)x.x); });
+            sv = row_dot_local(0.0, sA, zl, rs, re);
+        } else if (kOne && ahead && first < hi) sv = row_dot(rs, re, zword);
         if (bad) s.fail = 1;
         __syncthreads();
         return !s.fail;
     };
-    bool ok = exchange(3, 1, 0, true);
+    bool ok = exchange(3, 1, 0, !kPoly);
+    if (kPoly && ok) {
+        const double r0 = sqrt(s.res[2][c]);
+        if (r0 > 0.0 && r0 < 1e300) {
+            up = exp2(-(double)ilogb(r0));
+            down = 1.0 / up;
+        }
+        s0 = 0.0;
+        if (task < 0) {
+            zv = polynomial(zv, (float)dinv, rs, re);
+            if (mine) {
+                word_store(z + first, zv, epoch);
+                s0 = rv * zv;
+            }
+        }
+        ok = exchange(1, 0, 0, true);   // r.z into res[0]; r.r and |r_0|^2 stay in res[1], res[2]
+    }
     if (threadIdx.x < a.nc) {
         s.rz[threadIdx.x] = s.res[0][threadIdx.x];
         s.rr[threadIdx.x] = s.res[1][threadIdx.x];
@@ -652,9 +825,10 @@ __global__ void __launch_bounds__(kCgMaxThreads, 1) cg_kernel(const __grid_const
         if (on) {
             const double alpha = s.coef[c];
             if (kOne) {
+                rv = __fma_rn(-alpha, qv, rv);
+                zv = rv * dinv;
+                if (kPoly) zv = polynomial(zv, (float)dinv, rs, re);
                 if (first < hi) {
-                    rv = __fma_rn(-alpha, qv, rv);
-                    zv = rv * dinv;
                     word_store(z + first, zv, epoch);
                     s0 = rv * zv;
                     if (test) s1 = rv * rv;
@@ -704,7 +878,7 @@ __global__ void sum_kernel(const double* __restrict__ x, int n, double* __restri
     if (threadIdx.x == 0) part[blockIdx.x] = sh[0];
 }
 
-constexpr size_t kCgSmemMax = 96 * 1024;
+constexpr size_t kCgSmemMax = 96 * 1024, kCgPolySmemMax = 192 * 1024;
 
 // words of the partial sums (cg_small_kernel's, cg_kernel's with its published sums)
 size_t cg_slot_words(int ctas)
@@ -714,7 +888,7 @@ size_t cg_slot_words(int ctas)
 
 cudaError_t cg_configure()
 {
-    cudaError_t e = cudaFuncSetAttribute(cg_kernel<true, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kCgSmemMax);
+    cudaError_t e = cudaFuncSetAttribute(cg_kernel<true, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kCgPolySmemMax);
     if (e == cudaSuccess)
         e = cudaFuncSetAttribute(cg_kernel<false, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kCgSmemMax);
     return e;
@@ -1099,8 +1273,34 @@ cudaError_t fem_build(const double* node_xy, int N, const int32_t* tri, int E, c
     F->n_comp = n_comp;
     F->period = period;
     F->row_host = row;
-    for (int i = 0; i < ndof; ++i) F->max_deg = std::max(F->max_deg, row[i + 1] - row[i]);
+    for (int i = 0; i < ndof; ++i) {
+        double total = 0.0;
+        for (int t = row[i]; t < row[i + 1]; ++t) total += std::fabs(Kval[t]);
+        F->lmaxK = std::max(F->lmaxK, (float)(total / Kdiag[i]));
+    }
+    // cg_kernel's partition (one CTA per SM): every CTA's rows of others that its rows refer to, and the
+    // columns as indices into (its own rows, those)
     F->cg_ctas = sm_count();
+    const int parts = std::max(1, std::min(F->cg_ctas, (ndof + 31) / 32));
+    std::vector<int> halo_ptr(parts + 1, 0), halo, lcol(col.size()), local(ndof, -1);
+    for (int b = 0; b < parts; ++b) {
+        const int lo = (int)((int64_t)ndof * b / parts), hi = (int)((int64_t)ndof * (b + 1) / parts);
+        const size_t h0 = halo.size();
+        for (int t = row[lo]; t < row[hi]; ++t)
+            if ((col[t] < lo || col[t] >= hi) && local[col[t]] != b) {
+                local[col[t]] = b;
+                halo.push_back(col[t]);
+            }
+        std::sort(halo.begin() + h0, halo.end());
+        for (int t = row[lo]; t < row[hi]; ++t)
+            lcol[t] = col[t] >= lo && col[t] < hi
+                          ? col[t] - lo
+                          : hi - lo + (int)(std::lower_bound(halo.begin() + h0, halo.end(), col[t]) - halo.begin() - h0);
+        halo_ptr[b + 1] = (int)halo.size();
+        F->max_halo = std::max(F->max_halo, halo_ptr[b + 1] - halo_ptr[b]);
+    }
+    if (halo.empty()) halo.push_back(0);
+    for (int i = 0; i < ndof; ++i) F->max_deg = std::max(F->max_deg, row[i + 1] - row[i]);
     if (seg.empty()) {
         seg.assign(4, 0.0);
         segn.assign(2, 0);
@@ -1109,7 +1309,8 @@ cudaError_t fem_build(const double* node_xy, int N, const int32_t* tri, int E, c
     if ((e = upload(&F->dof, dof)) || (e = upload(&F->dof_node, dof_node)) || (e = upload(&F->edof, edof)) ||
         (e = upload(&F->area, area)) || (e = upload(&F->grad, grad)) || (e = upload(&F->de_ptr, de_ptr)) ||
         (e = upload(&F->de_el, de_el)) || (e = upload(&F->darea, darea)) || (e = upload(&F->row, row)) ||
-        (e = upload(&F->col, col)) || (e = upload(&F->cptr, cptr)) || (e = upload(&F->cel, cel)) ||
+        (e = upload(&F->col, col)) || (e = upload(&F->lcol, lcol)) || (e = upload(&F->halo_ptr, halo_ptr)) ||
+        (e = upload(&F->halo, halo)) || (e = upload(&F->cptr, cptr)) || (e = upload(&F->cel, cel)) ||
         (e = upload(&F->Mval, Mval)) || (e = upload(&F->Kval, Kval)) || (e = upload(&F->Kdiag, Kdiag)) || (e = upload(&F->wall, wall)) ||
         (e = upload(&F->normal, normal)) || (e = upload(&F->xy, xy)) || (e = upload(&F->seg, seg)) ||
         (e = upload(&F->segn, segn)) || (e = upload(&F->seg_off, seg_off)) || (e = upload(&F->ncomp, ncomp_v)) || (e = cudaMalloc((void**)&F->wdist, sizeof(double) * std::max(1, N))) ||
@@ -1122,6 +1323,9 @@ cudaError_t fem_build(const double* node_xy, int N, const int32_t* tri, int E, c
         (e = cudaMemset(F->cg_slots, 0, sizeof(ulonglong2) * cg_slot_words(F->cg_ctas))) ||
         (e = cudaMalloc((void**)&F->cg_z, sizeof(ulonglong2) * kCgComps * ((size_t)ndof + 255))) ||
         (e = cudaMemset(F->cg_z, 0, sizeof(ulonglong2) * kCgComps * ((size_t)ndof + 255))) ||
+        (e = cudaMalloc((void**)&F->cg_zf, sizeof(unsigned long long) * 2 * kCgComps * (size_t)ndof)) ||
+        (e = cudaMemset(F->cg_zf, 0, sizeof(unsigned long long) * 2 * kCgComps * (size_t)ndof)) ||
+        (e = cudaMalloc((void**)&F->lmax, sizeof(float))) ||
         (e = cudaMalloc((void**)&F->cg_out, sizeof(int) * kCgOut)) ||
         (e = cudaMallocHost((void**)&F->cg_host, sizeof(int) * kCgOut)) || (e = cg_configure())) {
         fem_free(F);
@@ -1134,8 +1338,8 @@ cudaError_t fem_build(const double* node_xy, int N, const int32_t* tri, int E, c
 void fem_free(Fem* F)
 {
     if (!F) return;
-    void* ps[] = {F->dof, F->dof_node, F->edof, F->area, F->grad, F->de_ptr, F->de_el, F->darea, F->row, F->col,
-                  F->cptr, F->cel, F->Mval, F->Kval, F->Kdiag, F->Aval, F->wall, F->normal, F->work, F->part, F->cg_slots, F->cg_z, F->cg_out,
+    void* ps[] = {F->dof, F->dof_node, F->edof, F->area, F->grad, F->de_ptr, F->de_el, F->darea, F->row, F->col, F->lcol, F->halo_ptr, F->halo,
+                  F->cptr, F->cel, F->Mval, F->Kval, F->Kdiag, F->Aval, F->wall, F->normal, F->work, F->part, F->cg_slots, F->cg_z, F->cg_zf, F->lmax, F->cg_out,
                   F->xy, F->seg, F->segn, F->seg_off, F->ncomp, F->wdist, F->wseg, F->wt};
     for (void* p : ps) cudaFree(p);
     cudaFreeHost(F->cg_host);
@@ -1171,12 +1375,32 @@ cudaError_t launch_cg(Fem& F, CgArgs& a, cudaStream_t st)
     int slice = 0;
     for (int b = 0; b < G; ++b)
         slice = std::max(slice, F.row_host[(int64_t)n * (b + 1) / G] - F.row_host[(int64_t)n * b / G]);
-    const size_t entry = sizeof(int) + sizeof(double) * ((a.nv0 > 0) + (a.nc > a.nv0));
-    const bool one = rows <= 32 * a.wpc, smem = slice * entry <= kCgSmemMax;
+    const bool one = rows <= 32 * a.wpc;
+    const int systems = (a.nv0 > 0) + (a.nc > a.nv0);
+    a.width = rows + F.max_halo;
+    size_t bytes = slice * (sizeof(int) + sizeof(double) * systems);
+    const size_t poly = bytes + slice * sizeof(float) * systems + a.nc * (size_t)a.width * 16 + sizeof(int) * (size_t)F.max_halo;
+    const bool smem = one ? poly <= kCgPolySmemMax && a.maxit < (1 << 24) : bytes <= kCgSmemMax;
+    if (one) bytes = poly;
+    if (one && smem) {
+        // the 8-byte words' epochs are 32 bits wide: start again from cleared words before they run out
+        const unsigned need = (unsigned)kCheb * ((unsigned)a.maxit + 2u);
+        if (F.cg_epoch32 > 0xffffffffu - need) {
+            const cudaError_t z = cudaMemsetAsync(F.cg_zf, 0, sizeof(unsigned long long) * 2 * kCgComps * (size_t)n, st);
+            if (z != cudaSuccess) return z;
+            F.cg_epoch32 = 1;
+        }
+        a.epoch32 = F.cg_epoch32;
+        F.cg_epoch32 += need;
+        a.zf = F.cg_zf;
+        a.lcol = F.lcol;
+        a.halo_ptr = F.halo_ptr;
+        a.halo = F.halo;
+    }
     a.slice = smem ? slice : 0;
     const void* fn = one ? (smem ? (const void*)cg_kernel<true, true> : (const void*)cg_kernel<true, false>)
                          : (smem ? (const void*)cg_kernel<false, true> : (const void*)cg_kernel<false, false>);
-    return cudaLaunchCooperativeKernel(fn, dim3(G), dim3(32 * (a.nc * a.wpc + kCgTasks)), args, smem ? slice * entry : 0, st);
+    return cudaLaunchCooperativeKernel(fn, dim3(G), dim3(32 * (a.nc * a.wpc + kCgTasks)), args, smem ? bytes : 0, st);
 }
 
 }  // namespace
@@ -1223,10 +1447,14 @@ cudaError_t node_fields_solve(Fem& F, const double* stats, const lpdf_params& P,
     a.tol = tol;
     a.maxit = maxit;
     a.z = F.cg_z;
+    a.lmax0 = F.lmax;
+    a.lmax1 = F.lmaxK;
     a.state = cgs;
     if (relax) {
         elem_L2_kernel<<<ge, 256, 0, st>>>(F, L2, ew);
-        assemble_kernel<<<gd, 256, 0, st>>>(F, ew, F.Aval, diag);
+        const cudaError_t e = cudaMemsetAsync(F.lmax, 0, sizeof(float), st);
+        if (e != cudaSuccess) return e;
+        assemble_kernel<<<gd, 256, 0, st>>>(F, ew, F.Aval, diag, F.lmax);
         const bool warm = P.cg_warm_start && F.has_wp;
         er_setup_kernel<<<gd, 256, 0, st>>>(F, eps, P.C0, tmp, wp, warm ? wp_prev : nullptr, xref);
         spmv_kernel<<<gd, 256, 0, st>>>(F, F.Mval, tmp, rhs, 0, 4);     // b = M wp^h
