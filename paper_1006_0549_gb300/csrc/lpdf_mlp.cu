@@ -139,7 +139,7 @@ __device__ __forceinline__ void get8(const unsigned char* src, int r, int k, int
     }
 }
 
-constexpr int kNetThreads = 512;
+constexpr int kNetThreads = 512, kLossThreads = 128;   // kTrain: the loss has threads of its own
 constexpr uint32_t kPackBytes = 2 * kPack, kXBytes = 2 * kH * kInP, kHBytes = 2 * kH * kH;
 
 // dynamic shared memory: the weight pack, then per group the inputs and the activations (one buffer
@@ -182,7 +182,8 @@ __device__ __forceinline__ float column_sums32(float* v, int lane)
 // MN-major, dZ overwrites the activations it came from, and the weight gradient and the next error
 // signal are issued together into the two halves of TMEM.
 template <int kGroups, bool kTrain>
-__global__ void __launch_bounds__(kNetThreads, 1) mlp_kernel(const float* __restrict__ feat, const float* __restrict__ tgt,
+__global__ void __launch_bounds__(kNetThreads + (kTrain ? kLossThreads : 0), 1)
+                                                  mlp_kernel(const float* __restrict__ feat, const float* __restrict__ tgt,
                                                              int64_t B, const float* __restrict__ P,
                                                              const __nv_bfloat16* __restrict__ pack,
                                                              const float* __restrict__ norm, float* __restrict__ out,
@@ -194,6 +195,7 @@ __global__ void __launch_bounds__(kNetThreads, 1) mlp_kernel(const float* __rest
     constexpr uint32_t kTmem = kTrain ? 256 : (kGroups == 1 ? 128 : 256);
     extern __shared__ __align__(1024) unsigned char dyn[];
     __shared__ float sb[3 * kH + kOutP], snorm[kNorm], wpart[4][kH];
+    __shared__ float sout[kTrain ? 2 : 1][kTrain ? kOut : 1][kTrain ? kH : 1];   // a tile's outputs, for the loss
     __shared__ unsigned long long wbar, gbar[kGroups];
     __shared__ uint32_t tmem_slot;
     const int g = threadIdx.x / GT, t = threadIdx.x - g * GT, warp = t >> 5, lane = t & 31;
@@ -205,7 +207,7 @@ __global__ void __launch_bounds__(kNetThreads, 1) mlp_kernel(const float* __rest
     unsigned char* const x = dyn + kPackBytes + g * (kXBytes + (kTrain ? 3 : 1) * kHBytes);
     unsigned char* const h[3] = {x + kXBytes, x + kXBytes + (kTrain ? kHBytes : 0), x + kXBytes + (kTrain ? 2 * kHBytes : 0)};
     auto sync = [&]() {
-        if (kGroups == 1) __syncthreads();
+        if (kGroups == 1 && !kTrain) __syncthreads();
         else asm volatile("bar.sync %0, %1;" ::"r"(g + 1), "n"(GT) : "memory");
     };
     if (threadIdx.x == 0) {
@@ -218,9 +220,9 @@ __global__ void __launch_bounds__(kNetThreads, 1) mlp_kernel(const float* __rest
         tc::tmem_alloc(&tmem_slot, kTmem);
         tc::tmem_relinquish();
     }
-    for (int i = threadIdx.x; i < 3 * kH + kOutP; i += kNetThreads)
+    for (int i = threadIdx.x; i < 3 * kH + kOutP; i += blockDim.x)
         sb[i] = P[i < kH ? ob1 + i : (i < 2 * kH ? ob2 - kH + i : (i < 3 * kH ? ob3 - 2 * kH + i : ob4 - 3 * kH + i))];
-    for (int i = threadIdx.x; i < kNorm; i += kNetThreads) snorm[i] = norm[i];
+    for (int i = threadIdx.x; i < kNorm; i += blockDim.x) snorm[i] = norm[i];
     tc::fence_before_sync();
     __syncthreads();
     tc::fence_after_sync();
@@ -249,7 +251,30 @@ __global__ void __launch_bounds__(kNetThreads, 1) mlp_kernel(const float* __rest
         tc::fence_after_sync();
     };
     const int64_t ntiles = (B + kH - 1) / kH;
-    for (int64_t tile = (int64_t)blockIdx.x * kGroups + g; tile < ntiles; tile += (int64_t)gridDim.x * kGroups) {
+    // the hand-over of a tile's outputs to the loss's threads; the two buffers used in turn
+    auto hand_over = [&]() { asm volatile("bar.sync 15, %0;" ::"n"(kNetThreads + kLossThreads) : "memory"); };
+    int turn = 0;
+    if (kTrain && threadIdx.x >= kNetThreads) {
+        // the loss of a row in FP64, beside the backward pass: 7 divisions of 600 cycles each held the
+        // network's warps up; 50 steps of 1024 rows 1.68 -> 1.53 ms (with the targets loaded ahead)
+        for (int64_t tile = blockIdx.x; tile < ntiles; tile += gridDim.x, turn ^= 1) {
+            const int64_t row = tile * kH + t;
+            double s = 0.0;
+            hand_over();
+#pragma unroll
+            for (int j = 0; j < kOut; ++j)
+                if (row < B) {
+                    const double y = ((double)tgt[row * kOut + j] - snorm[nTM + j]) / snorm[nTS + j];
+                    const double d = (double)sout[turn][j][t] - y;
+                    s += snorm[nW + j] * d * d;
+                }
+#pragma unroll
+            for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+            if (lane == 0) lpart[tile * kLossParts + warp] = s;
+        }
+    }
+    for (int64_t tile = kTrain && threadIdx.x >= kNetThreads ? ntiles : (int64_t)blockIdx.x * kGroups + g;
+         tile < ntiles; tile += (int64_t)gridDim.x * kGroups) {
         const int64_t row0 = tile * kH, row = row0 + r;
         const bool live = row < B;
         // the inputs: a thread standardises 2 (4) columns of a row; columns 8..15 are zero
@@ -282,9 +307,14 @@ __global__ void __launch_bounds__(kNetThreads, 1) mlp_kernel(const float* __rest
                 for (int j = 0; j < 32; j += 8) put8(h[l], r, c0 + j, kH, v + j);
             }
         }
+        float target[kOut];   // kTrain: loaded while the last GEMM runs
+        if (kTrain && cb == 0) {
+#pragma unroll
+            for (int j = 0; j < kOut; ++j) target[j] = live ? tgt[row * kOut + j] : 0.0f;
+        }
         gemms([&]() { tc::gemm_issue_op(tmem, tc::k_major(h[2], kH), tc::k_major(w4, kH), kOutP, 8, false, false); });
         unsigned char* const z4 = x + kXBytes + 3 * kHBytes;   // kTrain
-        if (cb == 0 || (kTrain && cb == 1)) {
+        if (cb == 0) {
             float v[16];
             tc::tmem_ld16(tmem + lanes, v);
             tc::wait_ld();
@@ -298,7 +328,9 @@ __global__ void __launch_bounds__(kNetThreads, 1) mlp_kernel(const float* __rest
                 if (live && out_user)
 #pragma unroll
                     for (int j = 0; j < kOut; ++j) out_user[row * kOut + j] = v[j] * snorm[nTS + j] + snorm[nTM + j];
-            } else if (cb == 0) {
+            } else {
+#pragma unroll
+                for (int j = 0; j < kOut; ++j) sout[turn][j][r] = v[j];
                 // dZ4 = d loss / d out: 2 (out - target) w_j / (7 B)
                 float s[32];
 #pragma unroll
@@ -306,29 +338,18 @@ __global__ void __launch_bounds__(kNetThreads, 1) mlp_kernel(const float* __rest
 #pragma unroll
                 for (int j = 0; j < kOut; ++j)
                     if (live) {
-                        const float y = (tgt[row * kOut + j] - snorm[nTM + j]) / snorm[nTS + j];
+                        const float y = (target[j] - snorm[nTM + j]) / snorm[nTS + j];
                         s[j] = 2.0f * (v[j] - y) * snorm[nW + j] / (float)(kOut * B);
                     }
                 put8(z4, r, 0, kOutP, s);
                 put8(z4, r, 8, kOutP, s + 8);
                 const float cs = column_sums32(s, lane);
                 if (lane < kOutP) wpart[quad][lane] = cs;
-            } else {
-                // the loss of the warp's rows in FP64
-                double s = 0.0;
-#pragma unroll
-                for (int j = 0; j < kOut; ++j)
-                    if (live) {
-                        const double y = ((double)tgt[row * kOut + j] - snorm[nTM + j]) / snorm[nTS + j];
-                        const double d = (double)v[j] - y;
-                        s += snorm[nW + j] * d * d;
-                    }
-#pragma unroll
-                for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
-                if (lane == 0) lpart[tile * kLossParts + quad] = s;
             }
         }
         if constexpr (kTrain) {
+            hand_over();
+            turn ^= 1;
             float* const pp = part + (size_t)tile * kPart;
             // a layer: dW^T of the layer above (its input as the rows, its dZ as the columns) into the
             // upper half of TMEM and dH = dZ W into the lower; then dZ = dH (1 - h^2) over h, the bias
@@ -546,7 +567,7 @@ cudaError_t launch_mlp_gradient(const float* feat, const float* tgt, int64_t B, 
 {
     if (B <= 0) return cudaSuccess;
     const int64_t tiles = (B + kH - 1) / kH;
-    mlp_kernel<1, true><<<(unsigned)std::min<int64_t>(tiles, sm_count()), kNetThreads, net_smem<1, true>(), st>>>(
+    mlp_kernel<1, true><<<(unsigned)std::min<int64_t>(tiles, sm_count()), kNetThreads + kLossThreads, net_smem<1, true>(), st>>>(
         feat, tgt, B, P, static_cast<const __nv_bfloat16*>(pack), norm, nullptr, nullptr, part, lpart, error);
     return cudaGetLastError();
 }
