@@ -295,9 +295,9 @@ cudaError_t mlp_configure();
 cudaError_t launch_mlp_forward(const float* feat, int64_t B, const float* P, const void* pack, const float* norm,
                                float* out, float* out_user, unsigned* error, cudaStream_t st);
 // forward and backward of a batch: gradient partials into part ((B + 127) / 128 x kPart) and losses
-// into lpart ((B + 127) / 128 x kLossParts)
+// into lpart ((B + 127) / 128 x kLossParts). follow: the stream's last launch is launch_mlp_reduce
 cudaError_t launch_mlp_gradient(const float* feat, const float* tgt, int64_t B, const float* P, const void* pack,
-                                const float* norm, float* part, double* lpart, unsigned* error, cudaStream_t st);
+                                const float* norm, float* part, double* lpart, unsigned* error, bool follow, cudaStream_t st);
 // the partials of a batch of B rows summed in tile order: the loss into loss[0]; with grad != NULL the
 // gradient into it, else an Adam step (number `step`) and the new pack
 cudaError_t launch_mlp_reduce(const float* part, const double* lpart, int64_t B, float* grad, float* P, float* m,

@@ -139,6 +139,45 @@ __device__ __forceinline__ void get8(const unsigned char* src, int r, int k, int
     }
 }
 
+// A training step's two kernels follow one another closely (programmatic dependent launch): each is
+// launched while its predecessor still runs, sets itself up, and waits here until that one has ended
+// (which itself began its work only when its own predecessor had, and so on); its successor may then be
+// set up in turn. 50 steps of 1024 rows 1.53 -> 1.29 ms. What the predecessor wrote is read by volatile loads below this point only: a plain
+// load through a const __restrict__ pointer could be moved above it.
+__device__ __forceinline__ void follow_grid()
+{
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+}
+__device__ __forceinline__ float load_after(const float* p)
+{
+    float v;
+    asm volatile("ld.global.f32 %0, [%1];" : "=f"(v) : "l"(p) : "memory");
+    return v;
+}
+__device__ __forceinline__ double load_after(const double* p)
+{
+    double v;
+    asm volatile("ld.global.f64 %0, [%1];" : "=d"(v) : "l"(p) : "memory");
+    return v;
+}
+template <class... P, class... A>
+cudaError_t launch_following(void (*kernel)(P...), unsigned grid, int threads, uint32_t smem, bool follow, cudaStream_t st,
+                             A... args)
+{
+    cudaLaunchConfig_t cfg{};
+    cfg.gridDim = dim3(grid);
+    cfg.blockDim = dim3((unsigned)threads);
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = st;
+    cudaLaunchAttribute at{};
+    at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at.val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = &at;
+    cfg.numAttrs = follow ? 1 : 0;
+    return cudaLaunchKernelEx(&cfg, kernel, static_cast<P>(args)...);
+}
+
 constexpr int kNetThreads = 512, kLossThreads = 128;   // kTrain: the loss has threads of its own
 constexpr uint32_t kPackBytes = 2 * kPack, kXBytes = 2 * kH * kInP, kHBytes = 2 * kH * kH;
 
@@ -213,15 +252,19 @@ __global__ void __launch_bounds__(kNetThreads + (kTrain ? kLossThreads : 0), 1)
     if (threadIdx.x == 0) {
         tc::mbar_init1(&wbar);
         for (int q = 0; q < kGroups; ++q) tc::mbar_init1(&gbar[q]);
-        mbar_expect_tx(&wbar, kPackBytes);
-        bulk_load(dyn, pack, kPackBytes, &wbar);
     }
     if (threadIdx.x < 32) {
         tc::tmem_alloc(&tmem_slot, kTmem);
         tc::tmem_relinquish();
     }
+    if (kTrain) follow_grid();   // the reduction that wrote P and pack, and read part and lpart
+    if (threadIdx.x == 0) {
+        asm volatile("fence.proxy.async.global;" ::: "memory");   // the pack was written by ordinary stores
+        mbar_expect_tx(&wbar, kPackBytes);
+        bulk_load(dyn, pack, kPackBytes, &wbar);
+    }
     for (int i = threadIdx.x; i < 3 * kH + kOutP; i += blockDim.x)
-        sb[i] = P[i < kH ? ob1 + i : (i < 2 * kH ? ob2 - kH + i : (i < 3 * kH ? ob3 - 2 * kH + i : ob4 - 3 * kH + i))];
+        sb[i] = load_after(P + (i < kH ? ob1 + i : (i < 2 * kH ? ob2 - kH + i : (i < 3 * kH ? ob3 - 2 * kH + i : ob4 - 3 * kH + i))));
     for (int i = threadIdx.x; i < kNorm; i += blockDim.x) snorm[i] = norm[i];
     tc::fence_before_sync();
     __syncthreads();
@@ -452,16 +495,17 @@ __global__ void mlp_reduce_kernel(const float* __restrict__ part, const double* 
                                   __nv_bfloat16* __restrict__ pack, double* __restrict__ loss)
 {
     __shared__ float corr[2];
+    if (threadIdx.x < 2 && !grad) corr[threadIdx.x] = 1.0f - powf(threadIdx.x ? b2 : b1, (float)step);
+    follow_grid();   // the kernel that wrote part and lpart
     if (blockIdx.x == gridDim.x - 1) {
         if (threadIdx.x >= 32) return;
         double s = 0.0;
-        for (int q = threadIdx.x; q < nparts * kLossParts; q += 32) s += lpart[q];
+        for (int q = threadIdx.x; q < nparts * kLossParts; q += 32) s += load_after(lpart + q);
 #pragma unroll
         for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
         if (threadIdx.x == 0) loss[0] = s / (double)(kOut * B);
         return;
     }
-    if (threadIdx.x < 2) corr[threadIdx.x] = 1.0f - powf(threadIdx.x ? b2 : b1, (float)step);
     __syncthreads();
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= kParams) return;
@@ -476,7 +520,7 @@ __global__ void mlp_reduce_kernel(const float* __restrict__ part, const double* 
     else src = gb4 + (i - ob4);
     double s = 0.0;
 #pragma unroll 8
-    for (int c = 0; c < nparts; ++c) s += part[(size_t)c * kPart + src];
+    for (int c = 0; c < nparts; ++c) s += load_after(part + (size_t)c * kPart + src);
     const float gi = (float)s;
     if (grad) {
         grad[i] = gi;
@@ -563,22 +607,21 @@ cudaError_t launch_mlp_forward(const float* feat, int64_t B, const float* P, con
 }
 
 cudaError_t launch_mlp_gradient(const float* feat, const float* tgt, int64_t B, const float* P, const void* pack,
-                                const float* norm, float* part, double* lpart, unsigned* error, cudaStream_t st)
+                                const float* norm, float* part, double* lpart, unsigned* error, bool follow, cudaStream_t st)
 {
     if (B <= 0) return cudaSuccess;
     const int64_t tiles = (B + kH - 1) / kH;
-    mlp_kernel<1, true><<<(unsigned)std::min<int64_t>(tiles, sm_count()), kNetThreads + kLossThreads, net_smem<1, true>(), st>>>(
-        feat, tgt, B, P, static_cast<const __nv_bfloat16*>(pack), norm, nullptr, nullptr, part, lpart, error);
-    return cudaGetLastError();
+    return launch_following(mlp_kernel<1, true>, (unsigned)std::min<int64_t>(tiles, sm_count()), kNetThreads + kLossThreads,
+                            net_smem<1, true>(), follow, st, feat, tgt, B, P, static_cast<const __nv_bfloat16*>(pack), norm,
+                            nullptr, nullptr, part, lpart, error);
 }
 
 cudaError_t launch_mlp_reduce(const float* part, const double* lpart, int64_t B, float* grad, float* P, float* m,
                               float* v, float lr, int step, void* pack, double* loss, cudaStream_t st)
 {
-    mlp_reduce_kernel<<<(kParams + 127) / 128 + 1, 128, 0, st>>>(part, lpart, (int)((B + kH - 1) / kH), B, grad, P, m, v,
-                                                                 lr, 0.9f, 0.999f, 1e-8f, step,
-                                                                 static_cast<__nv_bfloat16*>(pack), loss);
-    return cudaGetLastError();
+    return launch_following(mlp_reduce_kernel, (unsigned)((kParams + 127) / 128 + 1), 128, 0, true, st, part, lpart,
+                            (int)((B + kH - 1) / kH), B, grad, P, m, v, lr, 0.9f, 0.999f, 1e-8f, step,
+                            static_cast<__nv_bfloat16*>(pack), loss);
 }
 
 cudaError_t launch_mlp_pack(float* P, void* pack, cudaStream_t st)

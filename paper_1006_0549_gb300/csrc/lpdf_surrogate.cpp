@@ -202,7 +202,7 @@ int lpdf_mlp_gradient(lpdf_mlp* m, const float* feat, const float* tgt, int64_t 
         TRY(cudaMalloc((void**)&m->losses, sizeof(double) * 1));
         m->losses_cap = 1;
     }
-    TRY(launch_mlp_gradient(feat, tgt, B, m->P, m->pack, m->norm, m->part, m->lpart, m->error, st));
+    TRY(launch_mlp_gradient(feat, tgt, B, m->P, m->pack, m->norm, m->part, m->lpart, m->error, false, st));
     TRY(launch_mlp_reduce(m->part, m->lpart, B, m->grad, m->P, m->m, m->v, 0.0f, 0, m->pack, m->losses, st));
     std::vector<float> g(kParams);
     double l = 0.0;
@@ -233,7 +233,7 @@ int lpdf_mlp_train(lpdf_mlp* m, const float* feat, const float* tgt, int64_t B, 
         const int64_t off = (s % nchunk) * batch;
         const float* f = feat + off * kIn;
         const float* t = tgt + off * kOut;
-        TRY(launch_mlp_gradient(f, t, batch, m->P, m->pack, m->norm, m->part, m->lpart, m->error, st));
+        TRY(launch_mlp_gradient(f, t, batch, m->P, m->pack, m->norm, m->part, m->lpart, m->error, s > 0, st));
         TRY(launch_mlp_reduce(m->part, m->lpart, batch, nullptr, m->P, m->m, m->v, lr, ++m->step, m->pack,
                               m->losses + s, st));
     }
