@@ -516,35 +516,6 @@ __device__ __forceinline__ void bulk_store(void* dst, const void* src, uint32_t 
                  : "memory");
 }
 
-// Programmatic dependent launch: a kernel launched while its stream's predecessor still runs waits here
-// until that one has ended (which itself began its work only when its own predecessor
-// had, and so on); its own successor may then be set up in turn. What the predecessor wrote is read by
-// load_after below this point only: a plain load through a const __restrict__ pointer could be moved
-// above it. (What kernels before the predecessor wrote is there in any case.)
-__device__ __forceinline__ void follow_grid()
-{
-    asm volatile("griddepcontrol.wait;" ::: "memory");
-    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
-}
-__device__ __forceinline__ int load_after(const int* p)
-{
-    int v;
-    asm volatile("ld.global.s32 %0, [%1];" : "=r"(v) : "l"(p));
-    return v;
-}
-__device__ __forceinline__ float load_after(const float* p)
-{
-    float v;
-    asm volatile("ld.global.f32 %0, [%1];" : "=f"(v) : "l"(p));
-    return v;
-}
-__device__ __forceinline__ double load_after(const double* p)
-{
-    double v;
-    asm volatile("ld.global.f64 %0, [%1];" : "=d"(v) : "l"(p));
-    return v;
-}
-
 __device__ __forceinline__ void bulk_commit() { asm volatile("cp.async.bulk.commit_group;" ::: "memory"); }
 __device__ __forceinline__ void bulk_wait_read_all() { asm volatile("cp.async.bulk.wait_group.read 0;" ::: "memory"); }
 __device__ __forceinline__ void bulk_wait_all() { asm volatile("cp.async.bulk.wait_group 0;" ::: "memory"); }
@@ -635,6 +606,41 @@ __device__ __forceinline__ void particle_sources(const DevMesh& M, const StepPar
     else apply_sources<NS>(P, px, py, psi);
 }
 
+// Programmatic dependent launch: a kernel launched while its stream's predecessor still runs waits here
+// until that one has ended (which itself began its work only when its own predecessor
+// had, and so on); its own successor may then be set up in turn. What the predecessor wrote is read by
+// load_after below this point only: a plain load through a const __restrict__ pointer could be moved
+// above it. (What kernels before the predecessor wrote is there in any case.)
+__device__ __forceinline__ void follow_grid()
+{
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+}
+__device__ __forceinline__ int load_after(const int* p)
+{
+    int v;
+    asm volatile("ld.global.s32 %0, [%1];" : "=r"(v) : "l"(p));
+    return v;
+}
+__device__ __forceinline__ float load_after(const float* p)
+{
+    float v;
+    asm volatile("ld.global.f32 %0, [%1];" : "=f"(v) : "l"(p));
+    return v;
+}
+__device__ __forceinline__ double load_after(const double* p)
+{
+    double v;
+    asm volatile("ld.global.f64 %0, [%1];" : "=d"(v) : "l"(p));
+    return v;
+}
+__device__ __forceinline__ float4 load_after(const float4* p)
+{
+    float4 v;
+    asm volatile("ld.global.v4.f32 {%0, %1, %2, %3}, [%4];" : "=f"(v.x), "=f"(v.y), "=f"(v.z), "=f"(v.w) : "l"(p));
+    return v;
+}
+
 // Interpolated node fields at the particle, two sources:
 //   kElementTable = false: F is the node table (n_nodes x nfp); the P1 shape functions of the
 //                          element weight its three node rows;
@@ -652,7 +658,7 @@ __device__ __forceinline__ void interpolate_fields(const DevMesh& M, const float
         const float4* R = reinterpret_cast<const float4*>(F) + (size_t)e * (3 * NFP / 4);
 #pragma unroll
         for (int q = 0; q < NFP / 4; ++q) {
-            const float4 a = __ldg(R + q), gx = __ldg(R + NFP / 4 + q), gy = __ldg(R + 2 * (NFP / 4) + q);
+            const float4 a = load_after(R + q), gx = load_after(R + NFP / 4 + q), gy = load_after(R + 2 * (NFP / 4) + q);
             Fi[4 * q + 0] = fmaf(gx.x, dx, fmaf(gy.x, dy, a.x));
             Fi[4 * q + 1] = fmaf(gx.y, dx, fmaf(gy.y, dy, a.y));
             Fi[4 * q + 2] = fmaf(gx.z, dx, fmaf(gy.z, dy, a.z));

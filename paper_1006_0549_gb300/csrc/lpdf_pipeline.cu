@@ -209,6 +209,7 @@ advance_kernel(const __grid_constant__ DevMesh M, const __grid_constant__ Partic
                const __grid_constant__ StepParams P, unsigned long long* __restrict__ status,
                unsigned* __restrict__ tiles)
 {
+    follow_grid();
     const int lane = threadIdx.x & 31;
     unsigned err = 0;
     int hops = 0;
@@ -256,6 +257,7 @@ __global__ void element_fields_kernel(const __grid_constant__ DevMesh M, const f
                                       unsigned long long* __restrict__ flux, int64_t nf)
 {
     constexpr int NFP = (22 + NS + 3) / 4 * 4, NQ4 = NFP / 4;
+    follow_grid();
     const int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x, nt = (int64_t)gridDim.x * blockDim.x;
     for (int64_t i = t; i < nk; i += nt) kwork[i] = 0;
     for (int64_t i = t; i < na; i += nt) acc[i] = 0ull;
@@ -1330,9 +1332,9 @@ __global__ void step_counter_kernel(unsigned long long* __restrict__ c, unsigned
 inline unsigned nblocks(int64_t n, int t) { return (unsigned)((n + t - 1) / t); }
 
 // A launch that does not wait for its predecessor's end (the kernel does: follow_grid): 1-2 us less per
-// launch. A step of 50,000 particles 42 -> 38 us, of 3M (compensated) 264 -> 248, of 25M 1103 -> 1078. T and
-// K1 stay ordinary launches: they read the caller's fields and T's rows through the read-only path,
-// and what any later kernel reads of the kernels before its predecessor is there because of that.
+// launch. A step of 50,000 particles 42 -> 36 us, of 3M (compensated) 264 -> 245, of 25M 1103 -> 1075. T
+// stays an ordinary launch: it reads the caller's fields through the read-only path, and it makes
+// everything of the steps before visible to the kernels after it.
 template <class... P, class... A>
 void launch_follow(void (*kernel)(P...), dim3 grid, int threads, cudaStream_t st, A... args)
 {
@@ -1384,8 +1386,7 @@ void launch_advance_v(const DevMesh& m, const Particles& cur, const Particles& n
 {
     const int64_t ntiles = (cur.n + ABLK - 1) / ABLK;
     const int64_t grid = kGrid ? std::min<int64_t>(ntiles, (int64_t)sm_count_cached() * MINB) : ntiles;
-    advance_kernel<NS, kKind, ABLK, MINB, kGrid>
-        <<<(unsigned)grid, ABLK, 0, st>>>(m, cur, nxt, perm, ef, p, status, tiles);
+    launch_follow(advance_kernel<NS, kKind, ABLK, MINB, kGrid>, (unsigned)grid, ABLK, st, m, cur, nxt, perm, ef, p, status, tiles);
 }
 
 template <int NS, int kKind>
