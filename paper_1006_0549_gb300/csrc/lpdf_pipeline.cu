@@ -26,6 +26,8 @@
 //       particles; 1, per lane the sums of q, dx q and dy q ((dx, dy) from vertex 0) in
 //       compensated FP32 (double-floats), combined in FP64 with the element's FP64 affine
 //       barycentric coefficients.
+// H to S4 are one cluster launch for a small ensemble (rebucket_small_kernel). T also zeroes the step's
+// counters and sums. The kernels after T are set up while their predecessors still run (launch_follow).
 // Every step leaves perm_new as the next step's perm, so the ensemble is re-bucketed by element
 // every step without a separate sort, and the reduction never needs a hash or a binning pass.
 #include <algorithm>

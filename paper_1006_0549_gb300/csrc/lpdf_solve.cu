@@ -8,7 +8,7 @@
 //   * G_ij from elliptic relaxation (the paragraph after Eq. 4): P1 finite elements for
 //     wp_ij - L^2 lap wp_ij = -3/4 C0 eps delta_ij with wall values wp_ij = -4.5 eps n_i n_j,
 //     L = CL max(k^1.5/eps, Ceta nu^0.75/eps^0.25) (L^2 averaged over each element's nodes),
-//     solved by a Jacobi-preconditioned conjugate gradient in FP64 on the four components at
+//     solved by a conjugate gradient in FP64 (Jacobi, or a polynomial in it) on the four components at
 //     once; G_ij = (wp_ij - eps delta_ij/2)/k and C0 eps = -2/3 (eps + <u_i u_j> G_ij) (the
 //     k-consistency condition), or the simplified Langevin model;
 //   * mean pressure (optional; Section "Governing equations", the projection on the grid): weak
