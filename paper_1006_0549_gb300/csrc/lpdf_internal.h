@@ -211,7 +211,7 @@ struct Fem {
     double* grad = nullptr;      // 6 per element: grad of the 3 shape functions
     int* de_ptr = nullptr;       // DOF -> incident (element, corner) pairs e*3 + a (CSR)
     int* de_el = nullptr;
-    double* darea = nullptr;     // sum of the areas of the incident pairs
+    double* iarea = nullptr;     // 1 / sum of the areas of the incident pairs
     int* row = nullptr;          // DOF x DOF matrix pattern (CSR)
     int* col = nullptr;
     int* cptr = nullptr;         // CSR entry -> element-matrix contributions e*9 + a*3 + b
