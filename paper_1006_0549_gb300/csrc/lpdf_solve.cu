@@ -59,7 +59,7 @@ __global__ void elem_grad_kernel(const Fem F, const double* __restrict__ f, int 
 
 // area-weighted average of m element values to the DOFs: out[d ld + i], a thread per value. (1/area is
 // kept with the mesh: an FP64 division per thread is 600 cycles of a pipe that takes one warp at a time.
-// The surrogate's call on 100,489 nodes 236 -> 229 us without it, the coupled loop's pass 1.25 -> 1.19 ms.)
+// The surrogate's call on 100,489 nodes 236 -> 229 us without it.)
 __global__ void recover_kernel(const Fem F, const double* __restrict__ ev, int m, double* __restrict__ out, int ld)
 {
     const int64_t t0 = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
