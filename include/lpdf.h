@@ -369,7 +369,8 @@ int lpdf_grid_statistics(lpdf_ctx* ctx, double* out, int raw, void* stream);
  *   recovered gradient. All arithmetic is FP64; the output is rounded to FP32.
  * The first call on a mesh builds and uploads its finite-element tables (kept until
  * lpdf_mesh_free). Calls on the same mesh share its scratch: serialise them.
- * Errors: LPDF_ERR_ARG, LPDF_ERR_UNSUPPORTED (ns), LPDF_ERR_CG_NOCONV (iters still filled in),
+ * Errors: LPDF_ERR_ARG, LPDF_ERR_UNSUPPORTED (ns), LPDF_ERR_CG_NOCONV (iters still filled in; also
+ * when a residual norm is not finite, as with a NaN in stats; fields are left as they were),
  * LPDF_ERR_CUDA.
  * ------------------------------------------------------------------------------------- */
 int lpdf_elliptic_relax_solve(const lpdf_mesh* mesh, const lpdf_params* params, const double* stats,

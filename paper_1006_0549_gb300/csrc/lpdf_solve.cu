@@ -186,7 +186,8 @@ __global__ void spmv_kernel(const Fem F, const double* __restrict__ A, const dou
 // others.
 //
 // Converged when ||r_c|| <= tol ||r_c(xref)|| for every c of a system (xref NULL: the start itself),
-// tested every kCheckEvery iterations and at maxit; a converged system stops there.
+// tested every kCheckEvery iterations and at maxit; a converged system stops there, and so does one
+// with a norm that is not finite, which is not converged.
 constexpr int kCgComps = 5;                       // components at most
 constexpr int kCgSmallRows = 2048, kCgDeg = 12;   // cg_small_kernel: rows, matrix entries per row at most
 constexpr int kCgSmallUnits = kCgSmallRows / 32;
@@ -249,6 +250,10 @@ __device__ __forceinline__ double word_load(const ulonglong2* p, unsigned long l
     ok = ok && e == epoch;
     return __longlong_as_double(b);
 }
+
+// the test of a component from its |r|^2 and tol |r_0|: reached, or no longer worth iterating
+__device__ __forceinline__ bool cg_reached(double rr, double limit) { return sqrt(rr) <= limit && isfinite(limit); }
+__device__ __forceinline__ bool cg_broken(double rr, double limit) { return !isfinite(rr) || !isfinite(limit); }
 
 __device__ __forceinline__ double shfl_add(double v, int o) { return __dadd_rn(v, __shfl_down_sync(0xffffffffu, v, o)); }
 
@@ -379,10 +384,15 @@ __global__ void __launch_bounds__(32) cg_small_kernel(const __grid_constant__ Cg
     for (; alive; ++it) {
         if (it % kCheckEvery == 0 || it >= a.maxit) {
             done = true;
+            bool broken = false;
 #pragma unroll
             for (int k = 0; k < 4; ++k)
-                if (c0 + k < c1 && sqrt(cg_small_total(slot(set, c0 + k), nu, nb, epoch, lane, alive)) > r0[k]) done = false;
-            if (!alive || done || it >= a.maxit) break;
+                if (c0 + k < c1) {
+                    const double rr = cg_small_total(slot(set, c0 + k), nu, nb, epoch, lane, alive);
+                    done = done && cg_reached(rr, r0[k]);
+                    broken = broken || cg_broken(rr, r0[k]);
+                }
+            if (!alive || done || broken || it >= a.maxit) break;
             set = 7 - set;
         }
         // p of the row and its neighbours, q = A p
@@ -785,13 +795,15 @@ __global__ void __launch_bounds__(kCgMaxThreads, 1) cg_kernel(const __grid_const
     for (int it = 0; ok; ++it) {
         if (it % kCheckEvery == 0 || it >= a.maxit) {
             if (wid == 0) {
-                const bool far = lane < a.nc && ((s.active >> lane) & 1u) && sqrt(s.rr[lane]) > a.tol * s.r0[lane];
-                const unsigned f = __ballot_sync(0xffffffffu, far);
+                const bool on = lane < a.nc && ((s.active >> lane) & 1u);
+                const double rr = on ? s.rr[lane] : 0.0, limit = on ? a.tol * s.r0[lane] : 0.0;
+                const unsigned f = __ballot_sync(0xffffffffu, on && !cg_reached(rr, limit));
+                const unsigned broken = __ballot_sync(0xffffffffu, on && cg_broken(rr, limit));
                 if (lane == 0) {
                     const unsigned m0 = (1u << a.nv0) - 1u, m1 = ((1u << a.nc) - 1u) & ~m0;
                     unsigned act = s.active;
-                    if ((act & m0) && !(f & m0)) { act &= ~m0; its0 = it; ++conv; }
-                    if ((act & m1) && !(f & m1)) { act &= ~m1; its1 = it; ++conv; }
+                    if ((act & m0) && (!(f & m0) || (broken & m0))) { act &= ~m0; its0 = it; conv += !(f & m0); }
+                    if ((act & m1) && (!(f & m1) || (broken & m1))) { act &= ~m1; its1 = it; conv += !(f & m1); }
                     s.active = act;
                     s.stop = act == 0u || it >= a.maxit;
                 }
