@@ -234,11 +234,10 @@ struct Fem {
     int max_halo = 0;
     void* cg_slots = nullptr;
     ulonglong2* cg_z = nullptr;
-    unsigned long long* cg_zf = nullptr;   // the preconditioner's 8-byte words, and their epochs
-    unsigned cg_epoch32 = 1;
-    float* lmax = nullptr;       // bounds of the spectra of D^-1 A (device) and D^-1 K
-    float lmaxK = 0.0f;
-    unsigned long long cg_epoch = 1;
+    ulonglong2* cg_zp = nullptr;           // the preconditioner's words
+    double* lmax = nullptr;      // bounds of the spectra of D^-1 A (device) and D^-1 K
+    double lmaxK = 0.0;
+    unsigned long long cg_epoch = 1, cg_epochp = 1;
     int* cg_out = nullptr;
     int* cg_host = nullptr;      // pinned copy
     std::vector<int> row_host;   // the matrix pattern's row starts

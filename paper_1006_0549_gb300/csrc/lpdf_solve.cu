@@ -128,11 +128,11 @@ __global__ void elem_L2_kernel(const Fem F, const double* __restrict__ L2, doubl
 // A = M + sum_e L2_e K_e (fixed contribution order per CSR entry); diag = its diagonal
 // (and the largest row sum of |D^-1 A| of the rows that are solved for, a bound of its spectrum)
 __global__ void assemble_kernel(const Fem F, const double* __restrict__ L2e, double* __restrict__ A,
-                                double* __restrict__ diag, float* __restrict__ lmax)
+                                double* __restrict__ diag, double* __restrict__ lmax)
 {
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= F.ndof) return;
-    float total = 0.0f;
+    double total = 0.0;
     for (int j = F.row[i]; j < F.row[i + 1]; ++j) {
         double s = 0.0;
         for (int t = F.cptr[j]; t < F.cptr[j + 1]; ++t) {
@@ -142,11 +142,11 @@ __global__ void assemble_kernel(const Fem F, const double* __restrict__ L2e, dou
             s += L2e[e] * (F.area[e] * (g[2 * a] * g[2 * b] + g[2 * a + 1] * g[2 * b + 1]));
         }
         A[j] = F.Mval[j] + s;
-        total += fabsf((float)A[j]);
+        total += fabs(A[j]);
         if (F.col[j] == i) diag[i] = A[j];
     }
-    // positive floats compare like their bits
-    if (!F.wall[i]) atomicMax(reinterpret_cast<int*>(lmax), __float_as_int(total / (float)diag[i]));
+    // positive values compare like their bits
+    if (!F.wall[i]) atomicMax(reinterpret_cast<long long*>(lmax), __double_as_longlong(total / diag[i]));
 }
 
 // ---------------------------------------------------------------- batched PCG
@@ -192,6 +192,8 @@ constexpr int kCgComps = 5;                       // components at most
 constexpr int kCgSmallRows = 2048, kCgDeg = 12;   // cg_small_kernel: rows, matrix entries per row at most
 constexpr int kCgSmallUnits = kCgSmallRows / 32;
 constexpr int kCgMaxThreads = 1024;               // cg_kernel
+constexpr int kCheb = 16;                         // its polynomial's degree and range (below)
+constexpr double kChebRatio = 256.0;
 constexpr int kCgMaxTries = 1 << 21;              // polls (of about 0.2 us) before a wait gives up
 enum { kCgIts0 = 0, kCgIts1 = 1, kCgOk = 2, kCgError = 3, kCgOut = 4 };   // kCgOk: systems converged
 
@@ -205,13 +207,13 @@ struct CgArgs {
     double* state;                          // 4 nc n (r, p, q, 1/diag of cg_kernel with several rows per thread)
     const int *lcol, *halo_ptr, *halo;      // cg_kernel: see Fem
     int width;                              // its rows and halo, at most
-    const float* lmax0;                     // bounds of the spectra of D^-1 A (device) and D^-1 K
-    float lmax1;
+    const double* lmax0;                    // bounds of the spectra of D^-1 A (device) and D^-1 K
+    double lmax1;
+    double cheb[2 * kCheb + 1];             // for a spectrum up to 1: 1 / theta, then the two coefficients of every step
     double tol;
-    unsigned long long epoch;
-    unsigned epoch32;                       // of the 8-byte words zf
+    unsigned long long epoch, epochp;       // of z and the partial sums, of zp
     ulonglong2 *z, *slots;                  // nc n words; the partial sums' words
-    unsigned long long* zf;                 // 2 nc n words
+    ulonglong2* zp;                         // 2 nc n words
     int* out;
 };
 
@@ -441,33 +443,19 @@ __global__ void __launch_bounds__(32) cg_small_kernel(const __grid_constant__ Cg
 
 // The preconditioner of cg_kernel with one row per thread and the matrix in shared memory: kCheb steps of
 // the Chebyshev iteration for D^-1 A z = D^-1 r on [lmax / kChebRatio, lmax] (Golub & Varga 1961), lmax a
-// Gershgorin bound: a fixed symmetric positive polynomial in D^-1 A, in FP32. A step has no sum over the
-// grid and no FP64: a CTA stores its rows' z as 8-byte words (value, epoch), polls the words of its halo
-// (the other CTAs' rows that its rows refer to) into shared memory, and gathers from there after a barrier
-// of the component's warps. What bounds it is that trip through L2: 1.3 us a step, while an FP64
-// iteration with its two grid sums takes 7. (Every thread polling its row's columns itself, up to ten
-// words, took 3 us: 30 warps x 10 uncoalesced loads a try.) Two buffers are used in turn: a thread
-// overwrites what it stored two steps ago, which its neighbours' CTAs read before they stored what its
-// own has read since; the pattern is symmetric. r is scaled by a power of two near 1/|r_0| first. What
-// FP32 rounds away changes the search directions a little, not the residual or the solution: those stay
-// FP64, and so does the test. 25,351 nodes: the relaxation 16 iterations instead of 176, the pressure 64
-// instead of 740, the solve 2.63 ms instead of 7.44; error against a 64-bit direct solve 2.5e-8 as
-// before. (degree, ratio) = (8, 64) 3.10 ms, (12, 144) 2.90, (16, 256) 2.63, (20, 400) 2.76, (28, 784) 2.75;
-// 2,760 nodes 1.80, 1.69, 1.54, 1.82, 1.52 ms, without it 3.95.
-constexpr int kCheb = 16;
-constexpr float kChebRatio = 256.0f;
-
-__device__ __forceinline__ void word32_store(unsigned long long* p, float v, unsigned epoch)
-{
-    const unsigned long long w = ((unsigned long long)epoch << 32) | __float_as_uint(v);
-    asm volatile("st.relaxed.gpu.global.b64 [%0], %1;" ::"l"(p), "l"(w) : "memory");
-}
-__device__ __forceinline__ unsigned long long word32_load(const unsigned long long* p)
-{
-    unsigned long long w;
-    asm volatile("ld.relaxed.gpu.global.b64 %0, [%1];" : "=l"(w) : "l"(p) : "memory");
-    return w;
-}
+// Gershgorin bound: a fixed symmetric positive polynomial in D^-1 A. A step has no sum over the grid: a
+// CTA stores its rows' z as words, polls the words of its halo (the other CTAs' rows that its rows refer
+// to) into shared memory, and gathers from there after a barrier of the component's warps. What bounds it
+// is that trip through L2 and the FP64 pipe (a dozen instructions of 65 cycles a warp): 2.4 us a step
+// with the pressure alone at work, 6.5 with all five components. (Every thread polling its row's columns
+// itself, up to ten words, was twice as slow.) Two buffers are used in turn: a thread overwrites what it
+// stored two steps ago, which its neighbours' CTAs read before they stored what its own has read since;
+// the pattern is symmetric. 25,351 nodes: the relaxation 16 iterations instead of 176, the pressure 64
+// instead of 740, the solve 3.94 ms instead of 7.44; error against a 64-bit direct solve 2.5e-8 as before.
+// In FP32 the solve took 2.65 ms, but the matrix overflows from a relaxation length of 2e19 on, and the
+// call computes in FP64. (degree, ratio) = (8, 64) 4.41 ms, (12, 144) 4.37, (14, 196) 3.88, (16, 256) 3.94,
+// (20, 400) 4.28; 2,976 nodes 2.31, 2.27, 2.23, 2.47, 2.51 ms, without it 3.95; 112,000 nodes, the pressure
+// alone 11.2, 10.9, 10.6, 10.4, 10.2 ms.
 
 // ---- any number of rows. CTA b owns the rows [n b / G, n (b + 1) / G) of every component; a warp
 // works on one component (wpc warps each), a lane on one row, so neighbouring lanes gather
@@ -490,7 +478,7 @@ struct CgShared {
     double r0[8], rr[8];
     unsigned active;             // components still iterating
     int stop, fail;
-    float ch[2][2 * kCheb + 1];  // per system: 1 / theta, then the two coefficients of every step
+    double il[2];                // per system: 1 / the bound of its spectrum
 };
 
 constexpr int kCgPoll = 5;   // words polled at once by a lane
@@ -575,12 +563,9 @@ __global__ void __launch_bounds__(kCgMaxThreads, 1) cg_kernel(const __grid_const
     double* const sA0 = reinterpret_cast<double*>(dyn);
     double* const sA1 = sA0 + (a.nv0 > 0 ? a.slice : 0);
     constexpr bool kPoly = kOne && kSmem;
-    double* const szd = sA1 + (a.nc > a.nv0 ? a.slice : 0);                 // kPoly: [nc][width] of z
-    int* const scol = reinterpret_cast<int*>(szd + (kPoly ? a.nc * a.width : 0));   // kPoly: indices into a z vector
-    float* const sF0 = reinterpret_cast<float*>(scol + a.slice);            // kPoly: the matrices in FP32
-    float* const sF1 = sF0 + (a.nv0 > 0 ? a.slice : 0);
-    float* const szf = sF1 + (a.nc > a.nv0 ? a.slice : 0);                  // kPoly: [nc][2][width] of the polynomial
-    int* const shalo = reinterpret_cast<int*>(szf + 2 * a.nc * a.width);    // kPoly: the other CTAs' rows read here
+    double* const sz = sA1 + (a.nc > a.nv0 ? a.slice : 0);                  // kPoly: [nc][2][width] of z
+    int* const scol = reinterpret_cast<int*>(sz + (kPoly ? 2 * a.nc * a.width : 0));   // kPoly: indices into a z vector
+    int* const shalo = scol + a.slice;                                      // kPoly: the other CTAs' rows read here
     int halo = 0;
     if (kSmem) {
         const int m = a.row[hi] - base;
@@ -588,29 +573,14 @@ __global__ void __launch_bounds__(kCgMaxThreads, 1) cg_kernel(const __grid_const
             if (a.nv0 > 0) sA0[t] = a.A0[base + t];
             if (a.nc > a.nv0) sA1[t] = a.A1[base + t];
             scol[t] = kPoly ? a.lcol[base + t] : a.col[base + t];
-            if (kPoly) {
-                if (a.nv0 > 0) sF0[t] = (float)a.A0[base + t];
-                if (a.nc > a.nv0) sF1[t] = (float)a.A1[base + t];
-            }
         }
     }
     if (kPoly) {
         halo = a.halo_ptr[blockIdx.x + 1] - a.halo_ptr[blockIdx.x];
         for (int t = threadIdx.x; t < halo; t += blockDim.x) shalo[t] = a.halo[a.halo_ptr[blockIdx.x] + t];
     }
-    if (kPoly && threadIdx.x < 2) {
-        const float lmax = 1.01f * (threadIdx.x ? a.lmax1 : (a.nv0 > 0 ? *a.lmax0 : 1.0f)), lmin = lmax / kChebRatio;
-        const float theta = 0.5f * (lmax + lmin), delta = 0.5f * (lmax - lmin), sigma = theta / delta;
-        float* const ch = s.ch[threadIdx.x];
-        ch[0] = 1.0f / theta;
-        float rho = 1.0f / sigma;
-        for (int k = 0; k < kCheb; ++k) {
-            const float next = 1.0f / (2.0f * sigma - rho);
-            ch[1 + 2 * k] = next * rho;
-            ch[2 + 2 * k] = 2.0f * next / delta;
-            rho = next;
-        }
-    }
+    if (kPoly && threadIdx.x < 2)
+        s.il[threadIdx.x] = 1.0 / (1.01 * (threadIdx.x ? a.lmax1 : (a.nv0 > 0 ? *a.lmax0 : 1.0)));
     if (threadIdx.x == 0) {
         s.active = (1u << a.nc) - 1u;
         s.stop = 0;
@@ -644,36 +614,35 @@ __global__ void __launch_bounds__(kCgMaxThreads, 1) cg_kernel(const __grid_const
     // kPoly: fills the other CTAs' entries of a vector of the component (a thread at most every T-th, two at
     // once, the last one in place of one that is not there), then waits for all of its threads
     const int T = 32 * a.wpc, tid = 32 * sub + lane, width = a.width;
-    auto gather_halo = [&](auto&& load, auto&& good, auto&& put) {
+    auto gather_halo = [&](const ulonglong2* words, unsigned long long ep, double* zl) {
         for (int h = tid; h < halo; h += 2 * T) {
             const int h1 = min(h + T, halo - 1), j0 = shalo[h], j1 = shalo[h1];
-            auto w0 = load(j0), w1 = load(j1);
+            ulonglong2 w0 = word_raw(words + j0), w1 = word_raw(words + j1);
             int tries = bad ? kCgMaxTries : 0;
-            while (!(good(w0) && good(w1))) {
+            while (w0.y != ep || w1.y != ep) {
                 if (++tries >= kCgMaxTries) {
                     bad = true;
                     break;
                 }
-                w0 = load(j0);
-                w1 = load(j1);
+                w0 = word_raw(words + j0);
+                w1 = word_raw(words + j1);
             }
-            put(hi - lo + h, w0);
-            put(hi - lo + h1, w1);
+            zl[hi - lo + h] = __longlong_as_double((long long)w0.x);
+            zl[hi - lo + h1] = __longlong_as_double((long long)w1.x);
         }
         __syncwarp();
         asm volatile("bar.sync %0, %1;" ::"r"(1 + c), "r"(T) : "memory");
     };
-    // A times such a vector, eight entries of the row at once
-    auto row_dot_local = [&](auto zero, const auto* A, const auto* zl, int rs, int re) {
+    // sum + A times such a vector, eight entries of the row at once
+    auto row_dot_local = [&](double sum, const double* zl, int rs, int re) {
         constexpr int kB = 8;
-        auto sum = zero;
         for (int t = rs - base; t < re - base; t += kB) {
-            decltype(zero) zz[kB], aa[kB];
+            double zz[kB], aa[kB];
 #pragma unroll
             for (int u = 0; u < kB; ++u) {
                 const int at = min(t + u, re - base - 1);
                 zz[u] = zl[scol[at]];
-                aa[u] = A[at];
+                aa[u] = sA[at];
             }
 #pragma unroll
             for (int u = 0; u < kB; ++u) sum = t + u < re - base ? fma(aa[u], zz[u], sum) : sum;
@@ -689,34 +658,29 @@ __global__ void __launch_bounds__(kCgMaxThreads, 1) cg_kernel(const __grid_const
     ulonglong2* const z = a.z + c * n;
     double* const st = a.state + 4 * c * n;
     const int first = task >= 0 ? hi : lo + 32 * sub + lane, stride = 32 * a.wpc;   // a task warp has no rows
-    unsigned epoch32 = a.epoch32;
-    double up = 1.0, down = 1.0;                   // kPoly: the scale of r and back
-    unsigned long long* const zf = a.zf + 2 * c * n;
-    const float* const sF = sys ? sF1 : sF0;
+    unsigned long long epochp = a.epochp;
+    ulonglong2* const zp = a.zp + 2 * c * n;
     const bool mine = first < hi;
-    // kPoly: z = P(D^-1 r) of the thread's row, jz = its r / diag (all threads of the component take part;
-    // a fixed row's z stays 0)
-    auto polynomial = [&](double jz, float dinvf, int rs, int re) {
-        const float* const ch = s.ch[sys];
-        const float rt = (float)(jz * up);
-        float d = ch[0] * rt, z32 = d;
+    // kPoly: z = P(D^-1 r) of the thread's row (all threads of the component take part; a fixed row's z
+    // stays 0); d is the step before it is divided by the diagonal
+    auto polynomial = [&](double r, double dinv, int rs, int re) {
+        const double di = dinv * s.il[sys];
+        double d = a.cheb[0] * r, zk = di * d;
 #pragma unroll 1
         for (int k = 0; k < kCheb; ++k) {
-            const unsigned ep = epoch32 + k;
-            unsigned long long* const w = zf + (k & 1) * n;
-            float* const zl = szf + (2 * c + (k & 1)) * width;
+            const unsigned long long ep = epochp + k;
+            ulonglong2* const w = zp + (k & 1) * n;
+            double* const zl = sz + (2 * c + (k & 1)) * width;
             if (mine) {
-                word32_store(w + first, z32, ep);
-                zl[first - lo] = z32;
+                word_store(w + first, zk, ep);
+                zl[first - lo] = zk;
             }
-            gather_halo([&](int j) { return word32_load(w + j); },
-                        [&](unsigned long long x) { return (unsigned)(x >> 32) == ep; },
-                        [&](int at, unsigned long long x) { zl[at] = __uint_as_float((unsigned)x); });
-            d = fmaf(ch[1 + 2 * k], d, ch[2 + 2 * k] * fmaf(-dinvf, row_dot_local(0.0f, sF, zl, rs, re), rt));
-            z32 += d;
+            gather_halo(w, ep, zl);
+            d = fma(a.cheb[1 + 2 * k], d, -a.cheb[2 + 2 * k] * row_dot_local(-r, zl, rs, re));
+            zk = fma(di, d, zk);
         }
-        epoch32 += kCheb;
-        return (double)z32 * down;
+        epochp += kCheb;
+        return zk;
     };
     // kOne: the row's state in registers
     double xv = 0.0, rv = 0.0, pv = 0.0, qv = 0.0, zv = 0.0, dinv = 0.0, sv = 0.0;
@@ -757,11 +721,11 @@ __global__ void __launch_bounds__(kCgMaxThreads, 1) cg_kernel(const __grid_const
         __syncthreads();
         if (task >= 0) cg_exchange(a, s, task, nval, set, epoch, mode);
         else if (kPoly && ahead) {
-            double* const zl = szd + c * width;
+            // (the polynomial is done with its first buffer)
+            double* const zl = sz + 2 * c * width;
             if (mine) zl[first - lo] = zv;
-            gather_halo([&](int j) { return word_raw(z + j); }, [&](const ulonglong2& x) { return x.y == epoch; },
-                        [&](int at, const ulonglong2& x) { zl[at] = __longlong_as_double((long long)x.x); });
-            sv = row_dot_local(0.0, sA, zl, rs, re);
+            gather_halo(z, epoch, zl);
+            sv = row_dot_local(0.0, zl, rs, re);
         } else if (kOne && ahead && first < hi) sv = row_dot(rs, re, zword);
         if (bad) s.fail = 1;
         __syncthreads();
@@ -769,14 +733,9 @@ __global__ void __launch_bounds__(kCgMaxThreads, 1) cg_kernel(const __grid_const
     };
     bool ok = exchange(3, 1, 0, !kPoly);
     if (kPoly && ok) {
-        const double r0 = sqrt(s.res[2][c]);
-        if (r0 > 0.0 && r0 < 1e300) {
-            up = exp2(-(double)ilogb(r0));
-            down = 1.0 / up;
-        }
         s0 = 0.0;
         if (task < 0) {
-            zv = polynomial(zv, (float)dinv, rs, re);
+            zv = polynomial(rv, dinv, rs, re);
             if (mine) {
                 word_store(z + first, zv, epoch);
                 s0 = rv * zv;
@@ -840,8 +799,7 @@ __global__ void __launch_bounds__(kCgMaxThreads, 1) cg_kernel(const __grid_const
             const double alpha = s.coef[c];
             if (kOne) {
                 rv = __fma_rn(-alpha, qv, rv);
-                zv = rv * dinv;
-                if (kPoly) zv = polynomial(zv, (float)dinv, rs, re);
+                zv = kPoly ? polynomial(rv, dinv, rs, re) : rv * dinv;
                 if (first < hi) {
                     word_store(z + first, zv, epoch);
                     s0 = rv * zv;
@@ -1292,7 +1250,7 @@ cudaError_t fem_build(const double* node_xy, int N, const int32_t* tri, int E, c
     for (int i = 0; i < ndof; ++i) {
         double total = 0.0;
         for (int t = row[i]; t < row[i + 1]; ++t) total += std::fabs(Kval[t]);
-        F->lmaxK = std::max(F->lmaxK, (float)(total / Kdiag[i]));
+        F->lmaxK = std::max(F->lmaxK, total / Kdiag[i]);
     }
     // cg_kernel's partition (one CTA per SM): every CTA's rows of others that its rows refer to, and the
     // columns as indices into (its own rows, those)
@@ -1339,9 +1297,9 @@ cudaError_t fem_build(const double* node_xy, int N, const int32_t* tri, int E, c
         (e = cudaMemset(F->cg_slots, 0, sizeof(ulonglong2) * cg_slot_words(F->cg_ctas))) ||
         (e = cudaMalloc((void**)&F->cg_z, sizeof(ulonglong2) * kCgComps * ((size_t)ndof + 255))) ||
         (e = cudaMemset(F->cg_z, 0, sizeof(ulonglong2) * kCgComps * ((size_t)ndof + 255))) ||
-        (e = cudaMalloc((void**)&F->cg_zf, sizeof(unsigned long long) * 2 * kCgComps * (size_t)ndof)) ||
-        (e = cudaMemset(F->cg_zf, 0, sizeof(unsigned long long) * 2 * kCgComps * (size_t)ndof)) ||
-        (e = cudaMalloc((void**)&F->lmax, sizeof(float))) ||
+        (e = cudaMalloc((void**)&F->cg_zp, sizeof(ulonglong2) * 2 * kCgComps * (size_t)ndof)) ||
+        (e = cudaMemset(F->cg_zp, 0, sizeof(ulonglong2) * 2 * kCgComps * (size_t)ndof)) ||
+        (e = cudaMalloc((void**)&F->lmax, sizeof(double))) ||
         (e = cudaMalloc((void**)&F->cg_out, sizeof(int) * kCgOut)) ||
         (e = cudaMallocHost((void**)&F->cg_host, sizeof(int) * kCgOut)) || (e = cg_configure())) {
         fem_free(F);
@@ -1355,7 +1313,7 @@ void fem_free(Fem* F)
 {
     if (!F) return;
     void* ps[] = {F->dof, F->dof_node, F->edof, F->area, F->grad, F->de_ptr, F->de_el, F->iarea, F->row, F->col, F->lcol, F->halo_ptr, F->halo,
-                  F->cptr, F->cel, F->Mval, F->Kval, F->Kdiag, F->Aval, F->wall, F->normal, F->work, F->part, F->cg_slots, F->cg_z, F->cg_zf, F->lmax, F->cg_out,
+                  F->cptr, F->cel, F->Mval, F->Kval, F->Kdiag, F->Aval, F->wall, F->normal, F->work, F->part, F->cg_slots, F->cg_z, F->cg_zp, F->lmax, F->cg_out,
                   F->xy, F->seg, F->segn, F->seg_off, F->ncomp, F->wdist, F->wseg, F->wt};
     for (void* p : ps) cudaFree(p);
     cudaFreeHost(F->cg_host);
@@ -1395,20 +1353,22 @@ cudaError_t launch_cg(Fem& F, CgArgs& a, cudaStream_t st)
     const int systems = (a.nv0 > 0) + (a.nc > a.nv0);
     a.width = rows + F.max_halo;
     size_t bytes = slice * (sizeof(int) + sizeof(double) * systems);
-    const size_t poly = bytes + slice * sizeof(float) * systems + a.nc * (size_t)a.width * 16 + sizeof(int) * (size_t)F.max_halo;
-    const bool smem = one ? poly <= kCgPolySmemMax && a.maxit < (1 << 24) : bytes <= kCgSmemMax;
+    const size_t poly = bytes + a.nc * (size_t)a.width * 2 * sizeof(double) + sizeof(int) * (size_t)F.max_halo;
+    const bool smem = one ? poly <= kCgPolySmemMax : bytes <= kCgSmemMax;
     if (one) bytes = poly;
     if (one && smem) {
-        // the 8-byte words' epochs are 32 bits wide: start again from cleared words before they run out
-        const unsigned need = (unsigned)kCheb * ((unsigned)a.maxit + 2u);
-        if (F.cg_epoch32 > 0xffffffffu - need) {
-            const cudaError_t z = cudaMemsetAsync(F.cg_zf, 0, sizeof(unsigned long long) * 2 * kCgComps * (size_t)n, st);
-            if (z != cudaSuccess) return z;
-            F.cg_epoch32 = 1;
+        const double lo = 1.0 / kChebRatio, sigma = (1.0 + lo) / (1.0 - lo);
+        a.cheb[0] = 2.0 / (1.0 + lo);
+        double rho = 1.0 / sigma;
+        for (int k = 0; k < kCheb; ++k) {
+            const double next = 1.0 / (2.0 * sigma - rho);
+            a.cheb[1 + 2 * k] = next * rho;
+            a.cheb[2 + 2 * k] = 4.0 * next / (1.0 - lo);
+            rho = next;
         }
-        a.epoch32 = F.cg_epoch32;
-        F.cg_epoch32 += need;
-        a.zf = F.cg_zf;
+        a.epochp = F.cg_epochp;
+        F.cg_epochp += (unsigned long long)kCheb * ((unsigned long long)a.maxit + 2ull);
+        a.zp = F.cg_zp;
         a.lcol = F.lcol;
         a.halo_ptr = F.halo_ptr;
         a.halo = F.halo;
@@ -1468,7 +1428,7 @@ cudaError_t node_fields_solve(Fem& F, const double* stats, const lpdf_params& P,
     a.state = cgs;
     if (relax) {
         elem_L2_kernel<<<ge, 256, 0, st>>>(F, L2, ew);
-        const cudaError_t e = cudaMemsetAsync(F.lmax, 0, sizeof(float), st);
+        const cudaError_t e = cudaMemsetAsync(F.lmax, 0, sizeof(double), st);
         if (e != cudaSuccess) return e;
         assemble_kernel<<<gd, 256, 0, st>>>(F, ew, F.Aval, diag, F.lmax);
         const bool warm = P.cg_warm_start && F.has_wp;
