@@ -377,6 +377,17 @@ int lpdf_elliptic_relax_solve(const lpdf_mesh* mesh, const lpdf_params* params, 
                               float* fields, double tol, int32_t maxit, int32_t* iters, void* stream);
 
 /* ---------------------------------------------------------------------------------------
+ * lpdf_mesh_set_cg_wait -- the bounded waits of this mesh's conjugate gradients, whose thread blocks wait
+ * for one another's words. A wait that gives up makes the solve return LPDF_ERR_CUDA; the fields and the
+ * warm start stay as they were. polls: the limit of a wait, in polls of about 0.2 us (1..LPDF_CG_POLLS,
+ * the default). quit_cta >= 0: a test aid, that block of the launch gives up at its first wait, as one
+ * whose wait has run out (with several rows per thread it leaves its words of the preconditioned residual
+ * out as well); -1, the default: none. Errors: LPDF_ERR_ARG, LPDF_ERR_CUDA.
+ * ------------------------------------------------------------------------------------- */
+#define LPDF_CG_POLLS 2097152
+int lpdf_mesh_set_cg_wait(lpdf_mesh* mesh, int32_t polls, int32_t quit_cta);
+
+/* ---------------------------------------------------------------------------------------
  * lpdf_tc_gemm_bf16 -- the tensor-core tile of the learned relaxation surrogate, exposed to
  * test it: D = A B^T on the fifth-generation
  * tensor cores (tcgen05, BF16 inputs, FP32 accumulation in tensor memory). The paper has no

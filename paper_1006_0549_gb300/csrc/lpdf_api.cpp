@@ -1039,6 +1039,17 @@ int lpdf_elliptic_relax_solve(const lpdf_mesh* mesh, const lpdf_params* params, 
     return LPDF_OK;
 }
 
+int lpdf_mesh_set_cg_wait(lpdf_mesh* mesh, int32_t polls, int32_t quit_cta)
+{
+    if (!mesh || polls < 1 || polls > LPDF_CG_POLLS || quit_cta < -1)
+        return fail(LPDF_ERR_ARG, "mesh_set_cg_wait: polls = %d, quit_cta = %d", polls, quit_cta);
+    Fem* F = nullptr;
+    if (const int rc = mesh_fem(mesh, &F)) return rc;
+    F->cg_polls = polls;
+    F->cg_quit = quit_cta;
+    return LPDF_OK;
+}
+
 int lpdf_tc_gemm_bf16(const void* A, const void* B, float* D, int32_t M, int32_t N, int32_t K, void* stream)
 {
     if (!A || !B || !D) return fail(LPDF_ERR_ARG, "tc_gemm_bf16: NULL argument");

@@ -238,6 +238,8 @@ struct Fem {
     double* lmax = nullptr;      // bounds of the spectra of D^-1 A (device) and D^-1 K
     double lmaxK = 0.0;
     unsigned long long cg_epoch = 1, cg_epochp = 1;
+    // lpdf_mesh_set_cg_wait: the limit of a wait, and the CTA that gives up at its first one
+    int cg_polls = LPDF_CG_POLLS, cg_quit = -1;
     int* cg_out = nullptr;
     int* cg_host = nullptr;      // pinned copy
     std::vector<int> row_host;   // the matrix pattern's row starts

@@ -194,7 +194,6 @@ constexpr int kCgSmallUnits = kCgSmallRows / 32;
 constexpr int kCgMaxThreads = 1024;               // cg_kernel
 constexpr int kCheb = 16;                         // its polynomial's degree and range (below)
 constexpr double kChebRatio = 256.0;
-constexpr int kCgMaxTries = 1 << 21;              // polls (of about 0.2 us) before a wait gives up
 enum { kCgIts0 = 0, kCgIts1 = 1, kCgOk = 2, kCgError = 3, kCgOut = 4 };   // kCgOk: systems converged
 
 struct CgArgs {
@@ -214,6 +213,7 @@ struct CgArgs {
     unsigned long long epoch, epochp;       // of z and the partial sums, of zp
     ulonglong2 *z, *slots;                  // nc n words; the partial sums' words
     ulonglong2* zp;                         // 2 nc n words
+    int polls, quit;                        // polls (of about 0.2 us) before a wait gives up; see Fem
     int* out;
 };
 
@@ -287,7 +287,7 @@ __device__ __forceinline__ double cg_small_sum(double v0, double v1, int nu, int
 }
 
 __device__ __forceinline__ double cg_small_total(const ulonglong2* s, int nu, int nb, unsigned long long epoch, int lane,
-                                                 bool& alive)
+                                                 int polls, bool& alive)
 {
     double v0, v1;
     bool ok;
@@ -297,7 +297,7 @@ __device__ __forceinline__ double cg_small_total(const ulonglong2* s, int nu, in
         v0 = lane < nu ? word_load(s + lane, epoch, ok) : 0.0;
         v1 = lane + 32 < nu ? word_load(s + lane + 32, epoch, ok) : 0.0;
         ok = __all_sync(0xffffffffu, ok);
-    } while (!ok && ++tries < kCgMaxTries);
+    } while (!ok && ++tries < polls);
     alive = alive && ok;
     return cg_small_sum(v0, v1, nu, nb);
 }
@@ -311,7 +311,7 @@ __device__ __forceinline__ double warp_tree(double v)
 
 __global__ void __launch_bounds__(32) cg_small_kernel(const __grid_constant__ CgArgs a)
 {
-    const int lane = threadIdx.x, nb = (a.n + 255) / 256, nu = 8 * nb;
+    const int lane = threadIdx.x, nb = (a.n + 255) / 256, nu = 8 * nb, polls = a.polls;
     const int c = blockIdx.x / nu, u = blockIdx.x - c * nu;
     const bool sys = c >= a.nv0;
     const int v = sys ? c - a.nv0 : c, c0 = sys ? a.nv0 : 0, c1 = sys ? a.nc : a.nv0;   // the system's components
@@ -350,7 +350,7 @@ __global__ void __launch_bounds__(32) cg_small_kernel(const __grid_constant__ Cg
     double r = fixed ? 0.0 : __dsub_rn(b, y);
     double z = div_by(r, diag, dinv), q = 0.0;
     unsigned long long epoch = a.epoch;
-    bool alive = true;
+    bool alive = (int)blockIdx.x != a.quit;
     auto post = [&](int k, double value) {
         const double s = warp_tree(value);
         if (lane == 0) word_store(slot(k, c) + u, s, epoch);
@@ -371,8 +371,8 @@ __global__ void __launch_bounds__(32) cg_small_kernel(const __grid_constant__ Cg
             for (int t = 0; t < kCgDeg; ++t) zn[t] = word[t] >= 0 ? word_load(zw + word[t], epoch, ok) : 0.0;
         };
         load();
-        const double sum = cg_small_total(slot(1, c), nu, nb, epoch, lane, alive);
-        while (!__all_sync(0xffffffffu, ok) && ++tries < kCgMaxTries) load();   // mostly there by now
+        const double sum = cg_small_total(slot(1, c), nu, nb, epoch, lane, polls, alive);
+        while (!__all_sync(0xffffffffu, ok) && ++tries < polls) load();   // mostly there by now
         alive = alive && __all_sync(0xffffffffu, ok);
         return sum;
     };
@@ -380,7 +380,7 @@ __global__ void __launch_bounds__(32) cg_small_kernel(const __grid_constant__ Cg
     double r0[4], beta = 0.0;
 #pragma unroll
     for (int k = 0; k < 4; ++k)
-        r0[k] = c0 + k < c1 ? a.tol * sqrt(cg_small_total(slot(2, c0 + k), nu, nb, epoch, lane, alive)) : 0.0;
+        r0[k] = c0 + k < c1 ? a.tol * sqrt(cg_small_total(slot(2, c0 + k), nu, nb, epoch, lane, polls, alive)) : 0.0;
     bool done = false;
     int it = 0, set = 3;
     for (; alive; ++it) {
@@ -390,7 +390,7 @@ __global__ void __launch_bounds__(32) cg_small_kernel(const __grid_constant__ Cg
 #pragma unroll
             for (int k = 0; k < 4; ++k)
                 if (c0 + k < c1) {
-                    const double rr = cg_small_total(slot(set, c0 + k), nu, nb, epoch, lane, alive);
+                    const double rr = cg_small_total(slot(set, c0 + k), nu, nb, epoch, lane, polls, alive);
                     done = done && cg_reached(rr, r0[k]);
                     broken = broken || cg_broken(rr, r0[k]);
                 }
@@ -416,7 +416,7 @@ __global__ void __launch_bounds__(32) cg_small_kernel(const __grid_constant__ Cg
         }
         ++epoch;
         post(0, __dmul_rn(p, q));
-        const double pq = cg_small_total(slot(0, c), nu, nb, epoch, lane, alive);
+        const double pq = cg_small_total(slot(0, c), nu, nb, epoch, lane, polls, alive);
         const double alpha = pq != 0.0 ? rz / pq : 0.0;
         r = __fma_rn(-alpha, q, r);
         z = div_by(r, diag, dinv);
@@ -489,7 +489,7 @@ constexpr int kCgPoll = 5;   // words polled at once by a lane
 __device__ __forceinline__ void cg_exchange(const CgArgs& a, CgShared& s, int w, int nval, int set,
                                             unsigned long long epoch, int mode)
 {
-    const int lane = threadIdx.x & 31;
+    const int lane = threadIdx.x & 31, polls = a.polls;
     const int G = gridDim.x;
     ulonglong2* const part = a.slots + (size_t)set * 3 * kCgComps * G;
     ulonglong2* const pub = a.slots + 2 * (size_t)3 * kCgComps * G + set * 3 * kCgComps * 2;
@@ -515,7 +515,7 @@ __device__ __forceinline__ void cg_exchange(const CgArgs& a, CgShared& s, int w,
 #pragma unroll
                 for (int q = 0; q < kCgPoll; ++q)
                     v[q] = j0 + 32 * q < G ? word_load(part + (size_t)t * G + j0 + 32 * q, epoch, ok) : 0.0;
-            } while (!ok && ++tries < kCgMaxTries);
+            } while (!ok && ++tries < polls);
             if (!ok) s.fail = 1;
 #pragma unroll
             for (int q = 0; q < kCgPoll; ++q) sum = __dadd_rn(sum, v[q]);
@@ -539,7 +539,7 @@ __device__ __forceinline__ void cg_exchange(const CgArgs& a, CgShared& s, int w,
         do {
             ok = true;
             v = word_load(pub + 2 * t + (lane & 1), epoch, ok);
-        } while (!ok && ++tries < kCgMaxTries);
+        } while (!ok && ++tries < polls);
         if (!ok) s.fail = 1;
         if (lane & 1) s.res[k][c] = v;
         else if (mode && k == 0) s.coef[c] = v;
@@ -589,7 +589,9 @@ __global__ void __launch_bounds__(kCgMaxThreads, 1) cg_kernel(const __grid_const
     __syncthreads();
     const double* const sA = sys ? sA1 : sA0;
     unsigned long long epoch = a.epoch;
-    bool bad = false;
+    const int polls = a.polls;
+    const bool quit = (int)blockIdx.x == a.quit;
+    bool bad = quit;
     // (A f) of a row; f(j) loads entry j, up to kW at once, until every word has its epoch
     constexpr int kW = 10;
     auto row_dot = [&](int rs, int re, auto f) {
@@ -603,7 +605,7 @@ __global__ void __launch_bounds__(kCgMaxThreads, 1) cg_kernel(const __grid_const
 #pragma unroll
                 for (int u = 0; u < kW; ++u)
                     zv[u] = t + u < re ? f(kSmem && !kPoly ? scol[t + u - base] : __ldg(a.col + t + u), ok) : 0.0;
-            } while (!ok && ++tries < kCgMaxTries);
+            } while (!ok && ++tries < polls);
             bad = bad || !ok;
 #pragma unroll
             for (int u = 0; u < kW; ++u)
@@ -618,9 +620,9 @@ __global__ void __launch_bounds__(kCgMaxThreads, 1) cg_kernel(const __grid_const
         for (int h = tid; h < halo; h += 2 * T) {
             const int h1 = min(h + T, halo - 1), j0 = shalo[h], j1 = shalo[h1];
             ulonglong2 w0 = word_raw(words + j0), w1 = word_raw(words + j1);
-            int tries = bad ? kCgMaxTries : 0;
+            int tries = bad ? polls : 0;
             while (w0.y != ep || w1.y != ep) {
-                if (++tries >= kCgMaxTries) {
+                if (++tries >= polls) {
                     bad = true;
                     break;
                 }
@@ -698,7 +700,7 @@ __global__ void __launch_bounds__(kCgMaxThreads, 1) cg_kernel(const __grid_const
         rv = fixed ? 0.0 : b[i] - row_dot(rs, re, [&](int j, bool&) { return x[j]; });
         dinv = 1.0 / diag[i];
         zv = rv * dinv;
-        if (!kPoly) word_store(z + i, zv, epoch);
+        if (!kPoly && !quit) word_store(z + i, zv, epoch);
         s0 += rv * zv;
         s1 += rv * rv;
         if (fixed) re = rs;   // its row of A p is zero
@@ -928,12 +930,19 @@ __global__ void subtract_mean_kernel(int n, const double* __restrict__ part, int
     if (i < n) x[i] -= sum / n;
 }
 
+// every system converged and every wait got its word: CTA 0 counts the systems, but another CTA may have
+// given up after its last sum went out, and left its rows of x unwritten
+__device__ __forceinline__ bool cg_clean(const int* out, int systems)
+{
+    return out[kCgOk] == systems && out[kCgError] == 0;
+}
+
 // the converged solutions, kept as the next solve's start
 __global__ void keep_solution_kernel(const int* __restrict__ cg_out, int systems, int n4, const double* __restrict__ wp,
                                      double* __restrict__ wp_prev, int n, const double* __restrict__ p,
                                      double* __restrict__ p_prev)
 {
-    if (cg_out[kCgOk] != systems) return;
+    if (!cg_clean(cg_out, systems)) return;
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
     if (i < n4) wp_prev[i] = wp[i];
     if (i < n) p_prev[i] = p[i];
@@ -951,7 +960,7 @@ __global__ void fields_kernel(const Fem F, int ns, int nfp, const double* __rest
 {
     const int nd = blockIdx.x * blockDim.x + threadIdx.x;
     if (nd >= F.N) return;
-    if (cg_out && cg_out[kCgOk] != systems) return;   // a CG did not converge: the caller's fields stay
+    if (cg_out && !cg_clean(cg_out, systems)) return;   // no solution: the caller's fields stay
     const int d = F.dof[nd];
     const size_t n = F.ndof;
     const double* r = R + 6 * (size_t)d;       // uu, uv, uw, vv, vw, ww
@@ -1335,6 +1344,8 @@ cudaError_t launch_cg(Fem& F, CgArgs& a, cudaStream_t st)
     a.wall = F.wall;
     a.slots = static_cast<ulonglong2*>(F.cg_slots);
     a.out = F.cg_out;
+    a.polls = F.cg_polls;
+    a.quit = F.cg_quit;
     a.epoch = F.cg_epoch;
     F.cg_epoch += (unsigned long long)a.maxit + 4ull;
     const cudaError_t e = cudaMemsetAsync(F.cg_out, 0, sizeof(int) * kCgOut, st);

@@ -40,7 +40,8 @@ EXPORTS = ("lpdf_params_default", "lpdf_last_error", "lpdf_version", "lpdf_mesh_
            "lpdf_mlp_forward", "lpdf_mlp_gradient", "lpdf_mlp_train", "lpdf_surrogate_features",
            "lpdf_mlp_set_policy", "lpdf_surrogate_relax_solve", "lpdf_mesh_load_multi", "lpdf_ctx_set_components",
            "lpdf_particles_init_multi", "lpdf_pdf_steps", "lpdf_ctx_set_tune", "lpdf_ctx_autotune",
-           "lpdf_grid_flux_statistics", "lpdf_iecm_coefficients", "lpdf_ctx_set_iecm", "lpdf_mlp_request_check")
+           "lpdf_grid_flux_statistics", "lpdf_iecm_coefficients", "lpdf_ctx_set_iecm", "lpdf_mlp_request_check",
+           "lpdf_mesh_set_cg_wait")
 
 N_ADV_VARIANTS, N_MOM_VARIANTS = 6, 4
 
@@ -117,6 +118,7 @@ def lib():
     L.lpdf_ctx_set_timing.argtypes = [vp, ctypes.c_int]
     L.lpdf_ctx_timings.argtypes = [vp, vp, vp]
     L.lpdf_elliptic_relax_solve.argtypes = [vp, vp, vp, vp, ctypes.c_double, i32, vp, vp]
+    L.lpdf_mesh_set_cg_wait.argtypes = [vp, i32, i32]
     L.lpdf_mlp_create.argtypes = [i64, vp]
     L.lpdf_mlp_free.argtypes = [vp]
     L.lpdf_mlp_free.restype = None
@@ -235,6 +237,10 @@ class Mesh:
         _check(lib().lpdf_elliptic_relax_solve(self.h, ctypes.byref(params), _ptr(stats), _ptr(out), float(tol),
                                                int(maxit), _ptr(it), _stream(stream)))
         return int(it[0]), int(it[1])
+
+    def set_cg_wait(self, polls: int = 1 << 21, quit_cta: int = -1):
+        """lpdf_mesh_set_cg_wait: the bounded waits of the mesh's CGs (a test aid)."""
+        _check(lib().lpdf_mesh_set_cg_wait(self.h, int(polls), int(quit_cta)))
 
     def iecm_coefficients(self, ns: int, stats, flux, beta, stream=None):
         """lpdf_iecm_coefficients: beta (n_nodes x 3 ns FP32) from statistics and flux covariances."""
