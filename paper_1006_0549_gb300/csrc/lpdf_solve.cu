@@ -253,9 +253,8 @@ __device__ __forceinline__ double word_load(const ulonglong2* p, unsigned long l
     return __longlong_as_double(b);
 }
 
-// the test of a component from its |r|^2 and tol |r_0|: reached, or no longer worth iterating
-__device__ __forceinline__ bool cg_reached(double rr, double limit) { return sqrt(rr) <= limit && isfinite(limit); }
-__device__ __forceinline__ bool cg_broken(double rr, double limit) { return !isfinite(rr) || !isfinite(limit); }
+// neither infinite nor NaN, from the exponent (a comparison is an FP64 instruction: 65 cycles)
+__device__ __forceinline__ bool finite_bits(double v) { return (__double2hiint(v) & 0x7ff00000) != 0x7ff00000; }
 
 __device__ __forceinline__ double shfl_add(double v, int o) { return __dadd_rn(v, __shfl_down_sync(0xffffffffu, v, o)); }
 
@@ -378,22 +377,24 @@ __global__ void __launch_bounds__(32) cg_small_kernel(const __grid_constant__ Cg
     };
     double rz = gather();
     double r0[4], beta = 0.0;
+    bool broken = false, done = false;             // broken: a norm is not finite
 #pragma unroll
-    for (int k = 0; k < 4; ++k)
+    for (int k = 0; k < 4; ++k) {
         r0[k] = c0 + k < c1 ? a.tol * sqrt(cg_small_total(slot(2, c0 + k), nu, nb, epoch, lane, polls, alive)) : 0.0;
-    bool done = false;
+        broken = broken || !finite_bits(r0[k]);
+    }
     int it = 0, set = 3;
     for (; alive; ++it) {
         if (it % kCheckEvery == 0 || it >= a.maxit) {
             done = true;
-            bool broken = false;
 #pragma unroll
             for (int k = 0; k < 4; ++k)
                 if (c0 + k < c1) {
                     const double rr = cg_small_total(slot(set, c0 + k), nu, nb, epoch, lane, polls, alive);
-                    done = done && cg_reached(rr, r0[k]);
-                    broken = broken || cg_broken(rr, r0[k]);
+                    if (!(sqrt(rr) <= r0[k])) done = false;
+                    broken = broken || !finite_bits(rr);
                 }
+            done = done && !broken;
             if (!alive || done || broken || it >= a.maxit) break;
             set = 7 - set;
         }
@@ -758,8 +759,8 @@ __global__ void __launch_bounds__(kCgMaxThreads, 1) cg_kernel(const __grid_const
             if (wid == 0) {
                 const bool on = lane < a.nc && ((s.active >> lane) & 1u);
                 const double rr = on ? s.rr[lane] : 0.0, limit = on ? a.tol * s.r0[lane] : 0.0;
-                const unsigned f = __ballot_sync(0xffffffffu, on && !cg_reached(rr, limit));
-                const unsigned broken = __ballot_sync(0xffffffffu, on && cg_broken(rr, limit));
+                const unsigned broken = __ballot_sync(0xffffffffu, !finite_bits(rr) || !finite_bits(limit));
+                const unsigned f = __ballot_sync(0xffffffffu, !(sqrt(rr) <= limit)) | broken;
                 if (lane == 0) {
                     const unsigned m0 = (1u << a.nv0) - 1u, m1 = ((1u << a.nc) - 1u) & ~m0;
                     unsigned act = s.active;
