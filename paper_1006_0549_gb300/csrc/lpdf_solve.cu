@@ -479,6 +479,7 @@ struct CgShared {
     double r0[8], rr[8];
     unsigned active;             // components still iterating
     int stop, fail;
+    int lost;                    // a wait of the CTA gave up: its others poll once more only
     double il[2];                // per system: 1 / the bound of its spectrum
 };
 
@@ -492,6 +493,7 @@ __device__ __forceinline__ void cg_exchange(const CgArgs& a, CgShared& s, int w,
 {
     const int lane = threadIdx.x & 31, polls = a.polls;
     const int G = gridDim.x;
+    const bool lost = s.lost;
     ulonglong2* const part = a.slots + (size_t)set * 3 * kCgComps * G;
     ulonglong2* const pub = a.slots + 2 * (size_t)3 * kCgComps * G + set * 3 * kCgComps * 2;
     for (int t = w; t < nval * a.nc; t += kCgTasks) {
@@ -506,23 +508,26 @@ __device__ __forceinline__ void cg_exchange(const CgArgs& a, CgShared& s, int w,
         const int k = t / a.nc, c = t - k * a.nc;
         if (!((s.active >> c) & 1u) || blockIdx.x != t % G) continue;
         double sum = 0.0;
-        bool ok = true;
+        bool got = true;
         const double y = mode == 2 && k == 0 ? 1.0 / s.rz[c] : 0.0;
         for (int j0 = lane; j0 < G; j0 += 32 * kCgPoll) {
             double v[kCgPoll];
-            int tries = 0;
+            bool ok;
+            int tries = got && !lost ? 0 : polls;
             do {
                 ok = true;
 #pragma unroll
                 for (int q = 0; q < kCgPoll; ++q)
                     v[q] = j0 + 32 * q < G ? word_load(part + (size_t)t * G + j0 + 32 * q, epoch, ok) : 0.0;
             } while (!ok && ++tries < polls);
-            if (!ok) s.fail = 1;
+            got = got && ok;
 #pragma unroll
             for (int q = 0; q < kCgPoll; ++q) sum = __dadd_rn(sum, v[q]);
         }
+        got = __all_sync(0xffffffffu, got);
+        if (!got) s.fail = 1;
         sum = warp_tree(sum);
-        if (lane == 0) {
+        if (lane == 0 && got) {   // (a sum that lacks a part is not published)
             double coef = 0.0;
             if (mode == 1) coef = sum != 0.0 ? s.rz[c] / sum : 0.0;
             if (mode == 2 && k == 0) coef = s.rz[c] != 0.0 ? div_by(sum, s.rz[c], y) : 0.0;
@@ -536,7 +541,7 @@ __device__ __forceinline__ void cg_exchange(const CgArgs& a, CgShared& s, int w,
     if (t < nval * a.nc && ((s.active >> c) & 1u)) {
         bool ok;
         double v;
-        int tries = 0;
+        int tries = lost ? polls : 0;
         do {
             ok = true;
             v = word_load(pub + 2 * t + (lane & 1), epoch, ok);
@@ -586,6 +591,7 @@ __global__ void __launch_bounds__(kCgMaxThreads, 1) cg_kernel(const __grid_const
         s.active = (1u << a.nc) - 1u;
         s.stop = 0;
         s.fail = 0;
+        s.lost = 0;
     }
     __syncthreads();
     const double* const sA = sys ? sA1 : sA0;
@@ -593,21 +599,25 @@ __global__ void __launch_bounds__(kCgMaxThreads, 1) cg_kernel(const __grid_const
     const int polls = a.polls;
     const bool quit = (int)blockIdx.x == a.quit;
     bool bad = quit;
-    // (A f) of a row; f(j) loads entry j, up to kW at once, until every word has its epoch
+    // (A f) of a row; f(j) loads entry j, up to kW at once, until every word has its epoch. A CTA waits for a
+    // lost word once, however many rows refer to lost ones.
     constexpr int kW = 10;
     auto row_dot = [&](int rs, int re, auto f) {
         double sum = 0.0;
         for (int t = rs; t < re; t += kW) {
             double zv[kW];
             bool ok;
-            int tries = 0;
+            int tries = *(volatile int*)&s.lost ? polls : 0;
             do {
                 ok = true;
 #pragma unroll
                 for (int u = 0; u < kW; ++u)
                     zv[u] = t + u < re ? f(kSmem && !kPoly ? scol[t + u - base] : __ldg(a.col + t + u), ok) : 0.0;
             } while (!ok && ++tries < polls);
-            bad = bad || !ok;
+            if (!ok) {
+                bad = true;
+                *(volatile int*)&s.lost = 1;
+            }
 #pragma unroll
             for (int u = 0; u < kW; ++u)
                 if (t + u < re) sum = __fma_rn(kSmem ? sA[t + u - base] : __ldg(gA + t + u), zv[u], sum);
