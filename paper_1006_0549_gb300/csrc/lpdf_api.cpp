@@ -669,12 +669,14 @@ int lpdf_particles_init_multi(lpdf_ctx* c, const int32_t* n_per_elem, const floa
 }
 
 // The user's arrays into the records or back. Device arrays: one kernel. Host arrays: by way of a
-// stream-ordered staging buffer of at most kStage particles at a time (given back at the end).
-static int copy_state(lpdf_ctx* c, int64_t n, bool in, const UserArrays& user, int on_device, cudaStream_t st)
+// stream-ordered staging buffer of at most kStage particles at a time (given back at the end). *touched is
+// set once a record may have been written.
+static int copy_state(lpdf_ctx* c, int64_t n, bool in, const UserArrays& user, int on_device, cudaStream_t st, bool* touched)
 {
     if (n == 0) return LPDF_OK;
     const int ns = c->ns;
     if (on_device) {
+        *touched = in;
         CUDA_TRY(in ? launch_pack_state(c->s, 0, n, ns, user, st) : launch_unpack_state(c->s, 0, n, ns, user, st));
         return LPDF_OK;
     }
@@ -700,7 +702,10 @@ static int copy_state(lpdf_ctx* c, int64_t n, bool in, const UserArrays& user, i
             e = in ? cudaMemcpyAsync(d, h, sizeof(float) * (size_t)k, cudaMemcpyHostToDevice, st)
                    : cudaMemcpyAsync(h, d, sizeof(float) * (size_t)k, cudaMemcpyDeviceToHost, st);
         }
-        if (in && e == cudaSuccess) e = launch_pack_state(c->s, i0, k, ns, dev, st);
+        if (in && e == cudaSuccess) {
+            *touched = true;
+            e = launch_pack_state(c->s, i0, k, ns, dev, st);
+        }
     }
     const cudaError_t f = cudaFreeAsync(stage, st);
     CUDA_TRY(e);
@@ -717,13 +722,24 @@ int lpdf_set_state(lpdf_ctx* c, int64_t n, const float* x, const float* y, const
     if (n < 0 || n > c->s.cap) return fail(LPDF_ERR_ARG, "n = %lld outside 0..%lld", (long long)n, (long long)c->s.cap);
     if (n > 0 && (!x || !y || !u || !v || !w || !om || !psi || !elem || !pid))
         return fail(LPDF_ERR_ARG, "set_state needs every array");
-    c->s.n = n;
     const UserArrays user{(float*)x, (float*)y, (float*)u, (float*)v, (float*)w, (float*)om, (float*)psi, (int*)elem,
                           (uint32_t*)pid, n};
-    const int rc = copy_state(c, n, true, user, on_device, (cudaStream_t)stream);
-    if (rc) return rc;
+    // a failure before any record was written leaves the ensemble as it was, a later one none: the records
+    // and the order of a step belong to the same n
+    bool touched = false;
+    int rc = copy_state(c, n, true, user, on_device, (cudaStream_t)stream, &touched);
     // any order is valid input; the first step brings the ensemble into element order
-    CUDA_TRY(launch_iota(c->pipe.perm, n, (cudaStream_t)stream));
+    if (rc == LPDF_OK) {
+        touched = true;
+        const cudaError_t e = launch_iota(c->pipe.perm, n, (cudaStream_t)stream);
+        if (e != cudaSuccess) rc = fail(LPDF_ERR_CUDA, "set_state: %s", cudaGetErrorString(e));
+    }
+    if (rc) {
+        (void)cudaGetLastError();   // reported here
+        if (touched) c->s.n = 0;
+        return rc;
+    }
+    c->s.n = n;
     return LPDF_OK;
 }
 
@@ -732,7 +748,10 @@ int lpdf_get_state(const lpdf_ctx* c, float* x, float* y, float* u, float* v, fl
 {
     if (!c) return fail(LPDF_ERR_ARG, "ctx is NULL");
     const UserArrays user{x, y, u, v, w, om, psi, elem, pid, c->s.n};
-    return copy_state(const_cast<lpdf_ctx*>(c), c->s.n, false, user, on_device, (cudaStream_t)stream);
+    bool touched = false;
+    const int rc = copy_state(const_cast<lpdf_ctx*>(c), c->s.n, false, user, on_device, (cudaStream_t)stream, &touched);
+    if (rc) (void)cudaGetLastError();   // reported here
+    return rc;
 }
 
 int lpdf_sort(lpdf_ctx* c, void* stream)
