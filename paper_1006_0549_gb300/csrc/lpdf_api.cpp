@@ -668,14 +668,39 @@ int lpdf_particles_init_multi(lpdf_ctx* c, const int32_t* n_per_elem, const floa
                      (cudaStream_t)stream);
 }
 
-// The user's arrays into the records or back. Device arrays: one kernel. Host arrays: by way of a
+// whether a kernel on `device` may use `bytes` bytes at p: this device's or managed memory, of words (a
+// shorter allocation, another device's or pageable memory and odd addresses go through a copy, which
+// handles them or reports them)
+static bool in_reach(const void* p, size_t bytes, int device)
+{
+    if (!p) return true;
+    if ((uintptr_t)p % sizeof(float)) return false;
+    for (const char* q : {(const char*)p, (const char*)p + bytes - 1}) {
+        cudaPointerAttributes at;
+        if (cudaPointerGetAttributes(&at, q) != cudaSuccess) {
+            (void)cudaGetLastError();
+            return false;
+        }
+        if (at.type != cudaMemoryTypeManaged && (at.type != cudaMemoryTypeDevice || at.device != device)) return false;
+    }
+    return true;
+}
+
+static bool all_in_reach(const UserArrays& a, int64_t n, int ns, int device)
+{
+    for (const void* p : {(void*)a.x, (void*)a.y, (void*)a.u, (void*)a.v, (void*)a.w, (void*)a.om, (void*)a.elem, (void*)a.pid})
+        if (!in_reach(p, sizeof(float) * (size_t)n, device)) return false;
+    return in_reach(a.psi, sizeof(float) * (size_t)n * ns, device);
+}
+
+// The user's arrays into the records or back. Device arrays: one kernel. Other arrays: by way of a
 // stream-ordered staging buffer of at most kStage particles at a time (given back at the end). *touched is
 // set once a record may have been written.
 static int copy_state(lpdf_ctx* c, int64_t n, bool in, const UserArrays& user, int on_device, cudaStream_t st, bool* touched)
 {
     if (n == 0) return LPDF_OK;
     const int ns = c->ns;
-    if (on_device) {
+    if (on_device && all_in_reach(user, n, ns, c->mesh->device)) {
         *touched = in;
         CUDA_TRY(in ? launch_pack_state(c->s, 0, n, ns, user, st) : launch_unpack_state(c->s, 0, n, ns, user, st));
         return LPDF_OK;
@@ -699,8 +724,10 @@ static int copy_state(lpdf_ctx* c, int64_t n, bool in, const UserArrays& user, i
             if (!h) continue;
             h += sizeof(float) * (size_t)i0;
             float* d = stage + r * m;
-            e = in ? cudaMemcpyAsync(d, h, sizeof(float) * (size_t)k, cudaMemcpyHostToDevice, st)
-                   : cudaMemcpyAsync(h, d, sizeof(float) * (size_t)k, cudaMemcpyDeviceToHost, st);
+            const cudaMemcpyKind kind =
+                on_device ? cudaMemcpyDeviceToDevice : (in ? cudaMemcpyHostToDevice : cudaMemcpyDeviceToHost);
+            e = in ? cudaMemcpyAsync(d, h, sizeof(float) * (size_t)k, kind, st)
+                   : cudaMemcpyAsync(h, d, sizeof(float) * (size_t)k, kind, st);
         }
         if (in && e == cudaSuccess) {
             *touched = true;
