@@ -365,6 +365,11 @@ struct lpdf_ctx {
     cudaGraphExec_t graph[2] = {nullptr, nullptr};
     const float* graph_fields[2] = {nullptr, nullptr};
     unsigned long long* step_dev = nullptr;   // the step number the graph's kernels read
+    // staging buffer of lpdf_set_state / lpdf_get_state (stage_cap particles), free after stage_done
+    float* stage = nullptr;
+    int64_t stage_cap = 0;
+    cudaEvent_t stage_done = nullptr;
+    std::mutex stage_mutex;
     bool timing = false;
     std::vector<cudaEvent_t> ev_free;
     std::vector<std::array<cudaEvent_t, 4>> ev_pending;
