@@ -231,7 +231,7 @@ struct Fem {
     // per CTA of cg_kernel the other CTAs' rows that its rows refer to (halo, CSR over the CTAs), and the
     // matrix's columns as indices into (the CTA's rows, its halo)
     int *lcol = nullptr, *halo_ptr = nullptr, *halo = nullptr;
-    int max_halo = 0;
+    int max_halo = 0, max_slice = 0;   // rows of a halo, matrix entries of a CTA's rows, at most
     void* cg_slots = nullptr;
     ulonglong2* cg_z = nullptr;
     ulonglong2* cg_zp = nullptr;           // the preconditioner's words
@@ -242,7 +242,6 @@ struct Fem {
     int cg_polls = LPDF_CG_POLLS, cg_quit = -1;
     int* cg_out = nullptr;
     int* cg_host = nullptr;      // pinned copy
-    std::vector<int> row_host;   // the matrix pattern's row starts
     bool has_wp = false;         // the scratch holds a previous relaxation / pressure solution
     bool has_p = false;
     // wall distance of every geometric node (inputs of the learned surrogate)
