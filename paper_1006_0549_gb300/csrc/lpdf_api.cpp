@@ -515,9 +515,9 @@ int lpdf_ctx_create(const lpdf_mesh* mesh, const lpdf_params* params, int64_t ca
     s2.n = 0;
     s2.cap = cap;
     const size_t E = (size_t)mesh->d.n_tri;
-    const size_t rest = (size_t)cap * rest_words(c->ns);
-    if ((ce = pipeline_configure()) || (ce = dalloc(&s.rec, 8 * cap)) || (ce = dalloc(&s.elem, cap)) || (rest && (ce = dalloc(&s.rest, rest))) ||
-        (ce = dalloc(&s2.rec, 8 * cap)) || (ce = dalloc(&s2.elem, cap)) || (rest && (ce = dalloc(&s2.rest, rest))) ||
+    const size_t rest = (size_t)cap * rest_words(c->ns), pids = c->ns > 1 ? (size_t)cap : 0;
+    if ((ce = pipeline_configure()) || (ce = dalloc(&s.rec, 8 * cap)) || (ce = dalloc(&s.elem, cap)) || (rest && (ce = dalloc(&s.rest, rest))) || (pids && (ce = dalloc(&s.pid, pids))) ||
+        (ce = dalloc(&s2.rec, 8 * cap)) || (ce = dalloc(&s2.elem, cap)) || (rest && (ce = dalloc(&s2.rest, rest))) || (pids && (ce = dalloc(&s2.pid, pids))) ||
         (ce = dalloc(&c->sort.cnt, E + 1)) || (ce = dalloc(&c->sort.cursor, E + 1)) ||
         (ce = dalloc(&c->sort.start, E + 2)) || (ce = dalloc(&c->sort.perm, cap)) ||
         (ce = dalloc(&c->node_acc, (size_t)mesh->d.n_nodes * nq)) || (ce = dalloc(&c->status, 4)) ||
@@ -552,6 +552,7 @@ void lpdf_ctx_free(lpdf_ctx* c)
     for (Particles* s : {&c->s, &c->s2}) {
         cudaFree(s->rec);
         cudaFree(s->rest);
+        cudaFree(s->pid);
         cudaFree(s->elem);
     }
     cudaFree(c->sort.cnt); cudaFree(c->sort.cursor); cudaFree(c->sort.start); cudaFree(c->sort.perm);

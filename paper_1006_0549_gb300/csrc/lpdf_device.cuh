@@ -548,31 +548,33 @@ __device__ __forceinline__ void rec_store_stream(float* p, const float (&r)[8])
                  : "memory");
 }
 
-// the scalars from psi_1 on
+// the scalars from psi_2 on
 template <int NS>
 __device__ __forceinline__ void rest_load(const float* rest, int64_t j, float* psi)
 {
-    if (NS == 2) psi[1] = __ldcs(rest + j);
-    if (NS == 3) {
-        const float2 v = __ldcs(reinterpret_cast<const float2*>(rest) + j);
-        psi[1] = v.x;
-        psi[NS > 2 ? 2 : 0] = v.y;
-    }
+    if (NS == 3) psi[NS > 2 ? 2 : 0] = __ldcs(rest + j);
     if (NS == 4) {
-        const float4 v = __ldcs(reinterpret_cast<const float4*>(rest) + j);
-        psi[NS > 1 ? 1 : 0] = v.x;
-        psi[NS > 2 ? 2 : 0] = v.y;
-        psi[NS > 3 ? 3 : 0] = v.z;
+        const float2 v = __ldcs(reinterpret_cast<const float2*>(rest) + j);
+        psi[NS > 2 ? 2 : 0] = v.x;
+        psi[NS > 3 ? 3 : 0] = v.y;
     }
 }
 template <int NS>
 __device__ __forceinline__ void rest_store(float* rest, int64_t j, const float* psi)
 {
-    if (NS == 2) __stcs(rest + j, psi[1]);
-    if (NS == 3) __stcs(reinterpret_cast<float2*>(rest) + j, make_float2(psi[1], psi[NS > 2 ? 2 : 0]));
-    if (NS == 4)
-        __stcs(reinterpret_cast<float4*>(rest) + j,
-               make_float4(psi[NS > 1 ? 1 : 0], psi[NS > 2 ? 2 : 0], psi[NS > 3 ? 3 : 0], 0.0f));
+    if (NS == 3) __stcs(rest + j, psi[NS > 2 ? 2 : 0]);
+    if (NS == 4) __stcs(reinterpret_cast<float2*>(rest) + j, make_float2(psi[NS > 2 ? 2 : 0], psi[NS > 3 ? 3 : 0]));
+}
+// the last word of a record, and pid where it is an array of its own
+template <int NS>
+__device__ __forceinline__ float rec_last(const float* psi, uint32_t pid)
+{
+    return NS == 1 ? __uint_as_float(pid) : psi[NS > 1 ? 1 : 0];
+}
+template <int NS>
+__device__ __forceinline__ void pid_store(uint32_t* pids, int64_t j, uint32_t pid)
+{
+    if (NS > 1) __stcs(pids + j, pid);
 }
 
 __device__ __forceinline__ bool in_source(float px, float py, float sx, float sy, float r)

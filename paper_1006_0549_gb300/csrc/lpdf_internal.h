@@ -89,18 +89,22 @@ struct DevState {
     int64_t n, cap;
 };
 
-// A context's particles: a 32-byte record each (x, y, u, v, w, omega, psi_0, pid as bits), one sector of
+// A context's particles: a 32-byte record each (x, y, u, v, w, omega, psi_0, psi_1), one sector of
 // memory, so that a gather in element order moves no byte that it does not use, however the wanted
 // records are spread (as separate arrays the 32 values of a warp's gather lay in 10-25 sectors, eight
-// arrays over); the element, which the re-bucketing streams, is an array of its own, and so are the
-// scalars from psi_1 on (rest_words(ns) words a particle).
+// arrays over); the element, which the re-bucketing streams, is an array of its own, and so are pid, which
+// the moments do not read, and the scalars from psi_2 on (rest_words(ns) words a particle). With one scalar
+// pid (as bits) takes the place of psi_1. So the moments gather 36, 40 and 44 B a particle with two, three
+// and four scalars and a particle takes no padding: 5M particles with four scalars in 10,000 elements 79 us
+// (92 with pid in every record and rows of psi_1 to psi_3 padded to 16 B, 82 as separate arrays).
 struct Particles {
     float* rec;
     float* rest;
     int* elem;
+    uint32_t* pid;   // NULL with one scalar
     int64_t n, cap;
 };
-__host__ __device__ constexpr int rest_words(int ns) { return ns <= 3 ? ns - 1 : 4; }   // ns = 4: a float4, one unused
+__host__ __device__ constexpr int rest_words(int ns) { return ns <= 2 ? 0 : ns - 2; }
 
 // Status words (device): [0] error bits, [1] lost count, [2] one lost pid, [3] total hops
 enum : unsigned { kErrLost = 1u, kErrNonFinite = 2u, kErrOverflow = 4u, kErrTimeout = 8u, kErrCheck = 16u };

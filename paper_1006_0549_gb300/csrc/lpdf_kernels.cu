@@ -68,11 +68,12 @@ __global__ void particles_init_kernel(const __grid_constant__ DevMesh M, const _
         const uint32_t ew[6] = {b.z, b.w, c.x, c.y, c.z, c.w};
         float sum = 0.0f;
         for (int k = 0; k < m_erlang; ++k) sum += -logf(u01(ew[k]));
-        const float r[8] = {px, py, Fi[0] + Fi[3] * z0, Fi[1] + Fi[3] * z1, Fi[2] + Fi[3] * z2,
-                            Fi[4] * sum / (float)m_erlang, 0.0f, __uint_as_float(pid)};
-        rec_store_stream(S.rec + 8 * i, r);
         const float psi[NS] = {};
+        const float r[8] = {px, py, Fi[0] + Fi[3] * z0, Fi[1] + Fi[3] * z1, Fi[2] + Fi[3] * z2,
+                            Fi[4] * sum / (float)m_erlang, psi[0], rec_last<NS>(psi, pid)};
+        rec_store_stream(S.rec + 8 * i, r);
         rest_store<NS>(S.rest, i, psi);
+        pid_store<NS>(S.pid, i, pid);
         S.elem[i] = ne;
     }
     if (err) atomicOr(&status[0], (unsigned long long)err);
@@ -104,9 +105,11 @@ __global__ void pack_state_kernel(const __grid_constant__ Particles S, int64_t i
     float psi[NS];
 #pragma unroll
     for (int a = 0; a < NS; ++a) psi[a] = A.psi[a * A.ld + i];
-    const float r[8] = {A.x[i], A.y[i], A.u[i], A.v[i], A.w[i], A.om[i], psi[0], __uint_as_float(A.pid[i])};
+    const uint32_t pid = A.pid[i];
+    const float r[8] = {A.x[i], A.y[i], A.u[i], A.v[i], A.w[i], A.om[i], psi[0], rec_last<NS>(psi, pid)};
     rec_store_stream(S.rec + 8 * (i0 + i), r);
     rest_store<NS>(S.rest, i0 + i, psi);
+    pid_store<NS>(S.pid, i0 + i, pid);
     S.elem[i0 + i] = A.elem[i];
 }
 
@@ -119,6 +122,7 @@ __global__ void unpack_state_kernel(const __grid_constant__ Particles S, int64_t
     float r[8], psi[NS];
     rec_load_stream(S.rec + 8 * (i0 + i), r);
     psi[0] = r[6];
+    if (NS > 1) psi[NS > 1 ? 1 : 0] = r[7];
     rest_load<NS>(S.rest, i0 + i, psi);
     float* const out[6] = {A.x, A.y, A.u, A.v, A.w, A.om};
 #pragma unroll
@@ -128,7 +132,7 @@ __global__ void unpack_state_kernel(const __grid_constant__ Particles S, int64_t
 #pragma unroll
         for (int a = 0; a < NS; ++a) A.psi[a * A.ld + i] = psi[a];
     if (A.elem) A.elem[i] = S.elem[i0 + i];
-    if (A.pid) A.pid[i] = __float_as_uint(r[7]);
+    if (A.pid) A.pid[i] = NS == 1 ? __float_as_uint(r[7]) : S.pid[i0 + i];
 }
 
 cudaError_t launch_pack_state(const Particles& s, int64_t i0, int64_t n, int ns, const UserArrays& a, cudaStream_t st)

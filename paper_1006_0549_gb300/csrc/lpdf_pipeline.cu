@@ -165,9 +165,10 @@ __device__ __forceinline__ void advance_store(const DevMesh& M, const Particles&
         atomicAdd(&status[1], 1ull);
         atomicCAS(&status[2], ~0ull, (unsigned long long)p.pid);
     }
-    const float r[8] = {p.x, p.y, p.u, p.v, p.w, p.om, p.psi[0], __uint_as_float(p.pid)};
+    const float r[8] = {p.x, p.y, p.u, p.v, p.w, p.om, p.psi[0], rec_last<NS>(p.psi, p.pid)};
     rec_store_stream(nxt.rec + 8 * i, r);
     rest_store<NS>(nxt.rest, i, p.psi);
+    pid_store<NS>(nxt.pid, i, p.pid);
     __stcs(nxt.elem + i, ne);
 }
 
@@ -190,7 +191,9 @@ __device__ __forceinline__ void advance_one(const DevMesh& M, const Particles& c
     p.w = r[4];
     p.om = r[5];
     p.psi[0] = r[6];
-    p.pid = __float_as_uint(r[7]);
+    if (NS == 1) p.pid = __float_as_uint(r[7]);
+    else p.pid = (uint32_t)ld_stream(reinterpret_cast<const int*>(cur.pid) + src);
+    if (NS > 1) p.psi[NS > 1 ? 1 : 0] = r[7];
     rest_load<NS>(cur.rest, src, p.psi);
     advance_store<NS, kKind>(M, nxt, EF, P, status, i, p, err, hops);
 }
@@ -755,6 +758,7 @@ __device__ __forceinline__ void gather_fields(const Particles& S, int j, float& 
     if (G == 0) f[3] = b.y;
     if (G != 0) {
         psi[0] = b.z;
+        if (NS > 1) psi[NS > 1 ? 1 : 0] = b.w;
         rest_load<NS>(S.rest, j, psi);
 #pragma unroll
         for (int a_ = 0; a_ < NS; ++a_) f[(G == 2 ? 3 : 0) + a_] = psi[a_];
@@ -1091,6 +1095,7 @@ __global__ void __launch_bounds__(MBLK, MMINB) moments_kernel_f32(const __grid_c
                 bw[buf][k] = r[4];
                 bo[buf][k] = r[5];
                 bp[buf][k][0] = r[6];
+                if (NS > 1) bp[buf][k][NS > 1 ? 1 : 0] = r[7];
                 rest_load<NS>(S.rest, j, bp[buf][k]);
             }
         };
@@ -1264,6 +1269,7 @@ __global__ void __launch_bounds__(MBLK, MMINB) moments_kernel_f32h(const __grid_
                 bw[buf][k] = r[4];
                 bo[buf][k] = r[5];
                 bp[buf][k][0] = r[6];
+                if (NS > 1) bp[buf][k][NS > 1 ? 1 : 0] = r[7];
                 rest_load<NS>(S.rest, j, bp[buf][k]);
             }
         };

@@ -142,15 +142,13 @@ cudaError_t launch_sort(const DevMesh& m, const Particles& s, int ns, const Part
     segment_sort_kernel<<<E + 1, 256, 0, st>>>(w.start, w.perm, status);
     const int64_t nblk = (s.n + 255) / 256;
     const unsigned gg = (unsigned)(nblk < 152 * 16 ? nblk : 152 * 16);
-    // the records as 16-byte halves; the remaining scalars by their words
+    // the records, then the remaining scalars by their words
     gather_kernel<Rec><<<gg, 256, 0, st>>>(reinterpret_cast<const Rec*>(s.rec), reinterpret_cast<Rec*>(dst.rec), w.perm, s.n);
     if (rest_words(ns) == 1) gather_kernel<float><<<gg, 256, 0, st>>>(s.rest, dst.rest, w.perm, s.n);
     if (rest_words(ns) == 2)
         gather_kernel<float2><<<gg, 256, 0, st>>>(reinterpret_cast<const float2*>(s.rest), reinterpret_cast<float2*>(dst.rest),
                                                   w.perm, s.n);
-    if (rest_words(ns) == 4)
-        gather_kernel<float4><<<gg, 256, 0, st>>>(reinterpret_cast<const float4*>(s.rest), reinterpret_cast<float4*>(dst.rest),
-                                                  w.perm, s.n);
+    if (s.pid) gather_kernel<uint32_t><<<gg, 256, 0, st>>>(s.pid, dst.pid, w.perm, s.n);
     gather_kernel<int><<<gg, 256, 0, st>>>(s.elem, dst.elem, w.perm, s.n);
     return cudaGetLastError();
 }
