@@ -1513,8 +1513,8 @@ cudaError_t run_pipeline(const DevMesh& m, const Particles& cur, const Particles
         if (p.moment_sums == 1)
             moments_kernel_df<NS, 256, 2, true><<<nblocks((int64_t)E * 32, 256), 256, 0, st>>>(m, nxt, w.perm_new,
                                                                                              w.kstart, flux_acc, status);
-        else
-            moments_kernel_f32<NS, 256, 2, true><<<nblocks((int64_t)E * 32, 256), 256, 0, st>>>(m, nxt, w.perm_new,
+        else   // 24 warps per SM at 80 registers (16 at 89-102): a 5M-particle cavity with two scalars 702 -> 658 us a step
+            moments_kernel_f32<NS, 256, 3, true><<<nblocks((int64_t)E * 32, 256), 256, 0, st>>>(m, nxt, w.perm_new,
                                                                                               w.kstart, flux_acc, status);
     }
     if (ev) cudaEventRecord(ev[3], st);
