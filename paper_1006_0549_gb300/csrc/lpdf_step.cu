@@ -389,14 +389,16 @@ pdf_step_kernel(const __grid_constant__ DevMesh M, const __grid_constant__ DevSt
             start(B);
 #pragma unroll 1
             while (A.j >= 0 || B.j >= 0) {
-                // the certified test; the exact one where it is undecided (kWalkIn: inside, else the exit)
+                // the certified test; the exact one where it is undecided (kWalkIn: inside, else the exit, a
+                // wall only where no interior edge is crossed: a particle far outside is lost after the
+                // hops of the exact walk)
                 int ca = kWalkIn, cb = kWalkIn, next = -1;
                 if (A.j >= 0) {
-                    const int r = walk_test_fast(M, A.e, A.px, A.py, next);
+                    const int r = walk_test_fast<true>(M, A.e, A.px, A.py, next);
                     ca = r > 0 ? kWalkIn : (r == 0 ? next : walk_test_code(M, A.e, A.px, A.py));
                 }
                 if (B.j >= 0) {
-                    const int r = walk_test_fast(M, B.e, B.px, B.py, next);
+                    const int r = walk_test_fast<true>(M, B.e, B.px, B.py, next);
                     cb = r > 0 ? kWalkIn : (r == 0 ? next : walk_test_code(M, B.e, B.px, B.py));
                 }
                 if (A.j >= 0) step(A, ca == kWalkIn, ca);
