@@ -348,8 +348,8 @@ int lpdf_grid_statistics(lpdf_ctx* ctx, double* out, int raw, void* stream);
 
 /* ---------------------------------------------------------------------------------------
  * lpdf_elliptic_relax_solve -- the gridpoint side: node fields for lpdf_pdf_step from gridpoint
- * statistics (Introduction, item ii: Eulerian quantities are solved on the grid). sync (the
- * conjugate-gradient convergence tests read residual norms back to the host).
+ * statistics (Introduction, item ii: Eulerian quantities are solved on the grid). sync (one read
+ * at the end tells how the conjugate gradients ended).
  *   stats   device, n_nodes x (11 + 2 ns) FP64 as lpdf_grid_statistics(raw = 0) writes them
  *   fields  device out, n_nodes x nfp FP32 (columns LPDF_F_*)
  *   tol     relative residual of each conjugate gradient: |r| <= tol |r_ref|, r_ref the residual

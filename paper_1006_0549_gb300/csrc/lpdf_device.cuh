@@ -317,12 +317,14 @@ static __device__ __noinline__ int fast_wall_exit(float l0, float l1, float l2, 
 }
 
 // The walk test in the affine barycentric form relative to vertex 0, with a certified error
-// bound: 1 = (px, py) is strictly inside e; 0 = it is certainly outside, leave through `next`
-// (the edge opposite the most negative certainly negative lambda across an interior edge; if
-// only walls are crossed, -1 - k for the wall edge k of the most negative one); -1 = undecided
-// (within the rounding bound of an edge, or in a periodic image frame): the caller runs
-// walk_test. Preferring interior exits keeps the walk inside a non-convex domain: a point of the
-// domain can lie beyond the line of some wall edge, never beyond every negative edge's line.
+// bound: 1 = (px, py) is strictly inside e; 0 = it is certainly outside, leave through `next`;
+// -1 = undecided (within the rounding bound of an edge, or in a periodic image frame): the caller
+// runs walk_test. `next` without kWalls: the neighbour across the edge opposite the most negative
+// lambda, -1 when that edge is a wall (walls on the frame's sides: the point has left a convex
+// domain). With kWalls: the neighbour across the most negative certainly crossed interior edge; if
+// only walls are crossed, -1 - k for the wall edge k of the most negative lambda. Preferring interior
+// exits keeps the walk inside a non-convex domain: a point of the domain can lie beyond the line of
+// some wall edge, never beyond every negative edge's line.
 // Bound: with u = 2^-24, dx = fl(px - x_v0) (x_v0 exact in FP32) and the coefficients rounded
 // from FP64, |lambda_a' - lambda_a| <= 4.01 u (|b_a dx| + |g_a dy|) for a = 1, 2, and for
 // lambda_0 = 1 - lambda_1 - lambda_2 that sum plus 2 u (1 + |lambda_1| + |lambda_2|). One bound serves
@@ -534,7 +536,7 @@ struct ParticleState {
     uint32_t pid;
 };
 
-// one record, 32 bytes in one instruction: read once and not kept in L1; read and kept; written through
+// one record, 32 bytes in one instruction: read once and not kept in L1; written through
 __device__ __forceinline__ void rec_load_stream(const float* p, float (&r)[8])
 {
     asm("ld.global.nc.L1::no_allocate.v8.f32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];"

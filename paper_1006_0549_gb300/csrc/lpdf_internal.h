@@ -173,8 +173,10 @@ struct PipeScratch {
 // >= 10, persistent, warps taking 64-particle chunks from a counter. mom: moments kernel
 // 0 = 256 threads, >= 2 CTAs/SM; 1 = 128, >= 4 (four scalars: 5); 2 = 512, >= 1; 3 = 256,
 // >= 3.
-// The default is what the tuner picks or comes within 3 % of for every ensemble measured (0.05 to 25 million
-// particles, one to four scalars); the 256-thread grids it replaced took 9-18 % longer a step.
+// The default is the tuner's pick or within 3 % of it up to 20 million particles (channels of 0.05, 1, 3, 5
+// and 10 million, cavities of 5 and 20 with four scalars, curved walls with 7). Above that advance variant 5
+// leads: a 25M channel 1.104 against 1.004 ms a step, 64 channels of 268M together 12.7 against 11.1. The
+// 256-thread grids take up to 16 % longer than the default (10M: 0.526 against 0.455 ms).
 struct StepTune {
     int adv = 1, mom = 1;
 };

@@ -463,7 +463,7 @@ __global__ void __launch_bounds__(kScanThreads) scan_tiles_kernel(ScanPair sp, i
 }
 
 // the same in one launch for few tiles: every block first adds up all that lies before its tile
-// (at most kScanOneTiles - 1 tiles: 60 KB from L2) instead of waiting for the others
+// (at most kScanOneTiles - 1 tiles: 240 KB from L2) instead of waiting for the others
 constexpr int kScanOneTiles = 16;
 
 __global__ void __launch_bounds__(kScanThreads) scan_one_kernel(ScanPair sp, int n)
@@ -1073,7 +1073,7 @@ __global__ void __launch_bounds__(MBLK, MMINB) moments_kernel_f32(const __grid_c
         // current batch is accumulated, in position order per lane. Two buffers of one or two
         // particles are worth more than one buffer of two or four: the cavity's four-scalar moments
         // took 377 us with one buffer and two 128-bit loads per record, 329 us so.
-        constexpr int MB = kMomentBatch<NS>, NB = 2;
+        constexpr int MB = kMomentBatch<NS>;
         static_assert(LC % MB == 0, "whole batches per chunk");
         int idx[LC];
 #pragma unroll
@@ -1081,7 +1081,7 @@ __global__ void __launch_bounds__(MBLK, MMINB) moments_kernel_f32(const __grid_c
             const int pos = base + lane + 32 * k;
             idx[k] = pos < end ? load_after(perm + pos) : -1;
         }
-        float bx[NB][MB], by[NB][MB], bu[NB][MB], bv[NB][MB], bw[NB][MB], bo[NB][MB], bp[NB][MB][NS];
+        float bx[2][MB], by[2][MB], bu[2][MB], bv[2][MB], bw[2][MB], bo[2][MB], bp[2][MB][NS];
         auto gather = [&](int buf, int k0) {
 #pragma unroll
             for (int k = 0; k < MB; ++k) {
@@ -1099,16 +1099,12 @@ __global__ void __launch_bounds__(MBLK, MMINB) moments_kernel_f32(const __grid_c
                 rest_load<NS>(S.rest, j, bp[buf][k]);
             }
         };
-        if constexpr (NB == 2) gather(0, 0);
+        gather(0, 0);
 #pragma unroll
         for (int k0 = 0; k0 < LC; k0 += MB) {
             if (base + 32 * k0 >= end) break;
-            const int cb = NB == 2 ? (k0 / MB) & 1 : 0;
-            if constexpr (NB == 2) {
-                if (k0 + MB < LC && base + 32 * (k0 + MB) < end) gather(cb ^ 1, k0 + MB);
-            } else {
-                gather(0, k0);
-            }
+            const int cb = (k0 / MB) & 1;
+            if (k0 + MB < LC && base + 32 * (k0 + MB) < end) gather(cb ^ 1, k0 + MB);
             float* const sx = bx[cb];
             float* const sy = by[cb];
             float* const su = bu[cb];
@@ -1247,7 +1243,7 @@ __global__ void __launch_bounds__(MBLK, MMINB) moments_kernel_f32h(const __grid_
         float acc[NK];
 #pragma unroll
         for (int k = 0; k < NK; ++k) acc[k] = 0.0f;
-        constexpr int MB = kMomentBatch<NS>, NB = 2;
+        constexpr int MB = kMomentBatch<NS>;
         static_assert(LC % MB == 0, "whole batches per chunk");
         int idx[LC];
 #pragma unroll
@@ -1255,7 +1251,7 @@ __global__ void __launch_bounds__(MBLK, MMINB) moments_kernel_f32h(const __grid_
             const int pos = base + lane + 16 * k;
             idx[k] = pos < end ? load_after(perm + pos) : -1;
         }
-        float bx[NB][MB], by[NB][MB], bu[NB][MB], bv[NB][MB], bw[NB][MB], bo[NB][MB], bp[NB][MB][NS];
+        float bx[2][MB], by[2][MB], bu[2][MB], bv[2][MB], bw[2][MB], bo[2][MB], bp[2][MB][NS];
         auto gather = [&](int buf, int k0) {
 #pragma unroll
             for (int k = 0; k < MB; ++k) {
@@ -1274,16 +1270,12 @@ __global__ void __launch_bounds__(MBLK, MMINB) moments_kernel_f32h(const __grid_
             }
         };
         if (base < end) {
-            if constexpr (NB == 2) gather(0, 0);
+            gather(0, 0);
 #pragma unroll
             for (int k0 = 0; k0 < LC; k0 += MB) {
                 if (base + 16 * k0 >= end) break;
-                const int cb = NB == 2 ? (k0 / MB) & 1 : 0;
-                if constexpr (NB == 2) {
-                    if (k0 + MB < LC && base + 16 * (k0 + MB) < end) gather(cb ^ 1, k0 + MB);
-                } else {
-                    gather(0, k0);
-                }
+                const int cb = (k0 / MB) & 1;
+                if (k0 + MB < LC && base + 16 * (k0 + MB) < end) gather(cb ^ 1, k0 + MB);
 #pragma unroll
                 for (int k = 0; k < MB; ++k) {
                     if (idx[k0 + k] < 0) break;

@@ -157,21 +157,19 @@ __global__ void assemble_kernel(const Fem F, const double* __restrict__ L2e, dou
 // ---------------------------------------------------------------- batched PCG
 // vectors are stored component-major: v[c n + i]
 
-// y_c = A x_c; rows of fixed (wall) DOFs give 0 when `mask` is set
-__global__ void spmv_kernel(const Fem F, const double* __restrict__ A, const double* __restrict__ x,
-                            double* __restrict__ y, int mask, int nv)
+// y_c = A x_c of the relaxation's four components
+__global__ void spmv_kernel(const Fem F, const double* __restrict__ A, const double* __restrict__ x, double* __restrict__ y)
 {
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= F.ndof) return;
     const size_t n = F.ndof;
     double s[4] = {0, 0, 0, 0};
-    if (!(mask && F.wall[i]))
-        for (int t = F.row[i]; t < F.row[i + 1]; ++t) {
-            const int j = F.col[t];
-            const double a = A[t];
-            for (int c = 0; c < nv; ++c) s[c] += a * x[c * n + j];
-        }
-    for (int c = 0; c < nv; ++c) y[c * n + i] = s[c];
+    for (int t = F.row[i]; t < F.row[i + 1]; ++t) {
+        const int j = F.col[t];
+        const double a = A[t];
+        for (int c = 0; c < 4; ++c) s[c] += a * x[c * n + j];
+    }
+    for (int c = 0; c < 4; ++c) y[c * n + i] = s[c];
 }
 
 // Jacobi-preconditioned CG on one or two systems of the mesh's pattern (the relaxation's four
@@ -1458,7 +1456,7 @@ cudaError_t node_fields_solve(Fem& F, const double* stats, const lpdf_params& P,
         assemble_kernel<<<gd, 256, 0, st>>>(F, ew, F.Aval, diag, F.lmax);
         const bool warm = P.cg_warm_start && F.has_wp;
         er_setup_kernel<<<gd, 256, 0, st>>>(F, eps, P.C0, tmp, wp, warm ? wp_prev : nullptr, xref);
-        spmv_kernel<<<gd, 256, 0, st>>>(F, F.Mval, tmp, rhs, 0, 4);     // b = M wp^h
+        spmv_kernel<<<gd, 256, 0, st>>>(F, F.Mval, tmp, rhs);     // b = M wp^h
         a.A0 = F.Aval;
         a.d0 = diag;
         a.b0 = rhs;
