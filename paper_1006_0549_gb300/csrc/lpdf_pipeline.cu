@@ -1072,7 +1072,8 @@ __global__ void __launch_bounds__(MBLK, MMINB) moments_kernel_f32(const __grid_c
         // double-buffered: the next batch's records are loaded (one 256-bit load each) before the
         // current batch is accumulated, in position order per lane. Two buffers of one or two
         // particles are worth more than one buffer of two or four: the cavity's four-scalar moments
-        // took 377 us with one buffer and two 128-bit loads per record, 329 us so.
+        // took 377 us with one buffer and two 128-bit loads per record, 329 us so (304 since psi_1 lies in the
+        // record; 314 as ten separate arrays).
         constexpr int MB = kMomentBatch<NS>;
         static_assert(LC % MB == 0, "whole batches per chunk");
         int idx[LC];
@@ -1405,7 +1406,7 @@ void launch_advance(int v, const DevMesh& m, const Particles& cur, const Particl
 }
 
 // four scalars: 20 warps per SM at 96 registers (a few spills) hide more of the gathers than 16 at 128:
-// 1.205 against 1.230 ms per step of the 20M cavity
+// 1.255 against 1.300 ms per step of the 20M cavity with its statistics
 template <int NS>
 constexpr int kMomentCtas = NS == 4 ? 5 : 4;
 
