@@ -209,7 +209,7 @@ int lpdf_particles_init(lpdf_ctx* ctx, int32_t n_per_elem, const float* node_ini
  * lpdf_set_state / lpdf_get_state -- copy the state in or out of the caller's arrays, one per field. `on_device` = 1: the
  * pointers are device memory, 0: host memory. psi is ns rows of n values. set_state sets the
  * ensemble size to n (n <= capacity). async (a host copy is synchronous w.r.t. the host only
- * when the host memory is pageable: it then goes through a staging buffer of at most 4M particles,
+ * when the host memory is pageable: it then goes through a staging buffer of at most 16M particles,
  * made by the first such call and kept with the context). A set_state that fails leaves the ensemble as it was, or empty
  * when it had begun to write it.
  * ------------------------------------------------------------------------------------- */

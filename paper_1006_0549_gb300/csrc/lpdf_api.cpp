@@ -707,8 +707,10 @@ static bool all_in_reach(const UserArrays& a, int64_t n, int ns, int device, int
 }
 
 // The context's staging buffer of at most kStage particles, made by the first call that needs one and kept:
-// an allocation per call took 200 us. Smaller when memory is short.
-constexpr int64_t kStage = 1 << 22, kStageMin = 1 << 10;
+// an allocation per call took 200 us. Smaller when memory is short. A block costs a copy per array of 13 us
+// and more: 10M particles with one scalar, pageable, 2.32 ms in and 2.10 out in one block, 2.50 and 2.29 in
+// blocks of 4M (copies alone: 2.21 and 1.98).
+constexpr int64_t kStage = 1 << 24, kStageMin = 1 << 10;
 static cudaError_t staging(lpdf_ctx* c, cudaStream_t st)
 {
     if (c->stage) return cudaStreamWaitEvent(st, c->stage_done, 0);
